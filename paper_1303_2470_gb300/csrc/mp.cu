@@ -891,6 +891,7 @@ void destroy(mp_ctx* c)
 {
     if (!c) return;
     direct_free(c);
+    flux64_free(c);
     for (int b = 0; b < 2; ++b) {
         if (c->exec[b]) cudaGraphExecDestroy(c->exec[b]);
         if (c->graph[b]) cudaGraphDestroy(c->graph[b]);
@@ -1221,6 +1222,7 @@ int mp_init_batch(mp_ctx** out, const mp_geometry* g, const float* u, int n_spec
         rc = MP_ENEGPROB;
     }
     if (rc == MP_OK && c->scheme == MP_SCHEME_DIRECT) rc = direct_setup(c, opt.autotune, opt.variant);
+    if (rc == MP_OK && c->precision == MP_FP64) rc = flux64_setup(c);
     if (rc != MP_OK) {
         destroy(c);
         return rc;
@@ -1252,6 +1254,7 @@ int mp_step(mp_ctx* c, int64_t n)
         return MP_EINVAL;
     }
     if (c->scheme == MP_SCHEME_DIRECT) return direct_step(c, n);
+    if (c->flux64) return flux64_step(c, n);
     return c->precision == MP_FP64   ? step_typed<double, double>(c, n)
            : c->precision == MP_FP16 ? step_typed<float, __half>(c, n)
                                      : step_typed<float, float>(c, n);

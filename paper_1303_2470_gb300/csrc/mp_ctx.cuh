@@ -15,6 +15,7 @@ struct mp_group;
 namespace mp {
 struct DirectTables;
 struct DirectState;
+struct Flux64;
 }  // namespace mp
 
 struct mp_ctx {
@@ -58,6 +59,8 @@ struct mp_ctx {
     int scheme = MP_SCHEME_FLUX;
     mp::DirectTables* dtab = nullptr;
     mp::DirectState* dstate = nullptr;
+    // FP64 flux contexts: link tables of the tabulated step (NULL: terms recomputed)
+    mp::Flux64* flux64 = nullptr;
 };
 
 namespace mp {
@@ -71,6 +74,12 @@ int direct_setup(mp_ctx* c, int tune, int variant);
 int direct_step(mp_ctx* c, long long n);
 int direct_check(mp_ctx* c);
 void direct_free(mp_ctx* c);
+
+// Tabulated FP64 flux step (mp_flux64.cu): tables after the fields are initialised (c->flux64
+// stays NULL where they do not fit), n steps, release.
+int flux64_setup(mp_ctx* c);
+int flux64_step(mp_ctx* c, long long n);
+void flux64_free(mp_ctx* c);
 
 // A set of direct-scheme contexts stepped together (groups): created over n contexts, run on
 // `stream`, stepped n steps; variant and block size are autotuned when `tune` is nonzero.
