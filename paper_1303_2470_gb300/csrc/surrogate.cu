@@ -4,6 +4,9 @@
 // memory; the weight gradient with mma.sync m16n8k16; BF16 operands, FP32 accumulation),
 // pooling, upsampling, the masked loss and the Adam update. Nothing here belongs to the moment-propagation
 // method itself; the network's output only seeds lb_steady.
+#include <algorithm>
+
+#include <cuda.h>
 #include <cuda_bf16.h>
 
 #include "../../include/surrogate.h"
@@ -110,11 +113,14 @@ __device__ __forceinline__ unsigned long long tc_now_ns()
     return t;
 }
 
-// wait for the phase of parity `parity` of an mbarrier to complete; false after kTWaitNs
-__device__ __forceinline__ bool mbar_wait(uint32_t bar, uint32_t parity)
+// Wait for the phase of parity `parity` of an mbarrier to complete; false after kTWaitNs, or
+// once `fail` (a flag in shared memory that another waiter set) is nonzero; the wait that runs
+// out sets it. The global timer is read only every 64 polls: reading it costs hundreds of
+// clocks, as much as the stage of a convolution.
+__device__ __forceinline__ bool mbar_wait_or(uint32_t bar, uint32_t parity, volatile int* fail)
 {
-    const unsigned long long t0 = tc_now_ns();
-    while (true) {
+    unsigned long long t0 = 0;
+    for (uint32_t poll = 1;; ++poll) {
         uint32_t done;
         asm volatile(
             "{\n.reg .pred q;\nmbarrier.try_wait.parity.shared::cta.b64 q, [%1], %2;\nselp.b32 %0, 1, 0, q;\n}"
@@ -122,16 +128,32 @@ __device__ __forceinline__ bool mbar_wait(uint32_t bar, uint32_t parity)
             : "r"(bar), "r"(parity)
             : "memory");
         if (done) return true;
-        if ((long long)(tc_now_ns() - t0) > kTWaitNs) return false;
+        if (fail && *fail) return false;
+        if (poll % 64 == 0) {
+            const unsigned long long t = tc_now_ns();
+            if (t0 == 0) t0 = t;
+            if ((long long)(t - t0) > kTWaitNs) {
+                if (fail) *fail = 1;
+                return false;
+            }
+        }
     }
+}
+__device__ __forceinline__ bool mbar_wait(uint32_t bar, uint32_t parity) { return mbar_wait_or(bar, parity, nullptr); }
+
+// one lane of a converged warp
+__device__ __forceinline__ bool elect_one()
+{
+    uint32_t r;
+    asm volatile("{\n.reg .pred p;\nelect.sync _|p, 0xffffffff;\nselp.b32 %0, 1, 0, p;\n}" : "=r"(r));
+    return r != 0;
 }
 
 // Epilogue of the tensor-core convolutions: warp w reads accumulator rows 32w..32w+31 (its
 // lanes' voxels) from tensor memory, adds the bias, applies the ReLU and stores BF16 and/or
-// FP32 outputs of voxel v, channels n0..n0+BN-1.
-__device__ __forceinline__ void conv_epilogue(const ConvArgs& a, uint32_t tmem, int warp, int b, int v, int n0, int BN)
+// FP32 outputs of voxel e of the batch (skipped when negative), channels n0..n0+BN-1.
+__device__ __forceinline__ void conv_store_row(const ConvArgs& a, uint32_t tmem, int warp, long long e, int n0, int BN)
 {
-    const bool vok = v < a.V;
     for (int c0 = 0; c0 < BN; c0 += 16) {
         uint32_t r[16];
         const uint32_t addr = tmem + ((uint32_t)(32 * warp) << 16) + (uint32_t)c0;
@@ -141,30 +163,32 @@ __device__ __forceinline__ void conv_epilogue(const ConvArgs& a, uint32_t tmem, 
               "=r"(r[8]), "=r"(r[9]), "=r"(r[10]), "=r"(r[11]), "=r"(r[12]), "=r"(r[13]), "=r"(r[14]), "=r"(r[15])
             : "r"(addr));
         asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory");
-        if (!vok) continue;
-        const size_t o = ((size_t)b * a.V + v) * a.N + n0 + c0;
-        float f[16];
+        if (e >= 0) {
+            const size_t o = (size_t)e * a.N + n0 + c0;
+            float f[16];
 #pragma unroll
-        for (int c = 0; c < 16; ++c) {
-            float t = __uint_as_float(r[c]) + (a.bias ? a.bias[n0 + c0 + c] : 0.0f);
-            f[c] = a.relu ? fmaxf(t, 0.0f) : t;
-        }
-        if (a.y) {
-            uint32_t h[8];
-#pragma unroll
-            for (int c = 0; c < 8; ++c) {
-                const __nv_bfloat162 p2 = __floats2bfloat162_rn(f[2 * c], f[2 * c + 1]);
-                h[c] = *reinterpret_cast<const uint32_t*>(&p2);
+            for (int c = 0; c < 16; ++c) {
+                float t = __uint_as_float(r[c]) + (a.bias ? a.bias[n0 + c0 + c] : 0.0f);
+                f[c] = a.relu ? fmaxf(t, 0.0f) : t;
             }
-            uint4* dst = reinterpret_cast<uint4*>(a.y + o);
-            dst[0] = make_uint4(h[0], h[1], h[2], h[3]);
-            dst[1] = make_uint4(h[4], h[5], h[6], h[7]);
-        }
-        if (a.yf) {
-            float4* dst = reinterpret_cast<float4*>(a.yf + o);
+            if (a.y) {
+                uint32_t h[8];
 #pragma unroll
-            for (int c = 0; c < 4; ++c) dst[c] = make_float4(f[4 * c], f[4 * c + 1], f[4 * c + 2], f[4 * c + 3]);
+                for (int c = 0; c < 8; ++c) {
+                    const __nv_bfloat162 p2 = __floats2bfloat162_rn(f[2 * c], f[2 * c + 1]);
+                    h[c] = *reinterpret_cast<const uint32_t*>(&p2);
+                }
+                uint4* dst = reinterpret_cast<uint4*>(a.y + o);
+                dst[0] = make_uint4(h[0], h[1], h[2], h[3]);
+                dst[1] = make_uint4(h[4], h[5], h[6], h[7]);
+            }
+            if (a.yf) {
+                float4* dst = reinterpret_cast<float4*>(a.yf + o);
+#pragma unroll
+                for (int c = 0; c < 4; ++c) dst[c] = make_float4(f[4 * c], f[4 * c + 1], f[4 * c + 2], f[4 * c + 3]);
+            }
         }
+        __syncwarp();
     }
 }
 
@@ -303,133 +327,356 @@ __global__ void __launch_bounds__(kTThreads) k_conv_tc(const ConvArgs a)
     if (ok) ok = mbar_wait(smem_u32(&mbar[(nst - 1) % kTStages]), (uint32_t)(((nst - 1) / kTStages) & 1));
     if (!ok && tid == 0) atomicExch(&g_sg_tc_fail, 1);
     asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
-    if (__syncthreads_and(ok)) conv_epilogue(a, tmem, warp, b, v, n0, BN);
+    if (__syncthreads_and(ok)) conv_store_row(a, tmem, warp, v < a.V ? (long long)b * a.V + v : -1, n0, BN);
     asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
     __syncthreads();
     if (warp == 0) asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(tmem), "r"(ncols));
 }
 
 // ---------------------------------------------------------------------------------------
-// The same convolution where a block's 128 voxels are one stretch of an x-row (W a multiple
-// of 128) and K <= 64: the three taps that differ only in dx read the same source row, so a
-// stage holds that row once — the 130 voxels x0 - 1 .. x0 + 128 (periodic) of the source
-// row (y + s dy, z + s dz), s the sign — and the taps dx = -1, 0, +1 are three groups of MMAs
-// whose A descriptors start 0, 1 or 2 rows into it (the 128-byte swizzle is keyed to the
-// absolute shared-memory address, so a descriptor may start at any row of an atom). Nine
-// stages, one per (dz, dy), in tap order; within a stage the taps in dx order and each tap's
-// channels in order, so the accumulation order is that of k_conv_tc and the outputs are
-// bitwise the same. Three B tiles (one per dx) per stage.
+// The same convolution marching along y (W a multiple of 8, K = 16, 32, 64, 96 or 128): the
+// kernel of the network's layers. Measured, forward on one box (tap by tap -> marching): 128^3,
+// 32 -> 32 channels 463 -> 167 us, 64 -> 32 643 -> 238 us; 64^3, 64 -> 64 171 -> 60 us (960
+// TFLOP/s); 32^3, 96 -> 96 60 -> 29 us; 16^3, 128 -> 128 59 -> 15 us.
+//
+// What bounds a tap-by-tap implicit GEMM with few output channels is shared memory: every
+// K = 16 slice of every tap reads the 128 x 16 operand A (4 KB, 32 clocks) for as little as
+// 16 clocks of products (N = 32), and every tap's rows are copied in again. Here a block
+// computes T consecutive rows (y) of one column of 128 voxels and takes each source row once
+// per dz:
+//  * the three taps dy that read one source row go to three neighbouring output rows, whose
+//    accumulators are neighbouring column ranges of tensor memory: one MMA with the three taps'
+//    weights side by side (N' = 3 N columns) serves all three (two or one at the ends of the
+//    strip), so operand A is read a third as often;
+//  * the taps dx read the same staged row through descriptors that start one row earlier or
+//    later (the 128-byte swizzle is keyed to the absolute shared-memory address), so a row is
+//    copied 3 (T + 2) / T times instead of 27.
+// The column of 128 voxels is any 16 groups of 8 x-neighbours (b, z, x / 8): each group is
+// staged as 10 rows of 128 bytes, its voxels with their left and right neighbour (periodic),
+// and the descriptor's stride between 8-row groups is 1280 bytes. So a box of any W that is a
+// multiple of 8 fills the MMA's 128 rows.
+// Per accumulator the products are added in the order of k_conv_tc (taps ascending, then
+// channels): source rows ascend for sign = +1 and descend for sign = -1, and outputs are
+// bitwise the same.
+// A persistent block of 14 warps: 4 epilogue warps (tensor memory -> bias, ReLU -> global,
+// one accumulator set while the other is being computed), one warp that issues the MMAs, one
+// that loads weights (TMA; one dz at a time in two buffers, or all of them once per block where
+// they fit), 8 warps that copy rows (cp.async: a TMA box can't wrap around) into a ring of up
+// to eight. The copies of a thread are the same pieces of every row, so that one costs an
+// address and a copy instruction: with four warps and the addresses formed per piece the
+// copying warps were the limit at 1000 clocks a row.
+// Every wait is bounded; one that gives up sets a flag in shared memory that ends every role
+// and is reported through g_sg_tc_fail.
 // ---------------------------------------------------------------------------------------
-constexpr int kRRows = 136;                  // staged source row: 130 voxels in 17 atoms
-constexpr int kRABytes = (kRRows / 8) * kTAtom;
-constexpr int kRMaxN = 64;                   // output channels: the ring stays below 90 KB
+constexpr int kMCopy = 256;              // copying threads
+constexpr int kMThreads = 192 + kMCopy;
+constexpr int kMRows = 160;      // staged rows: 16 groups of 8 voxels with two neighbours
+constexpr int kMChunk = kMRows * 128;  // bytes of 64 channels of a staged row
+constexpr int kMStages = 8;      // most ring stages
+constexpr int kMSmem = 232448 - 1024;  // dynamic shared memory a block may use (227 KB less static)
+
+struct MarchArgs {
+    ConvArgs c;
+    int GX, NG;           // groups per x-row, groups over the batch
+    int T, nstrip;        // output rows per unit, strips along y
+    int NB, nblk;         // output channels per unit, channel blocks
+    int units;            // columns x strips x channel blocks
+    int nA;               // ring stages
+    int resident;         // all weights loaded once per block (nblk = 1)
+    int bufs;             // accumulator sets
+    uint32_t ncols;       // tensor-memory columns
+};
+
+// barrier 1 over the copying threads, true when `v` is true in all of them
+__device__ __forceinline__ bool bar_and(bool v)
+{
+    uint32_t r;
+    asm volatile(
+        "{\n.reg .pred p, q;\nsetp.ne.b32 p, %1, 0;\nbarrier.cta.red.and.pred q, 1, %2, p;\nselp.b32 %0, 1, 0, q;\n}"
+        : "=r"(r)
+        : "r"((uint32_t)v), "n"(kMCopy)
+        : "memory");
+    return r != 0;
+}
+
+__device__ __forceinline__ void mbar_arrive(uint32_t bar)
+{
+    asm volatile("{\n.reg .b64 t;\nmbarrier.arrive.shared::cta.b64 t, [%0];\n}" ::"r"(bar) : "memory");
+}
+
+__device__ __forceinline__ void tc_commit(uint32_t bar)
+{
+    asm volatile("tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%0];" ::"r"(bar) : "memory");
+}
+
+__device__ __forceinline__ void tc_mma(uint32_t d, uint64_t ad, uint64_t bd, uint32_t idesc, uint32_t accum)
+{
+    asm volatile(
+        "{\n.reg .pred p;\nsetp.ne.b32 p, %4, 0;\n"
+        "tcgen05.mma.cta_group::1.kind::f16 [%0], %1, %2, %3, p;\n}" ::"r"(d),
+        "l"(ad), "l"(bd), "r"(idesc), "r"(accum)
+        : "memory");
+}
+
+// K-major 128-byte-swizzled descriptor with `stride` bytes between 8-row groups (tc_desc: 1024)
+__device__ __forceinline__ uint64_t tc_desc_stride(uint32_t addr, uint32_t stride)
+{
+    return (uint64_t)((addr & 0x3FFFFu) >> 4) | (1ull << 16) | ((uint64_t)(stride >> 4) << 32) | (1ull << 46) |
+           (2ull << 61);
+}
 
 template <int kK>
-__global__ void __launch_bounds__(kTThreads) k_conv_row(const ConvArgs a)
+__global__ void __launch_bounds__(kMThreads, 1) k_conv_march(const __grid_constant__ MarchArgs m, const __grid_constant__ CUtensorMap wmap)
 {
-    static_assert(kK == 16 || kK == 32 || kK == 64, "one swizzle atom row per voxel");
+    constexpr int kCh = (kK + 63) / 64;   // 64-channel chunks of a staged row
+    constexpr int kKC = kK / 8;           // 16-byte pieces of a voxel
+    constexpr uint32_t kABytes = kCh * kMChunk;
     extern __shared__ __align__(1024) unsigned char tc_smem_raw[];
-    __shared__ __align__(8) uint64_t mbar[kTStages];
-    __shared__ uint32_t tmem_base;
-    const int tid = threadIdx.x, warp = tid >> 5;
-    const int n0 = blockIdx.y * kTMaxN;
-    const int BN = a.N - n0 < kTMaxN ? a.N - n0 : kTMaxN;  // a multiple of 16
-    const int BTile = (BN / 8) * kTAtom;                   // one tap's B tile
-    unsigned char* tc_smem = tc_smem_raw + ((kTAtom - (smem_u32(tc_smem_raw) & (kTAtom - 1))) & (kTAtom - 1));
-    unsigned char* sA = tc_smem;
-    unsigned char* sB = tc_smem + kTStages * kRABytes;
-    const int b = blockIdx.z;
-    const int v0 = blockIdx.x * kTM, v = v0 + tid;
-    const int x0 = v0 % a.W, y = (v0 / a.W) % a.H, z = v0 / (a.W * a.H);
-    constexpr int kJ = kK / 8;  // 16-byte chunks of a voxel's channels
-    uint32_t ncols = 32;
-    while ((int)ncols < BN) ncols <<= 1;
+    __shared__ __align__(8) uint64_t s_full[kMStages], s_empty[kMStages], s_bfull[3], s_bempty[2], s_afull[2],
+        s_aempty[2], s_drain;
+    __shared__ uint32_t s_tmem;
+    __shared__ int s_fail;
+    __shared__ int s_off[kMRows];  // source voxel of each staged row at y = 0 (-1: no such voxel)
+    const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
+    const uint32_t base = (smem_u32(tc_smem_raw) + kTAtom - 1) & ~(uint32_t)(kTAtom - 1);
+    const int NB = m.NB;
+    const uint32_t btap = (uint32_t)(3 * NB) * 128u;   // weights of one (dz, dx), one chunk: rows (dy block, n)
+    const uint32_t bbytes = 3u * kCh * btap;           // weights of one dz
+    const uint32_t sA = base + (m.resident ? 3u : 2u) * bbytes;
     if (tid == 0) {
-        for (int s = 0; s < kTStages; ++s) asm volatile("mbarrier.init.shared::cta.b64 [%0], 1;" ::"r"(smem_u32(&mbar[s])));
+        for (int s = 0; s < kMStages; ++s) {
+            asm volatile("mbarrier.init.shared::cta.b64 [%0], %1;" ::"r"(smem_u32(&s_full[s])), "n"(kMCopy));
+            asm volatile("mbarrier.init.shared::cta.b64 [%0], 1;" ::"r"(smem_u32(&s_empty[s])));
+        }
+        for (int s = 0; s < 3; ++s) asm volatile("mbarrier.init.shared::cta.b64 [%0], 1;" ::"r"(smem_u32(&s_bfull[s])));
+        for (int s = 0; s < 2; ++s) {
+            asm volatile("mbarrier.init.shared::cta.b64 [%0], 1;" ::"r"(smem_u32(&s_bempty[s])));
+            asm volatile("mbarrier.init.shared::cta.b64 [%0], 1;" ::"r"(smem_u32(&s_afull[s])));
+            asm volatile("mbarrier.init.shared::cta.b64 [%0], 4;" ::"r"(smem_u32(&s_aempty[s])));
+        }
+        asm volatile("mbarrier.init.shared::cta.b64 [%0], 1;" ::"r"(smem_u32(&s_drain)));
+        s_fail = 0;
         asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
     }
     if (warp == 0) {
-        asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(smem_u32(&tmem_base)),
-                     "r"(ncols));
+        asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(smem_u32(&s_tmem)),
+                     "r"(m.ncols));
         asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;");
     }
     asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
     __syncthreads();
     asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
-    const uint32_t tmem = tmem_base;
-    const bf16* xb = a.x + (size_t)b * a.V * kK;
+    const uint32_t tmem = s_tmem;
+    volatile int* fail = &s_fail;
+    const int H = m.c.H, W = m.c.W, sign = m.c.sign;
+    const int step = (int)gridDim.x;
 
-    // stage st = 3 (dz + 1) + (dy + 1): the source row and the three taps' weights
-    auto load_stage = [&](int st, int buf) {
-        const int dz = st / 3 - 1, dy = st % 3 - 1;
-        const int ys = wrap(y + a.sign * dy, a.H), zs = wrap(z + a.sign * dz, a.D);
-        const bf16* row = xb + (size_t)(zs * a.H + ys) * a.W * kK;
-        const uint32_t abase = smem_u32(sA + buf * kRABytes);
-        for (int p = tid; p < 130 * kJ; p += kTThreads) {
-            const int r = p / kJ, j = p - r * kJ;
-            const int x = wrap(x0 - 1 + r, a.W);
-            cp_async16(abase + swz(r, j), row + (size_t)x * kK + 8 * j, 16u);
-        }
-        const uint32_t bbase = smem_u32(sB + buf * 3 * BTile);
-        for (int p = tid; p < 3 * BN * kJ; p += kTThreads) {
-            const int t = p / (BN * kJ), q = p - t * (BN * kJ);
-            const int n = q / kJ, j = q - n * kJ;
-            const int tap = 3 * st + t;  // 9 (dz + 1) + 3 (dy + 1) + (dx + 1)
-            cp_async16(bbase + t * BTile + swz(n, j), a.w + ((size_t)tap * a.N + n0 + n) * kK + 8 * j, 16u);
-        }
-    };
-
-    bool ok = true;
-    constexpr int nst = 9;
-    for (int s = 0; s < kTStages - 1; ++s) {
-        load_stage(s, s);
-        asm volatile("cp.async.commit_group;" ::: "memory");
-    }
-    for (int st = 0; st < nst; ++st) {
-        const int buf = st % kTStages;
-        const int nxt = st + kTStages - 1;
-        if (nxt < nst) {
-            if (st >= 1) ok = mbar_wait(smem_u32(&mbar[(st - 1) % kTStages]), (uint32_t)(((st - 1) / kTStages) & 1));
-            if (ok) load_stage(nxt, nxt % kTStages);
-        }
-        asm volatile("cp.async.commit_group;" ::: "memory");
-        asm volatile("cp.async.wait_group %0;" ::"n"(kTStages - 1) : "memory");
-        asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
-        if (__syncthreads_or(!ok)) {
-            ok = false;
-            break;
-        }
-        if (tid == 0) {
-            asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
-            const uint32_t abase = smem_u32(sA + buf * kRABytes), bbase = smem_u32(sB + buf * 3 * BTile);
-            const uint32_t idesc = tc_idesc(BN);
+    if (warp >= 6) {
+        // ---- copies of source rows ----
+        constexpr int kP = (kMRows * kKC + kMCopy - 1) / kMCopy;  // 16-byte pieces per thread and row
+        const int pt = tid - 192;
+        int slot = 0;        // ring slot of the next stage
+        uint32_t round = 0;  // times the ring has been filled before
+        bool ok = true, all = true;  // all: no copying thread has given up (the same in every one of them)
+        for (int u = blockIdx.x; u < m.units && all; u += step) {
+            const int q = u / m.nblk;
+            const int strip = q % m.nstrip, tc = q / m.nstrip;
+            const int y0 = strip * m.T, te = min(m.T, H - y0);
+            for (int d = 0; d < 3; ++d) {
+                // the table's last readers are done; leave together when one of them gave up
+                all = bar_and(ok);
+                if (!all) break;
+                for (int row = pt; row < kMRows; row += kMCopy) {
+                    const int g = tc * 16 + row / 10;
+                    int off = -1;
+                    if (g < m.NG) {
+                        const int xg = g % m.GX, r = g / m.GX;
+                        const int z = r % m.c.D, b = r / m.c.D;
+                        const int x = wrap(8 * xg - 1 + row % 10, W);
+                        off = ((b * m.c.D + wrap(z + sign * (d - 1), m.c.D)) * H) * W + x;
+                    }
+                    s_off[row] = off;
+                }
+                asm volatile("barrier.cta.sync 1, %0;" ::"n"(kMCopy) : "memory");
+                int voff[kP];  // source voxel (at y = 0) of this thread's pieces of a row
 #pragma unroll
-            for (int t = 0; t < 3; ++t) {
-                // tap dx = t - 1 reads source voxel x + s dx: row 1 + s dx of the stage
-                const uint32_t arow = (uint32_t)(1 + a.sign * (t - 1)) * 128u;
+                for (int i = 0; i < kP; ++i) {
+                    const int p = pt + kMCopy * i;
+                    voff[i] = p < kMRows * kKC ? s_off[p / kKC] : -1;
+                }
+                for (int rr = 0; rr < te + 2; ++rr) {
+                    const int ys = wrap(y0 - 1 + (sign > 0 ? rr : te + 1 - rr), H);
+                    if (round > 0) ok = mbar_wait_or(smem_u32(&s_empty[slot]), (round - 1) & 1u, fail);
+                    if (!ok) break;
+                    const uint32_t dst = sA + (uint32_t)slot * kABytes;
+                    const bf16* xr = m.c.x + (size_t)ys * W * kK;
 #pragma unroll
-                for (int kk = 0; kk < kK; kk += 16) {
-                    const uint64_t ad = tc_desc(abase + arow + kk * 2), bd = tc_desc(bbase + t * BTile + kk * 2);
-                    const uint32_t accum = (st > 0 || t > 0 || kk > 0) ? 1u : 0u;
-                    asm volatile(
-                        "{\n.reg .pred p;\nsetp.ne.b32 p, %4, 0;\n"
-                        "tcgen05.mma.cta_group::1.kind::f16 [%0], %1, %2, %3, p;\n}" ::"r"(tmem),
-                        "l"(ad), "l"(bd), "r"(idesc), "r"(accum));
+                    for (int i = 0; i < kP; ++i) {
+                        const int p = pt + kMCopy * i, row = p / kKC, j = p - row * kKC;
+                        if (voff[i] >= 0)
+                            cp_async16(dst + (uint32_t)((j >> 3) * kMChunk + row * 128 + (((j & 7) ^ (row & 7)) << 4)),
+                                       xr + (size_t)voff[i] * kK + 8 * j, 16u);
+                    }
+                    // this thread's arrival at the stage's barrier, once its copies have landed
+                    asm volatile("cp.async.mbarrier.arrive.noinc.shared::cta.b64 [%0];" ::"r"(smem_u32(&s_full[slot]))
+                                 : "memory");
+                    if (++slot == m.nA) {
+                        slot = 0;
+                        ++round;
+                    }
                 }
             }
-            asm volatile("tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%0];" ::"r"(
-                             smem_u32(&mbar[buf]))
-                         : "memory");
+        }
+        asm volatile("cp.async.wait_all;" ::: "memory");
+    } else if (warp == 5) {
+        // ---- weights: those of one dz as nine boxes (dx, dy) of NB rows and 64 channels ----
+        if (lane == 0) {
+            int loads = 0;
+            bool ok = true;
+            for (int u = blockIdx.x; u < m.units && ok; u += step) {
+                const int n0 = (u % m.nblk) * NB;
+                if (m.resident && loads > 0) break;
+                for (int d = 0; d < 3; ++d, ++loads) {
+                    const int b = m.resident ? d : loads & 1;
+                    if (!m.resident && loads >= 2)
+                        ok = mbar_wait_or(smem_u32(&s_bempty[b]), (uint32_t)((loads >> 1) - 1) & 1u, fail);
+                    if (!ok) break;
+                    const uint32_t bar = smem_u32(&s_bfull[b]);
+                    asm volatile("{\n.reg .b64 t;\nmbarrier.arrive.expect_tx.shared::cta.b64 t, [%0], %1;\n}" ::"r"(bar),
+                                 "r"(bbytes)
+                                 : "memory");
+                    for (int dx = 0; dx < 3; ++dx)
+                        for (int ch = 0; ch < kCh; ++ch)
+                            for (int blk = 0; blk < 3; ++blk) {
+                                const int tap = 9 * d + 3 * (sign * (1 - blk) + 1) + dx;
+                                asm volatile(
+                                    "cp.async.bulk.tensor.3d.shared::cluster.global.tile.mbarrier::complete_tx::bytes "
+                                    "[%0], [%1, {%3, %4, %5}], [%2];" ::"r"(base + (uint32_t)b * bbytes +
+                                                                            (uint32_t)(dx * kCh + ch) * btap +
+                                                                            (uint32_t)(blk * NB) * 128u),
+                                    "l"(&wmap), "r"(bar), "r"(64 * ch), "r"(n0), "r"(tap)
+                                    : "memory");
+                            }
+                }
+            }
+            // no load may be in flight when the block ends (also after a failure elsewhere)
+            for (int k = max(0, loads - (m.resident ? 3 : 2)); k < loads; ++k)
+                mbar_wait(smem_u32(&s_bfull[m.resident ? k : k & 1]), m.resident ? 0u : (uint32_t)(k >> 1) & 1u);
+        }
+        __syncwarp();
+    } else if (warp == 4) {
+        // ---- MMAs: the warp stays converged (so that addresses stay in uniform registers) and
+        // one elected lane issues ----
+        const bool lead = elect_one();
+        int slot = 0, nu = 0;
+        uint32_t round = 0;
+        int nb_used = 0;
+        bool ok = true;
+        const int jfirst = sign > 0 ? 2 : 0;  // the block of the tap dy = -1: its output row's first
+        for (int u = blockIdx.x; u < m.units && ok; u += step, ++nu) {
+            const int strip = (u / m.nblk) % m.nstrip;
+            const int te = min(m.T, H - strip * m.T);
+            const int buf = m.bufs == 2 ? nu & 1 : 0;
+            const uint32_t acc = tmem + (uint32_t)(buf * m.T * NB);
+            const int use = m.bufs == 2 ? nu >> 1 : nu;
+            if (use > 0) ok = mbar_wait_or(smem_u32(&s_aempty[buf]), (uint32_t)(use - 1) & 1u, fail);
+            ok = __all_sync(0xffffffffu, ok);
+            if (!ok) break;
+            asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
+            for (int d = 0; d < 3 && ok; ++d) {
+                const int bb = m.resident ? d : nb_used & 1;
+                const uint32_t sB = base + (uint32_t)bb * bbytes;
+                if (!m.resident || nb_used < 3) {
+                    ok = mbar_wait_or(smem_u32(&s_bfull[bb]), m.resident ? 0u : (uint32_t)(nb_used >> 1) & 1u, fail);
+                    ok = __all_sync(0xffffffffu, ok);
+                    if (!ok) break;
+                }
+                for (int rr = 0; rr < te + 2; ++rr) {
+                    const int r = sign > 0 ? rr : te + 1 - rr;
+                    ok = mbar_wait_or(smem_u32(&s_full[slot]), round & 1u, fail);
+                    ok = __all_sync(0xffffffffu, ok);
+                    if (!ok) break;
+                    // the copies' writes, ordered before this thread by the barrier, are made
+                    // visible to the tensor core's reads (here and not in the copying
+                    // threads, where the fence would wait for every copy in flight)
+                    asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
+                    asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
+                    const int jlo = max(0, 2 - r), jhi = min(2, te + 1 - r);
+                    const uint32_t dcol = acc + (uint32_t)((r - 2 + jlo) * NB);
+                    const uint32_t idesc = tc_idesc((jhi - jlo + 1) * NB);
+                    const uint64_t a0 = tc_desc_stride(sA + (uint32_t)slot * kABytes + 128u, 1280u);
+                    const uint64_t b0 = tc_desc_stride(sB + (uint32_t)(jlo * NB) * 128u, kTAtom);
+                    if (lead) {
+#pragma unroll
+                        for (int dx = 0; dx < 3; ++dx) {
+#pragma unroll
+                            for (int sl = 0; sl < kK / 16; ++sl) {
+                                // descriptor addresses count 16 bytes
+                                const uint64_t ad = a0 + (uint64_t)((sl >> 2) * (kMChunk / 16) + (sl & 3) * 2) +
+                                                    (uint64_t)(int64_t)(sign * (dx - 1) * 8);
+                                const uint64_t bd = b0 + (uint64_t)((uint32_t)(dx * kCh + (sl >> 2)) * (btap / 16u)) +
+                                                    (uint64_t)((sl & 3) * 2);
+                                if (dx == 0 && sl == 0 && d == 0 && jfirst >= jlo && jfirst <= jhi) {
+                                    // this row is the first of output row r - 2 + jfirst: its
+                                    // accumulator starts here, the others go on
+                                    const uint32_t fo = (uint32_t)((jfirst - jlo) * NB);
+                                    tc_mma(dcol + fo, ad, bd + fo * 8u, tc_idesc(NB), 0u);
+                                    if (jhi > jlo) {
+                                        const uint32_t ro = jfirst == jlo ? (uint32_t)NB : 0u;
+                                        tc_mma(dcol + ro, ad, bd + ro * 8u, tc_idesc((jhi - jlo) * NB), 1u);
+                                    }
+                                } else {
+                                    tc_mma(dcol, ad, bd, idesc, 1u);
+                                }
+                            }
+                        }
+                        tc_commit(smem_u32(&s_empty[slot]));
+                    }
+                    if (++slot == m.nA) {
+                        slot = 0;
+                        ++round;
+                    }
+                }
+                if (ok && !m.resident && lead) tc_commit(smem_u32(&s_bempty[nb_used & 1]));
+                ++nb_used;
+            }
+            if (ok && lead) tc_commit(smem_u32(&s_afull[buf]));
+        }
+        if (!ok && lead) {
+            // MMAs issued before the failure still use this block's memories: wait for them
+            tc_commit(smem_u32(&s_drain));
+            mbar_wait(smem_u32(&s_drain), 0u);
+        }
+        __syncwarp();
+    } else {
+        // ---- epilogue ----
+        int nu = 0;
+        bool ok = true;
+        for (int u = blockIdx.x; u < m.units; u += step, ++nu) {
+            const int nbk = u % m.nblk, q = u / m.nblk;
+            const int strip = q % m.nstrip, tc = q / m.nstrip;
+            const int y0 = strip * m.T, te = min(m.T, H - y0);
+            const int buf = m.bufs == 2 ? nu & 1 : 0;
+            const int use = m.bufs == 2 ? nu >> 1 : nu;
+            const int g = tc * 16 + tid / 8;
+            const int xg = g % m.GX, r = g / m.GX;   // r = b D + z
+            const long long v0 = g < m.NG ? ((long long)r * H + y0) * W + 8 * xg + (tid & 7) : -1;
+            ok = mbar_wait_or(smem_u32(&s_afull[buf]), (uint32_t)use & 1u, fail);
+            if (!__all_sync(0xffffffffu, ok)) break;
+            asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
+            for (int t = 0; t < te; ++t)
+                conv_store_row(m.c, tmem + (uint32_t)((buf * m.T + t) * NB), warp, v0 < 0 ? -1 : v0 + (long long)t * W,
+                               nbk * NB, NB);
+            asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
+            __syncwarp();
+            if (lane == 0) mbar_arrive(smem_u32(&s_aempty[buf]));
         }
     }
-    asm volatile("cp.async.wait_all;" ::: "memory");
-    if (ok) ok = mbar_wait(smem_u32(&mbar[(nst - 1) % kTStages]), (uint32_t)(((nst - 1) / kTStages) & 1));
-    if (!ok && tid == 0) atomicExch(&g_sg_tc_fail, 1);
-    asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
-    if (__syncthreads_and(ok)) conv_epilogue(a, tmem, warp, b, v, n0, BN);
     asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
     __syncthreads();
-    if (warp == 0) asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(tmem), "r"(ncols));
+    if (tid == 0 && s_fail) atomicExch(&g_sg_tc_fail, 1);
+    if (warp == 0)
+        asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(tmem), "r"(m.ncols));
 }
 
 struct WgradArgs {
@@ -783,6 +1030,101 @@ __global__ void k_adam(float* __restrict__ p, const float* __restrict__ g, float
     }
 }
 
+// Tensor map of the weights [27][N][K] for boxes of NB output channels x 64 input channels
+// (channels beyond K read as zero; 128-byte swizzle). False where the driver does not offer the
+// encoder or refuses the address.
+typedef CUresult (*EncodeTiledFn)(CUtensorMap*, CUtensorMapDataType, cuuint32_t, void*, const cuuint64_t*,
+                                  const cuuint64_t*, const cuuint32_t*, const cuuint32_t*, CUtensorMapInterleave,
+                                  CUtensorMapSwizzle, CUtensorMapL2promotion, CUtensorMapFloatOOBfill);
+EncodeTiledFn tensor_map_encoder()
+{
+    static const EncodeTiledFn fn = [] {
+        void* p = nullptr;
+        cudaDriverEntryPointQueryResult q;
+        if (cudaGetDriverEntryPointByVersion("cuTensorMapEncodeTiled", &p, 12000, cudaEnableDefault, &q) != cudaSuccess ||
+            q != cudaDriverEntryPointSuccess) {
+            (void)cudaGetLastError();
+            p = nullptr;
+        }
+        return (EncodeTiledFn)p;
+    }();
+    return fn;
+}
+
+bool weight_map(const ConvArgs& a, int NB, CUtensorMap* map)
+{
+    const EncodeTiledFn encode = tensor_map_encoder();
+    if (!encode) return false;
+    const cuuint64_t dims[3] = {(cuuint64_t)a.K, (cuuint64_t)a.N, 27};
+    const cuuint64_t strides[2] = {(cuuint64_t)a.K * 2, (cuuint64_t)a.K * a.N * 2};
+    const cuuint32_t box[3] = {64, (cuuint32_t)NB, 1}, one[3] = {1, 1, 1};
+    return encode(map, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 3, const_cast<bf16*>(a.w), dims, strides, box, one,
+                  CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_128B, CU_TENSOR_MAP_L2_PROMOTION_L2_128B,
+                  CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) == CUDA_SUCCESS;
+}
+
+// Shape of the marching kernel for one layer, or false where it does not apply. The channel
+// block NB and the strip length T are those with the least estimated time: waves of one unit
+// per SM times the clocks of a unit, where a staged row costs the larger of its MMAs (products
+// at 4096 per clock, operands at 128 bytes per clock), its copies (about 40 bytes per clock
+// and SM from L2) and 250 clocks of hand-over.
+bool march_plan(const ConvArgs& a, int B, int sms, MarchArgs* out, size_t* smem)
+{
+    const int K = a.K, N = a.N;
+    if (a.W % 8 || !(K == 16 || K == 32 || K == 64 || K == 96 || K == 128) || (long long)B * a.V >= (1LL << 31)) return false;
+    const int kch = (K + 63) / 64;
+    const size_t abytes = (size_t)kch * kMChunk;
+    MarchArgs best{};
+    double best_cost = 0.0;
+    size_t best_smem = 0;
+    for (int nblk = 1; nblk * 16 <= N; ++nblk) {
+        if (N % (16 * nblk)) continue;
+        const int NB = N / nblk;
+        if (3 * NB > 256) continue;
+        const size_t bbytes = (size_t)3 * kch * 3 * NB * 128;
+        const bool resident = nblk == 1 && 3 * bbytes + 3 * abytes <= (size_t)kMSmem - 1024;
+        const size_t bsm = (resident ? 3 : 2) * bbytes;
+        if (bsm + 2 * abytes > (size_t)kMSmem - 1024) continue;
+        const int nA = (int)std::min<size_t>(kMStages, ((size_t)kMSmem - 1024 - bsm) / abytes);
+        for (int T = 1; T <= a.H && T <= 16 && T * NB <= 512; T = T < 4 ? T + 1 : T + 2) {
+            const int bufs = 2 * T * NB <= 512 ? 2 : 1;
+            const int GX = a.W / 8, NG = B * a.D * GX;
+            const long long units = (long long)((NG + 15) / 16) * ((a.H + T - 1) / T) * nblk;
+            if (units > (1LL << 30)) continue;
+            double rows = 0.0;
+            for (int r = 0; r < T + 2; ++r) {
+                const int nn = (std::min(2, T + 1 - r) - std::max(0, 2 - r) + 1) * NB;
+                const double mma = 3.0 * (K / 16) * std::max(nn / 2.0, 32.0 + nn / 4.0);
+                rows += std::max(std::max(mma, kMRows * K * 2 / 40.0), 250.0);
+            }
+            const double unit = 3.0 * rows + (resident ? 0.0 : 3.0 * 9 * NB * K * 2 / 100.0) +
+                                (bufs == 1 ? 8.0 * T * NB : 0.0) + 500.0;
+            const double cost = (double)((units + sms - 1) / sms) * unit + 3000.0 + 8.0 * T * NB;
+            if (best_cost == 0.0 || cost < best_cost) {
+                best_cost = cost;
+                best.c = a;
+                best.GX = GX;
+                best.NG = NG;
+                best.T = T;
+                best.nstrip = (a.H + T - 1) / T;
+                best.NB = NB;
+                best.nblk = nblk;
+                best.units = (int)units;
+                best.nA = nA;
+                best.resident = resident ? 1 : 0;
+                best.bufs = bufs;
+                best.ncols = 32;
+                while ((int)best.ncols < bufs * T * NB) best.ncols <<= 1;
+                best_smem = bsm + nA * abytes + 1024;
+            }
+        }
+    }
+    if (best_cost == 0.0) return false;
+    *out = best;
+    *smem = best_smem;
+    return true;
+}
+
 int grid1(long long n, int block) { return (int)((n + block - 1) / block); }
 
 }  // namespace
@@ -800,14 +1142,20 @@ int sg_conv3d(const void* x, const void* w, const float* bias, void* y, float* y
     }
     ConvArgs a{(const bf16*)x, (const bf16*)w, bias, (bf16*)y, yf, D, H, W, D * H * W, K, N, sign, relu != 0};
     const int bn = N < kTMaxN ? N : kTMaxN;
-    if (W % kTM == 0 && (K == 16 || K == 32 || K == 64) && N <= kRMaxN) {
-        // blocks of 128 voxels lie in one x-row: the row-staged kernel
-        void (*rkern)(const ConvArgs) = K == 16 ? k_conv_row<16> : K == 32 ? k_conv_row<32> : k_conv_row<64>;
-        const size_t rsmem = (size_t)kTStages * (kRABytes + 3 * (size_t)(bn / 8) * kTAtom) + kTAtom;
-        MP_CUDA(cudaFuncSetAttribute(rkern, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                     (int)(kTStages * (kRABytes + 3 * (kRMaxN / 8) * kTAtom) + kTAtom)));
-        dim3 grid(a.V / kTM, (N + kTMaxN - 1) / kTMaxN, B);
-        rkern<<<grid, kTThreads, rsmem, (cudaStream_t)stream>>>(a);
+    int dev = 0, sms = 0;
+    MP_CUDA(cudaGetDevice(&dev));
+    MP_CUDA(cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev));
+    MarchArgs m;
+    size_t msmem = 0;
+    CUtensorMap wmap;
+    if (march_plan(a, B, sms, &m, &msmem) && weight_map(a, m.NB, &wmap)) {
+        void (*mkern)(const MarchArgs, const CUtensorMap) = K == 16   ? k_conv_march<16>
+                                         : K == 32 ? k_conv_march<32>
+                                         : K == 64 ? k_conv_march<64>
+                                         : K == 96 ? k_conv_march<96>
+                                                   : k_conv_march<128>;
+        MP_CUDA(cudaFuncSetAttribute(mkern, cudaFuncAttributeMaxDynamicSharedMemorySize, kMSmem));
+        mkern<<<std::min(m.units, sms), kMThreads, msmem, (cudaStream_t)stream>>>(m, wmap);
         MP_CUDA(cudaGetLastError());
         return MP_OK;
     }
