@@ -679,6 +679,281 @@ __global__ void __launch_bounds__(kMThreads, 1) k_conv_march(const __grid_consta
         asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(tmem), "r"(m.ncols));
 }
 
+// ---------------------------------------------------------------------------------------
+// Weight gradient on the 5th-generation tensor cores (W a multiple of 8): dW[tap][ci][co] is a
+// product over voxels of x rows and dy rows, both channels-last, i.e. both operands with the
+// reduction index (voxels) as rows of shared memory: MN-major operands. What bounds a
+// tap-by-tap kernel is reading x and dy once per tap (27 times); here a unit takes one dz, a
+// block of CI input and CO output channels, a column of 128 voxels (16 groups of 8
+// x-neighbours, as in k_conv_march) and T rows of x:
+//  * N = 3 CI: the three taps dx are three column blocks of one operand, the staged x row
+//    read from row 0, 1 and 2 of each 10-row group: the descriptor's stride between
+//    64-, 32- or 16-channel blocks is one staged row;
+//  * M = 3 CO (padded to 128, or two tiles of 128 for CO = 64): the three taps dy are the dy
+//    rows y + 1, y, y - 1, neighbouring slots of a ring: the stride between channel blocks is
+//    one slot. The ring's first two slots are copied a second time behind its end, so that
+//    three consecutive rows are always consecutive slots; rows of M beyond 3 CO read whatever
+//    the next slots hold and are dropped.
+// So x and dy are read three times in all (once per dz), and an MMA of K = 16 voxels serves
+// nine taps. Rows of 128, 64 or 32 bytes use the swizzle of that width. A unit's sums (T rows,
+// at most 2048 voxels: partial sums stay as short as those of the kernel below) are added to
+// dw with one reduction per element, 32 consecutive output channels per warp.
+// Measured (tap by tap with mma.sync -> this): one 128^3 box 32 -> 32 channels 2266 -> 157 us,
+// 64 -> 32 2297 -> 208 us (1117 TFLOP/s); 64^3 64 -> 64 365 -> 60 us; 16^3 128 -> 128 56 -> 13 us.
+// 13 warps: 4 epilogue, 1 MMA, 8 copies (cp.async, zero-filled for groups beyond the batch).
+// Waits are bounded as in k_conv_march.
+// ---------------------------------------------------------------------------------------
+constexpr int kGThreads = 160 + kMCopy;
+constexpr int kGStages = 8;
+
+struct WgradTcArgs {
+    const bf16* x;
+    const bf16* dy;
+    float* dw;
+    int D, H, W, Cin, Cout;
+    int GX, NG;          // groups per x-row, groups over the batch
+    int T, nstrip;       // x rows per unit, strips along y
+    int nci, nco, units;
+    int nX;              // ring stages (x rows); the dy ring has nX + 4 slots
+    int bufs;            // accumulator sets
+    uint32_t ncols;      // tensor-memory columns
+};
+
+// MN-major descriptor: `lbo` bytes between channel blocks of one swizzle width, `sbo` between
+// groups of 8 rows; swizzle mode of a row of `row` bytes
+template <int kRow>
+__device__ __forceinline__ uint64_t tc_desc_mn(uint32_t addr, uint32_t lbo, uint32_t sbo)
+{
+    constexpr uint64_t mode = kRow == 128 ? 2 : (kRow == 64 ? 4 : 6);
+    return (uint64_t)((addr & 0x3FFFFu) >> 4) | ((uint64_t)(lbo >> 4) << 16) | ((uint64_t)(sbo >> 4) << 32) |
+           (1ull << 46) | (mode << 61);
+}
+
+// offset of 16-byte piece j of a row of kRow bytes under that swizzle (slots start on 1024 bytes)
+template <int kRow>
+__device__ __forceinline__ uint32_t swz_row(int r, int j)
+{
+    return (uint32_t)(r * kRow + ((j ^ (((r * kRow) >> 7) & (kRow / 16 - 1))) << 4));
+}
+
+template <int kCI, int kCO>
+__global__ void __launch_bounds__(kGThreads, 1) k_wgrad_tc(const __grid_constant__ WgradTcArgs m)
+{
+    constexpr int kRX = 2 * kCI, kRY = 2 * kCO;              // bytes of a staged row
+    constexpr uint32_t kXB = kMRows * kRX, kYB = kTM * kRY;  // bytes of a slot
+    constexpr int kTiles = kCO == 64 ? 2 : 1, kN = 3 * kCI;
+    extern __shared__ __align__(1024) unsigned char tc_smem_raw[];
+    __shared__ __align__(8) uint64_t s_full[kGStages], s_empty[kGStages], s_afull[2], s_aempty[2], s_drain;
+    __shared__ uint32_t s_tmem;
+    __shared__ int s_fail;
+    __shared__ int s_xoff[kMRows], s_yoff[kTM];  // voxels of the staged rows at y = 0 (-1: none)
+    const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
+    const uint32_t base = (smem_u32(tc_smem_raw) + kTAtom - 1) & ~(uint32_t)(kTAtom - 1);
+    const int R = m.nX + 4;
+    const uint32_t sX = base, sY = base + (uint32_t)m.nX * kXB;
+    if (tid == 0) {
+        for (int s = 0; s < kGStages; ++s) {
+            asm volatile("mbarrier.init.shared::cta.b64 [%0], %1;" ::"r"(smem_u32(&s_full[s])), "n"(kMCopy));
+            asm volatile("mbarrier.init.shared::cta.b64 [%0], 1;" ::"r"(smem_u32(&s_empty[s])));
+        }
+        for (int s = 0; s < 2; ++s) {
+            asm volatile("mbarrier.init.shared::cta.b64 [%0], 1;" ::"r"(smem_u32(&s_afull[s])));
+            asm volatile("mbarrier.init.shared::cta.b64 [%0], 4;" ::"r"(smem_u32(&s_aempty[s])));
+        }
+        asm volatile("mbarrier.init.shared::cta.b64 [%0], 1;" ::"r"(smem_u32(&s_drain)));
+        s_fail = 0;
+        asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
+    }
+    if (warp == 0) {
+        asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(smem_u32(&s_tmem)),
+                     "r"(m.ncols));
+        asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;");
+    }
+    asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
+    __syncthreads();
+    asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
+    const uint32_t tmem = s_tmem;
+    volatile int* fail = &s_fail;
+    const int H = m.H, W = m.W, step = (int)gridDim.x;
+    const int combos = 3 * m.nci * m.nco;
+
+    if (warp >= 5) {
+        // ---- copies ----
+        constexpr int kPX = kRX / 16, kPY = kRY / 16;
+        constexpr int kNX = (kMRows * kPX + kMCopy - 1) / kMCopy, kNY = kTM * kPY / kMCopy;
+        const int pt = tid - 160;
+        int slot = 0, ys = 0;  // x slot of the next stage, dy slot of the next dy row
+        uint32_t round = 0;
+        bool ok = true, all = true;
+        for (int u = blockIdx.x; u < m.units && all; u += step) {
+            const int combo = u % combos, q = u / combos;
+            const int d = combo % 3, ci0 = (combo / 3) % m.nci * kCI, co0 = combo / (3 * m.nci) * kCO;
+            const int strip = q % m.nstrip, tc = q / m.nstrip;
+            const int y0 = strip * m.T, te = min(m.T, H - y0);
+            all = bar_and(ok);
+            if (!all) break;
+            for (int row = pt; row < kMRows + kTM; row += kMCopy) {
+                const bool isx = row < kMRows;
+                const int r = isx ? row : row - kMRows;
+                const int g = tc * 16 + (isx ? r / 10 : r / 8);
+                int off = -1;
+                if (g < m.NG) {
+                    const int xg = g % m.GX, l = g / m.GX;
+                    const int z = l % m.D, b = l / m.D;
+                    const int x = isx ? wrap(8 * xg - 1 + r % 10, W) : 8 * xg + r % 8;
+                    off = ((b * m.D + (isx ? wrap(z + d - 1, m.D) : z)) * H) * W + x;
+                }
+                if (isx)
+                    s_xoff[r] = off;
+                else
+                    s_yoff[r] = off;
+            }
+            asm volatile("barrier.cta.sync 1, %0;" ::"n"(kMCopy) : "memory");
+            int xo[kNX], yo[kNY];
+#pragma unroll
+            for (int i = 0; i < kNX; ++i) {
+                const int p = pt + kMCopy * i;
+                xo[i] = p < kMRows * kPX ? s_xoff[p / kPX] : -2;
+            }
+#pragma unroll
+            for (int i = 0; i < kNY; ++i) yo[i] = s_yoff[(pt + kMCopy * i) / kPY];
+            // dy row y into the next slot of the ring (and its copy behind the ring's end)
+            auto load_y = [&](int y) {
+                const bf16* src = m.dy + (size_t)y * W * m.Cout + co0;
+#pragma unroll
+                for (int i = 0; i < kNY; ++i) {
+                    const int p = pt + kMCopy * i, row = p / kPY, j = p - row * kPY;
+                    const bf16* s = src + (yo[i] >= 0 ? (size_t)yo[i] * m.Cout + 8 * j : 0);
+                    const uint32_t at = sY + swz_row<kRY>(row, j), n = yo[i] >= 0 ? 16u : 0u;
+                    cp_async16(at + (uint32_t)ys * kYB, s, n);
+                    if (ys < 2) cp_async16(at + (uint32_t)(ys + R) * kYB, s, n);
+                }
+                ys = ys + 1 == R ? 0 : ys + 1;
+            };
+            for (int i = 0; i < te; ++i) {
+                if (round > 0) ok = mbar_wait_or(smem_u32(&s_empty[slot]), (round - 1) & 1u, fail);
+                if (!ok) break;
+                if (i == 0) {
+                    load_y(wrap(y0 - 1, H));
+                    load_y(y0);
+                }
+                load_y(wrap(y0 + i + 1, H));
+                const bf16* src = m.x + (size_t)(y0 + i) * W * m.Cin + ci0;
+#pragma unroll
+                for (int k = 0; k < kNX; ++k) {
+                    const int p = pt + kMCopy * k, row = p / kPX, j = p - row * kPX;
+                    if (xo[k] != -2)
+                        cp_async16(sX + (uint32_t)slot * kXB + swz_row<kRX>(row, j),
+                                   src + (xo[k] >= 0 ? (size_t)xo[k] * m.Cin + 8 * j : 0), xo[k] >= 0 ? 16u : 0u);
+                }
+                asm volatile("cp.async.mbarrier.arrive.noinc.shared::cta.b64 [%0];" ::"r"(smem_u32(&s_full[slot]))
+                             : "memory");
+                if (++slot == m.nX) {
+                    slot = 0;
+                    ++round;
+                }
+            }
+        }
+        asm volatile("cp.async.wait_all;" ::: "memory");
+    } else if (warp == 4) {
+        // ---- MMAs ----
+        constexpr uint32_t kIdesc = tc_idesc(kN) | (1u << 15) | (1u << 16);  // both operands MN-major
+        const bool lead = elect_one();
+        int slot = 0, ys = 0, nu = 0;
+        uint32_t round = 0;
+        bool ok = true;
+        for (int u = blockIdx.x; u < m.units && ok; u += step, ++nu) {
+            const int strip = (u / combos) % m.nstrip;
+            const int te = min(m.T, H - strip * m.T);
+            const int buf = m.bufs == 2 ? nu & 1 : 0;
+            const int use = m.bufs == 2 ? nu >> 1 : nu;
+            const uint32_t acc = tmem + (uint32_t)(buf * kTiles * kN);
+            if (use > 0) ok = mbar_wait_or(smem_u32(&s_aempty[buf]), (uint32_t)(use - 1) & 1u, fail);
+            ok = __all_sync(0xffffffffu, ok);
+            if (!ok) break;
+            asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
+            for (int i = 0; i < te; ++i) {
+                ok = mbar_wait_or(smem_u32(&s_full[slot]), round & 1u, fail);
+                ok = __all_sync(0xffffffffu, ok);
+                if (!ok) break;
+                asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
+                asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
+                const uint64_t a0 = tc_desc_mn<kRY>(sY + (uint32_t)ys * kYB, kYB, 8u * kRY);
+                const uint64_t b0 = tc_desc_mn<kRX>(sX + (uint32_t)slot * kXB, kRX, 10u * kRX);
+                if (lead) {
+#pragma unroll
+                    for (int k = 0; k < 8; ++k)
+#pragma unroll
+                        for (int t = 0; t < kTiles; ++t)
+                            tc_mma(acc + (uint32_t)(t * kN), a0 + (uint64_t)(k * (16 * kRY / 16) + t * (2 * (int)kYB / 16)),
+                                   b0 + (uint64_t)(k * (20 * kRX / 16)), kIdesc, (i > 0 || k > 0) ? 1u : 0u);
+                    tc_commit(smem_u32(&s_empty[slot]));
+                }
+                ys = ys + 1 == R ? 0 : ys + 1;
+                if (++slot == m.nX) {
+                    slot = 0;
+                    ++round;
+                }
+            }
+            ys = ys + 2 >= R ? ys + 2 - R : ys + 2;  // the unit's last two dy rows
+            if (ok && lead) tc_commit(smem_u32(&s_afull[buf]));
+        }
+        if (!ok && lead) {
+            // MMAs issued before the failure still use this block's memories: wait for them
+            tc_commit(smem_u32(&s_drain));
+            mbar_wait(smem_u32(&s_drain), 0u);
+        }
+        __syncwarp();
+    } else {
+        // ---- epilogue: accumulator row = (dy block, output channel), column = (dx, input channel) ----
+        int nu = 0;
+        for (int u = blockIdx.x; u < m.units; u += step, ++nu) {
+            const int combo = u % combos;
+            const int d = combo % 3, ci0 = (combo / 3) % m.nci * kCI, co0 = combo / (3 * m.nci) * kCO;
+            const int buf = m.bufs == 2 ? nu & 1 : 0;
+            const int use = m.bufs == 2 ? nu >> 1 : nu;
+            const bool ok = mbar_wait_or(smem_u32(&s_afull[buf]), (uint32_t)use & 1u, fail);
+            if (!__all_sync(0xffffffffu, ok)) break;
+            asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
+#pragma unroll
+            for (int t = 0; t < kTiles; ++t) {
+                if (t * 128 + 32 * warp >= 3 * kCO) continue;  // the whole warp's rows are padding
+                const int r = t * 128 + tid, j = r / kCO;  // j > 2: padding
+                // block j: dy row y - 1 + j, tap dy = 1 - j
+                float* out = m.dw + ((size_t)(9 * d + 3 * (2 - min(j, 2))) * m.Cin + ci0) * m.Cout + co0 + (r - j * kCO);
+#pragma unroll 1
+                for (int c0 = 0; c0 < kN; c0 += 16) {
+                    uint32_t v[16];
+                    const uint32_t addr =
+                        tmem + ((uint32_t)(32 * warp) << 16) + (uint32_t)((buf * kTiles + t) * kN + c0);
+                    asm volatile(
+                        "tcgen05.ld.sync.aligned.32x32b.x16.b32 "
+                        "{%0,%1,%2,%3,%4,%5,%6,%7,%8,%9,%10,%11,%12,%13,%14,%15}, [%16];"
+                        : "=r"(v[0]), "=r"(v[1]), "=r"(v[2]), "=r"(v[3]), "=r"(v[4]), "=r"(v[5]), "=r"(v[6]),
+                          "=r"(v[7]), "=r"(v[8]), "=r"(v[9]), "=r"(v[10]), "=r"(v[11]), "=r"(v[12]), "=r"(v[13]),
+                          "=r"(v[14]), "=r"(v[15])
+                        : "r"(addr));
+                    asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory");
+                    if (j < 3) {
+                        float* o = out + ((size_t)(c0 / kCI) * m.Cin + c0 % kCI) * m.Cout;
+#pragma unroll
+                        for (int c = 0; c < 16; ++c) atomicAdd(o + (size_t)c * m.Cout, __uint_as_float(v[c]));
+                    }
+                    __syncwarp();
+                }
+            }
+            asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
+            __syncwarp();
+            if (lane == 0) mbar_arrive(smem_u32(&s_aempty[buf]));
+        }
+    }
+    asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
+    __syncthreads();
+    if (tid == 0 && s_fail) atomicExch(&g_sg_tc_fail, 1);
+    if (warp == 0)
+        asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(tmem), "r"(m.ncols));
+}
+
 struct WgradArgs {
     const bf16* x;
     const bf16* dy;
@@ -1125,6 +1400,64 @@ bool march_plan(const ConvArgs& a, int B, int sms, MarchArgs* out, size_t* smem)
     return true;
 }
 
+int channel_block(int c) { return c % 64 == 0 ? 64 : (c % 32 == 0 ? 32 : 16); }
+
+// Shape of k_wgrad_tc for one layer, or false where it does not apply. T is the one with the
+// least estimated time (waves of units x clocks of a unit, as in march_plan) that keeps a
+// unit within 16 rows.
+bool wgrad_plan(const WgradArgs& a, int B, int sms, WgradTcArgs* m, size_t* smem)
+{
+    if (a.W % 8 || a.total >= (1LL << 31)) return false;
+    const int ci = channel_block(a.Cin), co = channel_block(a.Cout);
+    const size_t xb = (size_t)kMRows * 2 * ci, yb = (size_t)kTM * 2 * co;
+    const int tiles = co == 64 ? 2 : 1, n = 3 * ci;
+    // dy slots: the ring, two copies and what the padding rows of M read beyond a window
+    const int pad = tiles * 128 / co - 1;
+    int nX = kGStages;
+    while (nX > 1 && nX * xb + (nX + 4 + pad) * yb > (size_t)kMSmem - 2048) --nX;
+    if (nX < 2) return false;
+    m->x = a.x;
+    m->dy = a.dy;
+    m->dw = a.dw;
+    m->D = a.D;
+    m->H = a.H;
+    m->W = a.W;
+    m->Cin = a.Cin;
+    m->Cout = a.Cout;
+    m->GX = a.W / 8;
+    m->NG = B * a.D * m->GX;
+    m->nci = a.Cin / ci;
+    m->nco = a.Cout / co;
+    m->nX = nX;
+    m->bufs = 2 * tiles * n <= 512 ? 2 : 1;
+    m->ncols = 32;
+    while ((int)m->ncols < m->bufs * tiles * n) m->ncols <<= 1;
+    const double row = std::max(std::max(8.0 * tiles * std::max(n / 2.0, 32.0 + n / 4.0), (xb + yb) / 40.0), 300.0);
+    const double flush = 12.0 * tiles * n;
+    const long long per_row = (long long)3 * m->nci * m->nco * ((m->NG + 15) / 16);
+    double best = 0.0;
+    for (int T = 1; T <= a.H && T <= 16; ++T) {
+        const long long units = per_row * ((a.H + T - 1) / T);
+        if (units > (1LL << 30)) continue;
+        const double unit = std::max(T * row + 2.0 * yb / 40.0 + (m->bufs == 1 ? flush : 0.0), flush) + 500.0;
+        const double cost = (double)((units + sms - 1) / sms) * unit + flush;
+        if (best == 0.0 || cost < best) {
+            best = cost;
+            m->T = T;
+            m->nstrip = (a.H + T - 1) / T;
+            m->units = (int)units;
+        }
+    }
+    *smem = nX * xb + (nX + 4 + pad) * yb + 1024;
+    return best > 0.0;
+}
+
+template <int kCI>
+void (*wgrad_kernel(int co))(const WgradTcArgs)
+{
+    return co == 64 ? k_wgrad_tc<kCI, 64> : (co == 32 ? k_wgrad_tc<kCI, 32> : k_wgrad_tc<kCI, 16>);
+}
+
 int grid1(long long n, int block) { return (int)((n + block - 1) / block); }
 
 }  // namespace
@@ -1203,17 +1536,31 @@ int sg_conv3d_wgrad(const void* x, const void* dy, float* dw, float* dbias, int 
     const int ci_tiles = (Cin + kWM - 1) / kWM, co_tiles = (Cout + kWN - 1) / kWN;
     WgradArgs a{(const bf16*)x, (const bf16*)dy, dw, D, H, W, D * H * W, Cin, Cout, (long long)B * D * H * W, 2048,
                 ci_tiles};
+    cudaStream_t cs = (cudaStream_t)stream;
     const long long nchunk = (a.total + a.chunk - 1) / a.chunk;
+    int dev = 0, sms = 0;
+    MP_CUDA(cudaGetDevice(&dev));
+    MP_CUDA(cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev));
+    WgradTcArgs m;
+    size_t smem = 0;
+    const bool tc = wgrad_plan(a, B, sms, &m, &smem);
     if (nchunk * 27 > 2147483647LL || ci_tiles * co_tiles > 65535) {
         set_error("sg_conv3d_wgrad: too many voxels or channels");
         return MP_EINVAL;
     }
-    dim3 grid((unsigned)(nchunk * 27), (unsigned)(ci_tiles * co_tiles));
-    k_wgrad<<<grid, kWThreads, 0, (cudaStream_t)stream>>>(a);
+    if (tc) {
+        const int ci = channel_block(Cin), co = channel_block(Cout);
+        auto kern = ci == 64 ? wgrad_kernel<64>(co) : (ci == 32 ? wgrad_kernel<32>(co) : wgrad_kernel<16>(co));
+        MP_CUDA(cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, kMSmem - 1024));
+        kern<<<std::min(m.units, sms), kGThreads, smem, cs>>>(m);
+    } else {
+        dim3 grid((unsigned)(nchunk * 27), (unsigned)(ci_tiles * co_tiles));
+        k_wgrad<<<grid, kWThreads, 0, cs>>>(a);
+    }
     MP_CUDA(cudaGetLastError());
     if (dbias) {
         dim3 gb(grid1(a.total, 256), (Cout + 31) / 32);
-        k_bias_grad<<<gb, 256, 0, (cudaStream_t)stream>>>((const bf16*)dy, dbias, a.total, Cout);
+        k_bias_grad<<<gb, 256, 0, cs>>>((const bf16*)dy, dbias, a.total, Cout);
         MP_CUDA(cudaGetLastError());
     }
     return MP_OK;
