@@ -13,7 +13,7 @@
  *    [27][N][K] order (tap-major; tap = 9*(dz+1) + 3*(dy+1) + (dx+1)): N output channels by
  *    K input channels for the forward pass. Master weights and gradients are FP32 in
  *    [27][Cin][Cout] order. Biases are FP32.
- *  - Products run on the tensor cores (mma.sync m16n8k16, BF16 inputs, FP32 accumulation).
+ *  - Products run on the tensor cores (BF16 inputs, FP32 accumulation).
  *  - Every pointer is device memory; every call is asynchronous on `stream` (a
  *    cudaStream_t, NULL = legacy default stream) and returns MP_OK or MP_EINVAL/MP_ECUDA.
  */
@@ -42,6 +42,19 @@ int sg_conv3d(const void* x, const void* w, const float* bias, void* y, float* y
               int W, int K, int N, int sign, int relu, void* stream);
 
 /*
+ * sg_conv3d_ex -- sg_conv3d with what surrounds it in the network, the same results as the
+ * separate calls in one pass over memory:
+ *  y2, other  BF16 [B][V][N], given together with mode 1 or 2, NULL with mode 0. With yb =
+ *             act(...) rounded to BF16 (what y receives): mode 1, y2 = yb + other (the skip
+ *             connection; sg_add); mode 2, y2 = yb where other > 0, else 0 (the ReLU gradient;
+ *             sg_relu_grad). y, yf and y2 may be given in any combination, at least one.
+ *  up         nonzero: x is BF16 [B][D/2][H/2][W/2][K] and is read as its nearest-neighbour 2x
+ *             upsampling (sg_up2); D, H, W even.
+ */
+int sg_conv3d_ex(const void* x, const void* w, const float* bias, void* y, float* yf, void* y2, const void* other,
+                 int mode, int up, int B, int D, int H, int W, int K, int N, int sign, int relu, void* stream);
+
+/*
  * sg_check -- synchronises the stream and returns MP_ETIMEOUT (clearing the record) when a
  * bounded wait inside a tensor-core convolution launched since the last check gave up, so
  * that its output is not valid; MP_OK otherwise. (No counterpart in the paper.)
@@ -52,10 +65,15 @@ int sg_check(void* stream);
  * sg_conv3d_wgrad -- dw[tap][ci][co] += sum_{b, v} x[b][v + o_tap][ci] dy[b][v][co] and, when
  * dbias is not NULL, dbias[co] += sum_{b, v} dy[b][v][co] (FP32 accumulation; the caller
  * zeroes dw and dbias before the first call of a step). x BF16 [B][V][Cin], dy BF16
- * [B][V][Cout]. Summation order varies between runs (atomic adds).
+ * [B][V][Cout]. Summation order varies between runs (atomic adds). W a multiple of 8 runs on
+ * the 5th-generation tensor cores with bounded waits (sg_check), other widths with mma.sync.
+ * sg_conv3d_wgrad_ex: the same with x BF16 [B][D/2][H/2][W/2][Cin] read as its nearest-neighbour
+ * upsampling when `up` is nonzero (D, H, W even).
  */
 int sg_conv3d_wgrad(const void* x, const void* dy, float* dw, float* dbias, int B, int D, int H, int W, int Cin,
                     int Cout, void* stream);
+int sg_conv3d_wgrad_ex(const void* x, const void* dy, float* dw, float* dbias, int up, int B, int D, int H, int W,
+                       int Cin, int Cout, void* stream);
 
 /* sg_pool2 -- 2x2x2 average pooling, x [B][D][H][W][C] -> y [B][D/2][H/2][W/2][C] (even
  * D, H, W); sg_pool2_grad -- dx[child] = dy[parent] / 8. */
@@ -66,6 +84,13 @@ int sg_pool2_grad(const void* dy, void* dx, int B, int D, int H, int W, int C, v
  * sg_up2_grad -- dx[parent] = sum of dy over its 8 children. (D, H, W are the coarse sizes.) */
 int sg_up2(const void* x, void* y, int B, int D, int H, int W, int C, void* stream);
 int sg_up2_grad(const void* dy, void* dx, int B, int D, int H, int W, int C, void* stream);
+
+/* sg_up2_grad_relu -- sg_up2_grad, then 0 where act <= 0 (act [B][D][H][W][C], the coarse grid).
+ * sg_pool2_grad_relu -- dx = g + sg_pool2_grad(dy), then 0 where act <= 0 (g, act, dx on the fine
+ * grid; dx may alias g). Both: C a multiple of 8, 16-byte aligned buffers. */
+int sg_up2_grad_relu(const void* dy, const void* act, void* dx, int B, int D, int H, int W, int C, void* stream);
+int sg_pool2_grad_relu(const void* dy, const void* g, const void* act, void* dx, int B, int D, int H, int W, int C,
+                       void* stream);
 
 /* sg_add -- y = a + b (BF16, n values; y may alias a or b).
  * sg_relu_grad -- g[i] = 0 where act[i] <= 0 (in place; the post-activation output marks

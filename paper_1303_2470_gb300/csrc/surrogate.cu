@@ -39,7 +39,42 @@ struct ConvArgs {
     bf16* y;
     float* yf;
     int D, H, W, V, K, N, sign, relu;
+    // second BF16 output, from y = act(...) rounded to BF16 and `other` [B][V][N]: y + other
+    // (mode 1), or (kMask) y where other > 0, else 0
+    bf16* y2;
+    const bf16* other;
+    int mode;
+    int up;  // x is the coarse grid [B][D/2][H/2][W/2][K], read as its nearest upsampling
 };
+constexpr int kMask = 2;
+
+// voxel of the stored x that fine voxel (b, z, y, x) of a D x H x W box reads
+__device__ __forceinline__ int x_voxel(int up, int D, int H, int W, int b, int z, int y, int x)
+{
+    return up ? ((b * (D >> 1) + (z >> 1)) * (H >> 1) + (y >> 1)) * (W >> 1) + (x >> 1)
+              : ((b * D + z) * H + y) * W + x;
+}
+
+// eight BF16 values as FP32 and back
+__device__ __forceinline__ void unpack8(const uint4& v, float (&f)[8])
+{
+    const uint32_t w[4] = {v.x, v.y, v.z, v.w};
+#pragma unroll
+    for (int i = 0; i < 4; ++i) {
+        f[2 * i] = __uint_as_float(w[i] << 16);
+        f[2 * i + 1] = __uint_as_float(w[i] & 0xffff0000u);
+    }
+}
+__device__ __forceinline__ uint4 pack8(const float (&f)[8])
+{
+    uint32_t h[4];
+#pragma unroll
+    for (int i = 0; i < 4; ++i) {
+        const __nv_bfloat162 p2 = __floats2bfloat162_rn(f[2 * i], f[2 * i + 1]);
+        h[i] = *reinterpret_cast<const uint32_t*>(&p2);
+    }
+    return make_uint4(h[0], h[1], h[2], h[3]);
+}
 
 // ---------------------------------------------------------------------------------------
 // Forward (and transposed) convolution on the 5th-generation tensor cores: an implicit GEMM
@@ -150,8 +185,8 @@ __device__ __forceinline__ bool elect_one()
 }
 
 // Epilogue of the tensor-core convolutions: warp w reads accumulator rows 32w..32w+31 (its
-// lanes' voxels) from tensor memory, adds the bias, applies the ReLU and stores BF16 and/or
-// FP32 outputs of voxel e of the batch (skipped when negative), channels n0..n0+BN-1.
+// lanes' voxels) from tensor memory, adds the bias, applies the ReLU and stores BF16, FP32 and
+// second outputs of voxel e of the batch (skipped when negative), channels n0..n0+BN-1.
 __device__ __forceinline__ void conv_store_row(const ConvArgs& a, uint32_t tmem, int warp, long long e, int n0, int BN)
 {
     for (int c0 = 0; c0 < BN; c0 += 16) {
@@ -171,16 +206,32 @@ __device__ __forceinline__ void conv_store_row(const ConvArgs& a, uint32_t tmem,
                 float t = __uint_as_float(r[c]) + (a.bias ? a.bias[n0 + c0 + c] : 0.0f);
                 f[c] = a.relu ? fmaxf(t, 0.0f) : t;
             }
-            if (a.y) {
-                uint32_t h[8];
+            if (a.y || a.y2) {
+                uint4 h[2];
 #pragma unroll
-                for (int c = 0; c < 8; ++c) {
-                    const __nv_bfloat162 p2 = __floats2bfloat162_rn(f[2 * c], f[2 * c + 1]);
-                    h[c] = *reinterpret_cast<const uint32_t*>(&p2);
+                for (int k = 0; k < 2; ++k) {
+                    const float f8[8] = {f[8 * k],     f[8 * k + 1], f[8 * k + 2], f[8 * k + 3],
+                                         f[8 * k + 4], f[8 * k + 5], f[8 * k + 6], f[8 * k + 7]};
+                    h[k] = pack8(f8);
                 }
-                uint4* dst = reinterpret_cast<uint4*>(a.y + o);
-                dst[0] = make_uint4(h[0], h[1], h[2], h[3]);
-                dst[1] = make_uint4(h[4], h[5], h[6], h[7]);
+                if (a.y) {
+                    uint4* dst = reinterpret_cast<uint4*>(a.y + o);
+                    dst[0] = h[0];
+                    dst[1] = h[1];
+                }
+                if (a.y2) {
+                    const uint4* src = reinterpret_cast<const uint4*>(a.other + o);
+                    uint4* dst = reinterpret_cast<uint4*>(a.y2 + o);
+#pragma unroll
+                    for (int k = 0; k < 2; ++k) {
+                        float g8[8], o8[8];
+                        unpack8(h[k], g8);
+                        unpack8(__ldg(src + k), o8);
+#pragma unroll
+                        for (int c = 0; c < 8; ++c) g8[c] = a.mode == kMask ? (o8[c] > 0.0f ? g8[c] : 0.0f) : g8[c] + o8[c];
+                        dst[k] = pack8(g8);
+                    }
+                }
             }
             if (a.yf) {
                 float4* dst = reinterpret_cast<float4*>(a.yf + o);
@@ -223,8 +274,8 @@ __global__ void __launch_bounds__(kTThreads) k_conv_tc(const ConvArgs a)
         }
         for (int tap = 0; tap < 27; ++tap) {
             const int dz = tap / 9 - 1, dy = (tap / 3) % 3 - 1, dx = tap % 3 - 1;
-            s_src[tap][tid] = v < a.V ? (wrap(z + a.sign * dz, a.D) * a.H + wrap(y + a.sign * dy, a.H)) * a.W +
-                                            wrap(x + a.sign * dx, a.W)
+            s_src[tap][tid] = v < a.V ? x_voxel(a.up, a.D, a.H, a.W, 0, wrap(z + a.sign * dz, a.D),
+                                                wrap(y + a.sign * dy, a.H), wrap(x + a.sign * dx, a.W))
                                       : -1;
         }
     }
@@ -247,7 +298,7 @@ __global__ void __launch_bounds__(kTThreads) k_conv_tc(const ConvArgs a)
     __syncthreads();
     asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
     const uint32_t tmem = tmem_base;
-    const bf16* xb = a.x + (size_t)b * a.V * a.K;
+    const bf16* xb = a.x + (size_t)b * (a.up ? a.V / 8 : a.V) * a.K;
 
     // reduction elements of stage st (a multiple of 16), and the tap and channel of chunk j
     auto stage_kc = [&](int st) { return 27 * K - st * kTKC < kTKC ? 27 * K - st * kTKC : kTKC; };
@@ -493,7 +544,7 @@ __global__ void __launch_bounds__(kMThreads, 1) k_conv_march(const __grid_consta
                         const int xg = g % m.GX, r = g / m.GX;
                         const int z = r % m.c.D, b = r / m.c.D;
                         const int x = wrap(8 * xg - 1 + row % 10, W);
-                        off = ((b * m.c.D + wrap(z + sign * (d - 1), m.c.D)) * H) * W + x;
+                        off = x_voxel(m.c.up, m.c.D, H, W, b, wrap(z + sign * (d - 1), m.c.D), 0, x);
                     }
                     s_off[row] = off;
                 }
@@ -509,7 +560,7 @@ __global__ void __launch_bounds__(kMThreads, 1) k_conv_march(const __grid_consta
                     if (round > 0) ok = mbar_wait_or(smem_u32(&s_empty[slot]), (round - 1) & 1u, fail);
                     if (!ok) break;
                     const uint32_t dst = sA + (uint32_t)slot * kABytes;
-                    const bf16* xr = m.c.x + (size_t)ys * W * kK;
+                    const bf16* xr = m.c.x + (size_t)(m.c.up ? (ys >> 1) * (W >> 1) : ys * W) * kK;
 #pragma unroll
                     for (int i = 0; i < kP; ++i) {
                         const int p = pt + kMCopy * i, row = p / kKC, j = p - row * kKC;
@@ -711,6 +762,7 @@ struct WgradTcArgs {
     const bf16* dy;
     float* dw;
     int D, H, W, Cin, Cout;
+    int up;              // x is the coarse grid, read as its nearest upsampling
     int GX, NG;          // groups per x-row, groups over the batch
     int T, nstrip;       // x rows per unit, strips along y
     int nci, nco, units;
@@ -801,7 +853,7 @@ __global__ void __launch_bounds__(kGThreads, 1) k_wgrad_tc(const __grid_constant
                     const int xg = g % m.GX, l = g / m.GX;
                     const int z = l % m.D, b = l / m.D;
                     const int x = isx ? wrap(8 * xg - 1 + r % 10, W) : 8 * xg + r % 8;
-                    off = ((b * m.D + (isx ? wrap(z + d - 1, m.D) : z)) * H) * W + x;
+                    off = isx ? x_voxel(m.up, m.D, H, W, b, wrap(z + d - 1, m.D), 0, x) : ((b * m.D + z) * H) * W + x;
                 }
                 if (isx)
                     s_xoff[r] = off;
@@ -838,7 +890,7 @@ __global__ void __launch_bounds__(kGThreads, 1) k_wgrad_tc(const __grid_constant
                     load_y(y0);
                 }
                 load_y(wrap(y0 + i + 1, H));
-                const bf16* src = m.x + (size_t)(y0 + i) * W * m.Cin + ci0;
+                const bf16* src = m.x + (size_t)(m.up ? ((y0 + i) >> 1) * (W >> 1) : (y0 + i) * W) * m.Cin + ci0;
 #pragma unroll
                 for (int k = 0; k < kNX; ++k) {
                     const int p = pt + kMCopy * k, row = p / kPX, j = p - row * kPX;
@@ -962,6 +1014,7 @@ struct WgradArgs {
     long long total;  // B * V voxels of the reduction
     int chunk;        // voxels per block (a multiple of 32)
     int ci_tiles;     // tiles of 64 input channels
+    int up;           // x is the coarse grid, read as its nearest upsampling
 };
 
 // four 8x8 BF16 matrices from shared memory, transposed on the way (lanes 8j..8j+7 give the
@@ -1003,7 +1056,7 @@ __global__ void __launch_bounds__(kWThreads) k_wgrad(const WgradArgs a)
             const int v = (int)(ev - bb * a.V);
             const int xa = v % a.W, ya = (v / a.W) % a.H, za = v / (a.W * a.H);
             const int xs = wrap(xa + dx, a.W), ys = wrap(ya + dy, a.H), zs = wrap(za + dz, a.D);
-            const size_t src = (size_t)bb * a.V + (size_t)((zs * a.H + ys) * a.W + xs);
+            const size_t src = (size_t)bb * (a.up ? a.V / 8 : a.V) + (size_t)x_voxel(a.up, a.D, a.H, a.W, 0, zs, ys, xs);
             if (ci0 + lc < a.Cin) {
                 const bf16* p = a.x + src * a.Cin + ci0 + lc;
                 rx0 = *reinterpret_cast<const uint4*>(p);
@@ -1068,22 +1121,35 @@ __global__ void __launch_bounds__(kWThreads) k_wgrad(const WgradArgs a)
     }
 }
 
-// dbias[c] += sum over voxels of dy[.][c]: block = 256 voxels x one channel group of 32
-__global__ void k_bias_grad(const bf16* __restrict__ dy, float* __restrict__ db, long long total, int C)
+// dbias[c] += sum over voxels of dy[.][c]: a block sums kBiasRows voxels, a thread 8 channels
+// (16 bytes) of every (256 / (C / 8))-th of them; blockIdx.y: blocks of 2048 channels
+constexpr int kBiasRows = 1024, kBiasCh = 2048;
+__global__ void __launch_bounds__(256) k_bias_grad(const bf16* __restrict__ dy, float* __restrict__ db, long long total, int C)
 {
-    const int c = blockIdx.y * 32 + (threadIdx.x & 31);
-    const int r = threadIdx.x >> 5;  // 8 rows of voxels
-    float s = 0.0f;
-    if (c < C)
-        for (long long e = (long long)blockIdx.x * 256 + r; e < total && e < (long long)(blockIdx.x + 1) * 256; e += 8)
-            s += __bfloat162float(dy[(size_t)e * C + c]);
-    __shared__ float part[8][32];
-    part[r][threadIdx.x & 31] = s;
+    __shared__ float part[256][8];
+    const int c0 = blockIdx.y * kBiasCh, Cb = min(C - c0, kBiasCh);
+    const int C8 = Cb / 8, rows = 256 / C8;
+    const int j = threadIdx.x % C8, r = threadIdx.x / C8;
+    float s[8] = {0.f, 0.f, 0.f, 0.f, 0.f, 0.f, 0.f, 0.f};
+    if (r < rows) {
+        const long long e0 = (long long)blockIdx.x * kBiasRows;
+        const int n = (int)(total - e0 < kBiasRows ? total - e0 : kBiasRows);
+        const uint4* p = reinterpret_cast<const uint4*>(dy + (size_t)e0 * C + c0) + j;
+#pragma unroll 4
+        for (int e = r; e < n; e += rows) {
+            float f[8];
+            unpack8(__ldg(p + (size_t)e * (C / 8)), f);
+#pragma unroll
+            for (int c = 0; c < 8; ++c) s[c] += f[c];
+        }
+    }
+#pragma unroll
+    for (int c = 0; c < 8; ++c) part[threadIdx.x][c] = s[c];
     __syncthreads();
-    if (r == 0 && c < C) {
+    for (int c = threadIdx.x; c < Cb; c += 256) {
         float t = 0.0f;
-        for (int k = 0; k < 8; ++k) t += part[k][threadIdx.x];
-        atomicAdd(db + c, t);
+        for (int k = 0; k < rows; ++k) t += part[k * C8 + c / 8][c % 8];
+        atomicAdd(db + c0 + c, t);
     }
 }
 
@@ -1152,16 +1218,118 @@ __global__ void k_up2_grad(const bf16* __restrict__ dy, bf16* __restrict__ dx, i
     *reinterpret_cast<__nv_bfloat162*>(dx + (size_t)r * C + c) = __floats2bfloat162_rn(s0, s1);
 }
 
-__global__ void k_add(const bf16* __restrict__ a, const bf16* __restrict__ b, bf16* y, long long n)
+// The same passes with 16-byte accesses: a thread has one coarse voxel and 8 channels, reads or
+// writes its eight children. HBM-bound; with 4-byte accesses and 64-bit divisions per value they
+// ran at 8-40 % of the measured bandwidth (up2 of 64^3 x 64 channels 493 us).
+enum CoarseOp { kPool, kPoolGrad, kUp, kUpGrad, kPoolGradRelu, kUpGradRelu };
+
+// src: the fine grid for kPool, kUpGrad(Relu), else the coarse one. kPoolGradRelu: dst[child] =
+// (g[child] + src[parent] / 8) where act[child] > 0, else 0 (both BF16 roundings of the separate
+// passes); kUpGradRelu: dst[parent] = sum of the children where act[parent] > 0, else 0
+template <int kOp>
+__global__ void __launch_bounds__(256) k_coarse8(const bf16* __restrict__ src, const bf16* __restrict__ g,
+                                                 const bf16* __restrict__ act, bf16* __restrict__ dst, unsigned n,
+                                                 int D, int H, int W, int C8)
 {
-    const long long i = (long long)blockIdx.x * blockDim.x + threadIdx.x;
-    if (i < n) y[i] = __float2bfloat16_rn(__bfloat162float(a[i]) + __bfloat162float(b[i]));
+    // D, H, W: coarse sizes; n: coarse voxels of the batch x C8
+    const unsigned i = blockIdx.x * 256u + threadIdx.x;
+    if (i >= n) return;
+    const unsigned r = i / (unsigned)C8, c = i - r * (unsigned)C8;
+    const unsigned l = r / (unsigned)W, x = r - l * (unsigned)W;
+    const unsigned q = l / (unsigned)H, y = l - q * (unsigned)H;  // q = b D + z
+    const size_t f0 = (((size_t)(2 * q) * (2 * H) + 2 * y) * (2 * W) + 2 * x) * C8 + c;
+    auto child = [&](int k) {
+        return f0 + (((size_t)(k >> 2) * (2 * H) + (size_t)((k >> 1) & 1)) * (2 * W) + (size_t)(k & 1)) * C8;
+    };
+    const uint4* s = reinterpret_cast<const uint4*>(src);
+    uint4* d = reinterpret_cast<uint4*>(dst);
+    if constexpr (kOp == kPool || kOp == kUpGrad || kOp == kUpGradRelu) {
+        float t[8] = {0.f, 0.f, 0.f, 0.f, 0.f, 0.f, 0.f, 0.f};
+        uint4 v[8];
+#pragma unroll
+        for (int k = 0; k < 8; ++k) v[k] = __ldg(s + child(k));
+#pragma unroll
+        for (int k = 0; k < 8; ++k) {
+            float f[8];
+            unpack8(v[k], f);
+#pragma unroll
+            for (int e = 0; e < 8; ++e) t[e] += f[e];
+        }
+        if constexpr (kOp == kPool) {
+#pragma unroll
+            for (int e = 0; e < 8; ++e) t[e] *= 0.125f;
+        }
+        if constexpr (kOp == kUpGradRelu) {
+            float a[8];
+            unpack8(__ldg(reinterpret_cast<const uint4*>(act) + i), a);
+#pragma unroll
+            for (int e = 0; e < 8; ++e) t[e] = a[e] > 0.0f ? t[e] : 0.0f;
+        }
+        d[i] = pack8(t);
+    } else {
+        uint4 v = __ldg(s + i);
+        float p[8];
+        if constexpr (kOp == kPoolGrad || kOp == kPoolGradRelu) {
+            unpack8(v, p);
+#pragma unroll
+            for (int e = 0; e < 8; ++e) p[e] *= 0.125f;
+            v = pack8(p);
+            unpack8(v, p);  // rounded, as the separate pass stores it
+        }
+#pragma unroll
+        for (int k = 0; k < 8; ++k) {
+            const size_t o = child(k);
+            if constexpr (kOp == kPoolGradRelu) {
+                float gf[8], af[8];
+                unpack8(__ldg(reinterpret_cast<const uint4*>(g) + o), gf);
+                unpack8(__ldg(reinterpret_cast<const uint4*>(act) + o), af);
+#pragma unroll
+                for (int e = 0; e < 8; ++e) gf[e] = af[e] > 0.0f ? gf[e] + p[e] : 0.0f;
+                d[o] = pack8(gf);
+            } else {
+                d[o] = v;
+            }
+        }
+    }
 }
 
-__global__ void k_relu_grad(const bf16* __restrict__ act, bf16* __restrict__ g, long long n)
+bool aligned16(const void* a, const void* b = nullptr, const void* c = nullptr, const void* d = nullptr)
 {
-    const long long i = (long long)blockIdx.x * blockDim.x + threadIdx.x;
-    if (i < n && !(__bfloat162float(act[i]) > 0.0f)) g[i] = __float2bfloat16_rn(0.0f);
+    return (((uintptr_t)a | (uintptr_t)b | (uintptr_t)c | (uintptr_t)d) & 15) == 0;
+}
+
+// one pass of k_coarse8 where its 16-byte accesses and 32-bit index apply; false: use the
+// general kernels (D, H, W: coarse sizes)
+template <int kOp>
+bool coarse8(const void* src, const void* g, const void* act, void* dst, int B, int D, int H, int W, int C,
+             cudaStream_t s)
+{
+    const long long n = (long long)B * D * H * W * (C / 8);
+    if (C % 8 || n >= (1LL << 31) || !aligned16(src, g, act, dst)) return false;
+    k_coarse8<kOp><<<(unsigned)((n + 255) / 256), 256, 0, s>>>((const bf16*)src, (const bf16*)g, (const bf16*)act,
+                                                               (bf16*)dst, (unsigned)n, D, H, W, C / 8);
+    return true;
+}
+
+// y = a + b, or (kRelu) y[i] = b[i] where a[i] > 0, else 0 (y may alias either): eight values a
+// thread (16 bytes) where `vec`, the rest one by one
+template <bool kRelu>
+__global__ void __launch_bounds__(256) k_pair(const bf16* a, const bf16* b, bf16* y, long long n, int vec)
+{
+    const long long i = (long long)blockIdx.x * 256 + threadIdx.x;
+    const long long n8 = vec ? n / 8 : 0;
+    if (i < n8) {
+        float p[8], q[8];
+        unpack8(reinterpret_cast<const uint4*>(a)[i], p);
+        unpack8(reinterpret_cast<const uint4*>(b)[i], q);
+#pragma unroll
+        for (int e = 0; e < 8; ++e) q[e] = kRelu ? (p[e] > 0.0f ? q[e] : 0.0f) : p[e] + q[e];
+        reinterpret_cast<uint4*>(y)[i] = pack8(q);
+    } else if (i < n8 + (n - 8 * n8)) {
+        const long long e = 8 * n8 + (i - n8);
+        const float p = __bfloat162float(a[e]), q = __bfloat162float(b[e]);
+        y[e] = __float2bfloat16_rn(kRelu ? (p > 0.0f ? q : 0.0f) : p + q);
+    }
 }
 
 // network coordinates (p, q, r) of lattice node (x, y, z) for a force along `axis`: the
@@ -1259,26 +1427,52 @@ __global__ void k_pack_target(const float* __restrict__ u, const float* __restri
     t[(size_t)v * 4 + 3] = rho[n] > 0.0f ? scale_rho * (rho[n] - 1.0f) : 0.0f;
 }
 
-__global__ void k_mse(const float* __restrict__ y, int ldy, const float* __restrict__ t, int nc,
-                      const bf16* __restrict__ x, bf16* __restrict__ dy, double* __restrict__ loss, long long total,
-                      double inv)
+// A thread takes whole voxels (16-byte accesses where `vec`: ldy a multiple of 8, four channels of
+// targets, aligned); the block adds its FP64 sums before the one atomic addition
+__global__ void __launch_bounds__(256) k_mse(const float* __restrict__ y, int ldy, const float* __restrict__ t, int nc,
+                                             const bf16* __restrict__ x, bf16* __restrict__ dy,
+                                             double* __restrict__ loss, long long total, double inv, int vec)
 {
-    const long long e = (long long)blockIdx.x * blockDim.x + threadIdx.x;
     double s = 0.0;
-    if (e < total) {
+    const float scale = (float)(2.0 * inv);
+    for (long long e = (long long)blockIdx.x * 256 + threadIdx.x; e < total; e += (long long)gridDim.x * 256) {
         const bool fluid = __bfloat162float(x[(size_t)e * 16]) > 0.5f;
+        if (vec) {
+            float g[8] = {0.f, 0.f, 0.f, 0.f, 0.f, 0.f, 0.f, 0.f};
+            if (fluid) {
+                const float4 a = *reinterpret_cast<const float4*>(y + (size_t)e * ldy);
+                const float4 b = *reinterpret_cast<const float4*>(t + (size_t)e * 4);
+                const float d[4] = {a.x - b.x, a.y - b.y, a.z - b.z, a.w - b.w};
+#pragma unroll
+                for (int c = 0; c < 4; ++c) {
+                    s += (double)d[c] * d[c];
+                    g[c] = scale * d[c];
+                }
+            }
+            uint4* o = reinterpret_cast<uint4*>(dy + (size_t)e * ldy);
+            o[0] = pack8(g);
+            for (int c = 1; c < ldy / 8; ++c) o[c] = make_uint4(0u, 0u, 0u, 0u);
+            continue;
+        }
         for (int c = 0; c < ldy; ++c) {
             float gval = 0.0f;
             if (fluid && c < nc) {
                 const float d = y[(size_t)e * ldy + c] - t[(size_t)e * nc + c];
                 s += (double)d * d;
-                gval = (float)(2.0 * inv) * d;
+                gval = scale * d;
             }
             dy[(size_t)e * ldy + c] = __float2bfloat16_rn(gval);
         }
     }
+    __shared__ double part[8];
     for (int o = 16; o > 0; o >>= 1) s += __shfl_xor_sync(0xffffffffu, s, o);
-    if ((threadIdx.x & 31) == 0 && s != 0.0) atomicAdd(loss, s * inv);
+    if ((threadIdx.x & 31) == 0) part[threadIdx.x >> 5] = s;
+    __syncthreads();
+    if (threadIdx.x == 0) {
+        double b = 0.0;
+        for (int w = 0; w < 8; ++w) b += part[w];
+        if (b != 0.0) atomicAdd(loss, b * inv);
+    }
 }
 
 __global__ void k_adam(float* __restrict__ p, const float* __restrict__ g, float* __restrict__ m, float* __restrict__ v,
@@ -1424,6 +1618,7 @@ bool wgrad_plan(const WgradArgs& a, int B, int sms, WgradTcArgs* m, size_t* smem
     m->W = a.W;
     m->Cin = a.Cin;
     m->Cout = a.Cout;
+    m->up = a.up;
     m->GX = a.W / 8;
     m->NG = B * a.D * m->GX;
     m->nci = a.Cin / ci;
@@ -1464,16 +1659,11 @@ int grid1(long long n, int block) { return (int)((n + block - 1) / block); }
 
 extern "C" {
 
-int sg_conv3d(const void* x, const void* w, const float* bias, void* y, float* yf, int B, int D, int H, int W, int K,
-              int N, int sign, int relu, void* stream)
+static int conv3d(const void* x, const void* w, const float* bias, void* y, float* yf, void* y2, const void* other,
+                  int mode, int up, int B, int D, int H, int W, int K, int N, int sign, int relu, void* stream)
 {
-    clear_error();
-    if (!x || !w || (!y && !yf) || B < 1 || D < 1 || H < 1 || W < 1 || K < 16 || N < 16 || K % 16 || N % 16 ||
-        (sign != 1 && sign != -1) || (long long)D * H * W > (1LL << 30)) {
-        set_error("sg_conv3d: needs x, w, an output, B, D, H, W >= 1, K and N multiples of 16, sign +-1");
-        return MP_EINVAL;
-    }
-    ConvArgs a{(const bf16*)x, (const bf16*)w, bias, (bf16*)y, yf, D, H, W, D * H * W, K, N, sign, relu != 0};
+    ConvArgs a{(const bf16*)x, (const bf16*)w, bias, (bf16*)y, yf, D, H, W, D * H * W, K, N, sign, relu != 0,
+               (bf16*)y2, (const bf16*)other, mode, up != 0};
     const int bn = N < kTMaxN ? N : kTMaxN;
     int dev = 0, sms = 0;
     MP_CUDA(cudaGetDevice(&dev));
@@ -1509,6 +1699,36 @@ int sg_conv3d(const void* x, const void* w, const float* bias, void* y, float* y
     return MP_OK;
 }
 
+static bool conv_args_ok(const void* x, const void* w, int B, int D, int H, int W, int K, int N, int sign)
+{
+    return x && w && B >= 1 && D >= 1 && H >= 1 && W >= 1 && K >= 16 && N >= 16 && K % 16 == 0 && N % 16 == 0 &&
+           (sign == 1 || sign == -1) && (long long)D * H * W <= (1LL << 30);
+}
+
+int sg_conv3d(const void* x, const void* w, const float* bias, void* y, float* yf, int B, int D, int H, int W, int K,
+              int N, int sign, int relu, void* stream)
+{
+    clear_error();
+    if (!conv_args_ok(x, w, B, D, H, W, K, N, sign) || (!y && !yf)) {
+        set_error("sg_conv3d: needs x, w, an output, B, D, H, W >= 1, K and N multiples of 16, sign +-1");
+        return MP_EINVAL;
+    }
+    return conv3d(x, w, bias, y, yf, nullptr, nullptr, 0, 0, B, D, H, W, K, N, sign, relu, stream);
+}
+
+int sg_conv3d_ex(const void* x, const void* w, const float* bias, void* y, float* yf, void* y2, const void* other,
+                 int mode, int up, int B, int D, int H, int W, int K, int N, int sign, int relu, void* stream)
+{
+    clear_error();
+    if (!conv_args_ok(x, w, B, D, H, W, K, N, sign) || (!y && !yf && !y2) || mode < 0 || mode > 2 ||
+        ((mode != 0) != (y2 != nullptr)) || ((mode != 0) != (other != nullptr)) || (up && (D % 2 || H % 2 || W % 2))) {
+        set_error("sg_conv3d_ex: needs what sg_conv3d needs, y2 and other exactly with mode 1 or 2, and even D, H, W "
+                  "with up");
+        return MP_EINVAL;
+    }
+    return conv3d(x, w, bias, y, yf, y2, other, mode, up, B, D, H, W, K, N, sign, relu, stream);
+}
+
 int sg_check(void* stream)
 {
     clear_error();
@@ -1528,14 +1748,21 @@ int sg_check(void* stream)
 int sg_conv3d_wgrad(const void* x, const void* dy, float* dw, float* dbias, int B, int D, int H, int W, int Cin,
                     int Cout, void* stream)
 {
+    return sg_conv3d_wgrad_ex(x, dy, dw, dbias, 0, B, D, H, W, Cin, Cout, stream);
+}
+
+int sg_conv3d_wgrad_ex(const void* x, const void* dy, float* dw, float* dbias, int up, int B, int D, int H, int W,
+                       int Cin, int Cout, void* stream)
+{
     clear_error();
-    if (!x || !dy || !dw || B < 1 || D < 1 || H < 1 || W < 1 || Cin < 16 || Cout < 16 || Cin % 16 || Cout % 16) {
-        set_error("sg_conv3d_wgrad: needs x, dy, dw, positive sizes, Cin and Cout multiples of 16");
+    if (!x || !dy || !dw || B < 1 || D < 1 || H < 1 || W < 1 || Cin < 16 || Cout < 16 || Cin % 16 || Cout % 16 ||
+        (up && (D % 2 || H % 2 || W % 2))) {
+        set_error("sg_conv3d_wgrad: needs x, dy, dw, positive sizes (even with up), Cin and Cout multiples of 16");
         return MP_EINVAL;
     }
     const int ci_tiles = (Cin + kWM - 1) / kWM, co_tiles = (Cout + kWN - 1) / kWN;
     WgradArgs a{(const bf16*)x, (const bf16*)dy, dw, D, H, W, D * H * W, Cin, Cout, (long long)B * D * H * W, 2048,
-                ci_tiles};
+                ci_tiles, up != 0};
     cudaStream_t cs = (cudaStream_t)stream;
     const long long nchunk = (a.total + a.chunk - 1) / a.chunk;
     int dev = 0, sms = 0;
@@ -1559,8 +1786,7 @@ int sg_conv3d_wgrad(const void* x, const void* dy, float* dw, float* dbias, int 
     }
     MP_CUDA(cudaGetLastError());
     if (dbias) {
-        dim3 gb(grid1(a.total, 256), (Cout + 31) / 32);
-        k_bias_grad<<<gb, 256, 0, cs>>>((const bf16*)dy, dbias, a.total, Cout);
+        k_bias_grad<<<dim3(grid1(a.total, kBiasRows), (Cout + kBiasCh - 1) / kBiasCh), 256, 0, cs>>>((const bf16*)dy, dbias, a.total, Cout);
         MP_CUDA(cudaGetLastError());
     }
     return MP_OK;
@@ -1572,6 +1798,10 @@ int sg_pool2(const void* x, void* y, int B, int D, int H, int W, int C, void* st
     if (!x || !y || B < 1 || D < 2 || H < 2 || W < 2 || (D | H | W) & 1 || C < 2 || C & 1) {
         set_error("sg_pool2: needs even D, H, W and an even channel count");
         return MP_EINVAL;
+    }
+    if (coarse8<kPool>(x, nullptr, nullptr, y, B, D / 2, H / 2, W / 2, C, (cudaStream_t)stream)) {
+        MP_CUDA(cudaGetLastError());
+        return MP_OK;
     }
     const long long n = (long long)B * (D / 2) * (H / 2) * (W / 2) * (C / 2);
     k_pool2<<<grid1(n, 256), 256, 0, (cudaStream_t)stream>>>((const bf16*)x, (bf16*)y, B, D, H, W, C);
@@ -1585,6 +1815,10 @@ int sg_pool2_grad(const void* dy, void* dx, int B, int D, int H, int W, int C, v
     if (!dy || !dx || B < 1 || D < 2 || H < 2 || W < 2 || (D | H | W) & 1 || C < 2 || C & 1) {
         set_error("sg_pool2_grad: needs even D, H, W and an even channel count");
         return MP_EINVAL;
+    }
+    if (coarse8<kPoolGrad>(dy, nullptr, nullptr, dx, B, D / 2, H / 2, W / 2, C, (cudaStream_t)stream)) {
+        MP_CUDA(cudaGetLastError());
+        return MP_OK;
     }
     const long long n = (long long)B * D * H * W * (C / 2);
     k_fine_from_coarse<true><<<grid1(n, 256), 256, 0, (cudaStream_t)stream>>>((const bf16*)dy, (bf16*)dx, B, D / 2,
@@ -1600,6 +1834,10 @@ int sg_up2(const void* x, void* y, int B, int D, int H, int W, int C, void* stre
         set_error("sg_up2: needs positive sizes and an even channel count");
         return MP_EINVAL;
     }
+    if (coarse8<kUp>(x, nullptr, nullptr, y, B, D, H, W, C, (cudaStream_t)stream)) {
+        MP_CUDA(cudaGetLastError());
+        return MP_OK;
+    }
     const long long n = (long long)B * 8 * D * H * W * (C / 2);
     k_fine_from_coarse<false><<<grid1(n, 256), 256, 0, (cudaStream_t)stream>>>((const bf16*)x, (bf16*)y, B, D, H, W,
                                                                                 C);
@@ -1614,8 +1852,43 @@ int sg_up2_grad(const void* dy, void* dx, int B, int D, int H, int W, int C, voi
         set_error("sg_up2_grad: needs positive sizes and an even channel count");
         return MP_EINVAL;
     }
+    if (coarse8<kUpGrad>(dy, nullptr, nullptr, dx, B, D, H, W, C, (cudaStream_t)stream)) {
+        MP_CUDA(cudaGetLastError());
+        return MP_OK;
+    }
     const long long n = (long long)B * D * H * W * (C / 2);
     k_up2_grad<<<grid1(n, 256), 256, 0, (cudaStream_t)stream>>>((const bf16*)dy, (bf16*)dx, B, D, H, W, C);
+    MP_CUDA(cudaGetLastError());
+    return MP_OK;
+}
+
+int sg_up2_grad_relu(const void* dy, const void* act, void* dx, int B, int D, int H, int W, int C, void* stream)
+{
+    clear_error();
+    if (!dy || !act || !dx || B < 1 || D < 1 || H < 1 || W < 1 || C < 8 || C % 8) {
+        set_error("sg_up2_grad_relu: needs positive sizes and a channel count that is a multiple of 8");
+        return MP_EINVAL;
+    }
+    if (!coarse8<kUpGradRelu>(dy, nullptr, act, dx, B, D, H, W, C, (cudaStream_t)stream)) {
+        set_error("sg_up2_grad_relu: buffers must be 16-byte aligned, with less than 2^34 values");
+        return MP_EINVAL;
+    }
+    MP_CUDA(cudaGetLastError());
+    return MP_OK;
+}
+
+int sg_pool2_grad_relu(const void* dy, const void* g, const void* act, void* dx, int B, int D, int H, int W, int C,
+                       void* stream)
+{
+    clear_error();
+    if (!dy || !g || !act || !dx || B < 1 || D < 2 || H < 2 || W < 2 || (D | H | W) & 1 || C < 8 || C % 8) {
+        set_error("sg_pool2_grad_relu: needs even D, H, W and a channel count that is a multiple of 8");
+        return MP_EINVAL;
+    }
+    if (!coarse8<kPoolGradRelu>(dy, g, act, dx, B, D / 2, H / 2, W / 2, C, (cudaStream_t)stream)) {
+        set_error("sg_pool2_grad_relu: buffers must be 16-byte aligned, with less than 2^34 values");
+        return MP_EINVAL;
+    }
     MP_CUDA(cudaGetLastError());
     return MP_OK;
 }
@@ -1628,7 +1901,9 @@ int sg_add(const void* a, const void* b, void* y, int64_t n, void* stream)
         return MP_EINVAL;
     }
     if (n == 0) return MP_OK;
-    k_add<<<grid1(n, 256), 256, 0, (cudaStream_t)stream>>>((const bf16*)a, (const bf16*)b, (bf16*)y, n);
+    const int vec = aligned16(a, b, y);
+    k_pair<false><<<grid1(vec ? n / 8 + n % 8 : n, 256), 256, 0, (cudaStream_t)stream>>>((const bf16*)a, (const bf16*)b,
+                                                                                         (bf16*)y, n, vec);
     MP_CUDA(cudaGetLastError());
     return MP_OK;
 }
@@ -1641,7 +1916,9 @@ int sg_relu_grad(const void* act, void* g, int64_t n, void* stream)
         return MP_EINVAL;
     }
     if (n == 0) return MP_OK;
-    k_relu_grad<<<grid1(n, 256), 256, 0, (cudaStream_t)stream>>>((const bf16*)act, (bf16*)g, n);
+    const int vec = aligned16(act, g);
+    k_pair<true><<<grid1(vec ? n / 8 + n % 8 : n, 256), 256, 0, (cudaStream_t)stream>>>(
+        (const bf16*)act, (const bf16*)g, (bf16*)g, n, vec);
     MP_CUDA(cudaGetLastError());
     return MP_OK;
 }
@@ -1712,8 +1989,10 @@ int sg_mse(const float* y, int ldy, const float* t, int nc, const void* x, void*
         return MP_EINVAL;
     }
     const long long total = (long long)B * V;
-    k_mse<<<grid1(total, 256), 256, 0, (cudaStream_t)stream>>>(y, ldy, t, nc, (const bf16*)x, (bf16*)dy, loss, total,
-                                                                1.0 / (nc * n_fluid));
+    const int vec = ldy % 8 == 0 && nc == 4 && aligned16(y, t, dy);
+    const int blocks = (int)std::min<long long>((total + 255) / 256, 152 * 16);
+    k_mse<<<blocks, 256, 0, (cudaStream_t)stream>>>(y, ldy, t, nc, (const bf16*)x, (bf16*)dy, loss, total,
+                                                    1.0 / (nc * n_fluid), vec);
     MP_CUDA(cudaGetLastError());
     return MP_OK;
 }

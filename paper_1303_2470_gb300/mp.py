@@ -99,6 +99,10 @@ _lib.mp_group_variant.restype = ctypes.c_char_p
 _lib.mp_grid_wait_selftest.argtypes = [_c_int, _c_int, _c_int, _c_i64, _c_vp]
 _f32, _c_i, _vp = ctypes.c_float, _c_int, _c_vp
 _lib.sg_conv3d.argtypes = [_vp, _vp, _vp, _vp, _vp] + [_c_i] * 8 + [_vp]
+_lib.sg_conv3d_ex.argtypes = [_vp] * 7 + [_c_i] * 10 + [_vp]
+_lib.sg_conv3d_wgrad_ex.argtypes = [_vp, _vp, _vp, _vp] + [_c_i] * 7 + [_vp]
+_lib.sg_up2_grad_relu.argtypes = [_vp] * 3 + [_c_i] * 5 + [_vp]
+_lib.sg_pool2_grad_relu.argtypes = [_vp] * 4 + [_c_i] * 5 + [_vp]
 _lib.sg_conv3d_wgrad.argtypes = [_vp, _vp, _vp, _vp] + [_c_i] * 6 + [_vp]
 _lib.sg_check.argtypes = [_vp]
 for _f in ("sg_pool2", "sg_pool2_grad", "sg_up2", "sg_up2_grad"):
@@ -113,7 +117,8 @@ _lib.sg_adam.argtypes = [_vp, _vp, _vp, _vp, _c_i64, _f32, _f32, _f32, _f32, _c_
 for _f in ("mp_init", "mp_init_batch", "mp_step", "mp_vacf", "mp_mass", "mp_info", "mp_get_field",
            "mp_set_field", "lb_steady", "mp_classify", "mp_step_noalloc", "mp_group_create", "mp_group_create_ex",
            "mp_grid_wait_selftest",
-           "mp_group_step", "mp_group_block_size", "sg_conv3d", "sg_conv3d_wgrad", "sg_check", "sg_pool2",
+           "mp_group_step", "mp_group_block_size", "sg_conv3d", "sg_conv3d_wgrad", "sg_conv3d_ex",
+           "sg_conv3d_wgrad_ex", "sg_up2_grad_relu", "sg_pool2_grad_relu", "sg_check", "sg_pool2",
            "sg_pool2_grad", "sg_up2", "sg_up2_grad", "sg_add", "sg_relu_grad", "sg_pack_input",
            "sg_unpack_output", "sg_pack_target", "sg_mse", "sg_adam"):
     getattr(_lib, _f).restype = _c_int
@@ -464,6 +469,11 @@ def sg_conv3d(x, w, bias, y, yf, B, D, H, W, K, N, sign=1, relu=False, stream=No
                           int(bool(relu)), _stream(stream)))
 
 
+def sg_conv3d_ex(x, w, bias, y, yf, y2, other, mode, up, B, D, H, W, K, N, sign=1, relu=False, stream=None):
+    _check(_lib.sg_conv3d_ex(_addr(x), _addr(w), _addr(bias), _addr(y), _addr(yf), _addr(y2), _addr(other), mode,
+                             int(bool(up)), B, D, H, W, K, N, sign, int(bool(relu)), _stream(stream)))
+
+
 def sg_check(stream=None):
     """sg_check of include/surrogate.h: raises MPError (MP_ETIMEOUT) if a tensor-core
     convolution since the last check gave up a bounded wait."""
@@ -473,6 +483,19 @@ def sg_check(stream=None):
 def sg_conv3d_wgrad(x, dy, dw, dbias, B, D, H, W, Cin, Cout, stream=None):
     _check(_lib.sg_conv3d_wgrad(_addr(x), _addr(dy), _addr(dw), _addr(dbias), B, D, H, W, Cin, Cout,
                                 _stream(stream)))
+
+
+def sg_conv3d_wgrad_ex(x, dy, dw, dbias, up, B, D, H, W, Cin, Cout, stream=None):
+    _check(_lib.sg_conv3d_wgrad_ex(_addr(x), _addr(dy), _addr(dw), _addr(dbias), int(bool(up)), B, D, H, W, Cin, Cout,
+                                   _stream(stream)))
+
+
+def sg_up2_grad_relu(dy, act, dx, B, D, H, W, C, stream=None):
+    _check(_lib.sg_up2_grad_relu(_addr(dy), _addr(act), _addr(dx), B, D, H, W, C, _stream(stream)))
+
+
+def sg_pool2_grad_relu(dy, g, act, dx, B, D, H, W, C, stream=None):
+    _check(_lib.sg_pool2_grad_relu(_addr(dy), _addr(g), _addr(act), _addr(dx), B, D, H, W, C, _stream(stream)))
 
 
 def sg_pool2(x, y, B, D, H, W, C, stream=None):

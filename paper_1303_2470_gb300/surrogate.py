@@ -105,18 +105,26 @@ class Surrogate:
         return sum(t["W"].numel() + t["b"].numel() for t in self.p.values())
 
     # ---------------------------------------------------------------------------------
-    def _conv(self, name, x, B, dims, out_f32=False):
+    def _conv(self, name, x, B, dims, out_f32=False, skip=None, up=False, keep=True):
+        """Convolution layer `name` at output size dims; up: x is the coarse grid, read as its
+        nearest upsampling. With `skip` returns (output, output + skip), the output itself only
+        when `keep`."""
         torch = _torch()
         t = self.p[name]
         D, H, W = dims
         relu = dict((l[0], l[3]) for l in LAYERS)[name]
+
+        def new(dtype):
+            return torch.empty((B, D * H * W, t["cout"]), dtype=dtype, device=x.device)
         if out_f32:
-            y = torch.empty((B, D * H * W, t["cout"]), dtype=torch.float32, device=x.device)
+            y = new(torch.float32)
             self.mp.sg_conv3d(x, t["Wf"], t["b"], None, y, B, D, H, W, t["cin"], t["cout"], 1, relu)
-        else:
-            y = torch.empty((B, D * H * W, t["cout"]), dtype=torch.bfloat16, device=x.device)
-            self.mp.sg_conv3d(x, t["Wf"], t["b"], y, None, B, D, H, W, t["cin"], t["cout"], 1, relu)
-        return y
+            return y
+        y = new(torch.bfloat16) if keep or skip is None else None
+        h = new(torch.bfloat16) if skip is not None else None
+        self.mp.sg_conv3d_ex(x, t["Wf"], t["b"], y, None, h, skip, 0 if skip is None else 1, up, B, D, H, W, t["cin"],
+                             t["cout"], 1, relu)
+        return y if skip is None else (y, h)
 
     def forward(self, x0, B, dims, keep=False):
         """x0 BF16 [B][V][16]; dims = (D, H, W) of the network box (multiples of 8).
@@ -147,38 +155,34 @@ class Surrogate:
         mp.sg_pool2(a["s2"], a["p2"], B, *l2, 96)
         a["a3"] = self._conv("b0", a["p2"], B, l3)
         a["c3"] = self._conv("b1", a["a3"], B, l3)
-        a["u2"] = new(l2, 128)
-        mp.sg_up2(a["c3"], a["u2"], B, *l3, 128)
-        a["d2"] = self._conv("d2a", a["u2"], B, l2)
-        a["h2"] = new(l2, 96)
-        mp.sg_add(a["d2"], a["s2"], a["h2"], a["h2"].numel())
+        # the decoder's first layer of a level reads the coarser level upsampled and adds the skip
+        a["d2"], a["h2"] = self._conv("d2a", a["c3"], B, l2, skip=a["s2"], up=True, keep=keep)
         a["e2"] = self._conv("d2b", a["h2"], B, l2)
-        a["u1"] = new(l1, 96)
-        mp.sg_up2(a["e2"], a["u1"], B, *l2, 96)
-        a["d1"] = self._conv("d1a", a["u1"], B, l1)
-        a["h1"] = new(l1, 64)
-        mp.sg_add(a["d1"], a["s1"], a["h1"], a["h1"].numel())
+        a["d1"], a["h1"] = self._conv("d1a", a["e2"], B, l1, skip=a["s1"], up=True, keep=keep)
         a["e1"] = self._conv("d1b", a["h1"], B, l1)
-        a["u0"] = new(l0, 64)
-        mp.sg_up2(a["e1"], a["u0"], B, *l1, 64)
-        a["d0"] = self._conv("d0a", a["u0"], B, l0)
-        a["h0"] = new(l0, 32)
-        mp.sg_add(a["d0"], a["s0"], a["h0"], a["h0"].numel())
+        a["d0"], a["h0"] = self._conv("d0a", a["e1"], B, l0, skip=a["s0"], up=True, keep=keep)
         a["e0"] = self._conv("d0b", a["h0"], B, l0)
         y = self._conv("out", a["e0"], B, l0, out_f32=True)
         return y, (a if keep else None)
 
-    def _back(self, name, x, g, B, dims, need_input_grad=True):
-        """Accumulate the weight and bias gradients of layer `name` (input x, output gradient
-        g already masked by its ReLU) and return the input gradient."""
+    def _back(self, name, x, g, B, dims, up=False, mask=None, plain=True):
+        """Accumulate the weight and bias gradients of layer `name` (input x, read upsampled
+        with `up`; output gradient g already masked by its ReLU). Returns the gradient of the
+        input (of the upsampled one with `up`): as it is (plain), zeroed where mask <= 0 (mask),
+        or both as a pair; None with neither."""
         torch = _torch()
         t = self.p[name]
-        self.mp.sg_conv3d_wgrad(x, g, t["gW"], t["gb"], B, *dims, t["cin"], t["cout"])
-        if not need_input_grad:
+        self.mp.sg_conv3d_wgrad_ex(x, g, t["gW"], t["gb"], up, B, *dims, t["cin"], t["cout"])
+        if not plain and mask is None:
             return None
-        gx = torch.empty((B, x.shape[1], t["cin"]), dtype=torch.bfloat16, device=x.device)
-        self.mp.sg_conv3d(g, t["Wb"], None, gx, None, B, *dims, t["cout"], t["cin"], -1, False)
-        return gx
+
+        def new():
+            return torch.empty((B, g.shape[1], t["cin"]), dtype=torch.bfloat16, device=g.device)
+        gx = new() if plain else None
+        gm = new() if mask is not None else None
+        self.mp.sg_conv3d_ex(g, t["Wb"], None, gx, None, gm, mask, 0 if mask is None else 2, False, B, *dims,
+                             t["cout"], t["cin"], -1, False)
+        return (gx, gm) if plain and mask is not None else (gx if plain else gm)
 
     def backward(self, a, gy, B, dims):
         """gy BF16 [B][V][16] (from sg_mse); accumulates every layer's gradients."""
@@ -187,36 +191,26 @@ class Surrogate:
         D, H, W = dims
         l0, l1, l2, l3 = (D, H, W), (D // 2, H // 2, W // 2), (D // 4, H // 4, W // 4), (D // 8, H // 8, W // 8)
 
-        def relu_g(act, g):
-            mp.sg_relu_grad(act, g, g.numel())
-            return g
-
         def up_g(g, act, C, coarse):
-            out = torch.empty((B, act.shape[1], C), dtype=torch.bfloat16, device=gy.device)
-            mp.sg_up2_grad(g, out, B, *coarse, C)
+            out = torch.empty_like(act)
+            mp.sg_up2_grad_relu(g, act, out, B, *coarse, C)
             return out
 
-        g = self._back("out", a["e0"], gy, B, l0)
-        g = self._back("d0b", a["h0"], relu_g(a["e0"], g), B, l0)
-        g_s0 = g.clone()
-        g = self._back("d0a", a["u0"], relu_g(a["d0"], g), B, l0)
-        g = self._back("d1b", a["h1"], relu_g(a["e1"], up_g(g, a["e1"], 64, l1)), B, l1)
-        g_s1 = g.clone()
-        g = self._back("d1a", a["u1"], relu_g(a["d1"], g), B, l1)
-        g = self._back("d2b", a["h2"], relu_g(a["e2"], up_g(g, a["e2"], 96, l2)), B, l2)
-        g_s2 = g.clone()
-        g = self._back("d2a", a["u2"], relu_g(a["d2"], g), B, l2)
-        g = self._back("b1", a["a3"], relu_g(a["c3"], up_g(g, a["c3"], 128, l3)), B, l3)
-        g = self._back("b0", a["p2"], relu_g(a["a3"], g), B, l3)
-        for lvl, gs, act_s, pin, C, fine in ((2, g_s2, "s2", "a2", 96, l2), (1, g_s1, "s1", "a1", 64, l1),
-                                             (0, g_s0, "s0", "a0", 32, l0)):
-            gp = torch.empty_like(gs)
-            mp.sg_pool2_grad(g, gp, B, *fine, C)
-            mp.sg_add(gs, gp, gs, gs.numel())
-            names = {2: ("e2b", "e2a"), 1: ("e1b", "e1a"), 0: ("e0b", "e0a")}[lvl]
-            below = {2: "p1", 1: "p0", 0: "x0"}[lvl]
-            g = self._back(names[0], a[pin], relu_g(a[act_s], gs), B, fine)
-            g = self._back(names[1], a[below], relu_g(a[pin], g), B, fine, need_input_grad=lvl > 0)
+        g = self._back("out", a["e0"], gy, B, l0, mask=a["e0"], plain=False)
+        g_s0, g = self._back("d0b", a["h0"], g, B, l0, mask=a["d0"])
+        g = up_g(self._back("d0a", a["e1"], g, B, l0, up=True), a["e1"], 64, l1)
+        g_s1, g = self._back("d1b", a["h1"], g, B, l1, mask=a["d1"])
+        g = up_g(self._back("d1a", a["e2"], g, B, l1, up=True), a["e2"], 96, l2)
+        g_s2, g = self._back("d2b", a["h2"], g, B, l2, mask=a["d2"])
+        g = up_g(self._back("d2a", a["c3"], g, B, l2, up=True), a["c3"], 128, l3)
+        g = self._back("b1", a["a3"], g, B, l3, mask=a["a3"], plain=False)
+        g = self._back("b0", a["p2"], g, B, l3)
+        for gs, act_s, (fine, coarse), pin, below, C, lvl in (
+                (g_s2, "s2", ("e2b", "e2a"), "a2", "p1", 96, l2), (g_s1, "s1", ("e1b", "e1a"), "a1", "p0", 64, l1),
+                (g_s0, "s0", ("e0b", "e0a"), "a0", "x0", 32, l0)):
+            mp.sg_pool2_grad_relu(g, gs, a[act_s], gs, B, *lvl, C)
+            g = self._back(fine, a[pin], gs, B, lvl, mask=a[pin], plain=False)
+            g = self._back(coarse, a[below], g, B, lvl, plain=below != "x0")
 
     def zero_grad(self):
         for t in self.p.values():
