@@ -282,6 +282,20 @@ int mp_classify(const mp_geometry* g, uint8_t* cls, int64_t* n_fluid, int64_t* n
                 int64_t* n_cluster, void* stream);
 
 /*
+ * mp_classify_device -- mp_classify with cls in device memory (N bytes), written on `stream`;
+ * asking for n_cluster synchronises the stream. Same errors.
+ */
+int mp_classify_device(const mp_geometry* g, uint8_t* cls, int64_t* n_fluid, int64_t* n_interface,
+                       int64_t* n_cluster, void* stream);
+
+/*
+ * mp_release_cached -- gives back the device memory (at most 256 MiB per device) that the
+ * library keeps mapped between calls for the scratch of mp_classify and lb_steady. Synchronises
+ * the current device. It never fails; the next call maps memory again.
+ */
+void mp_release_cached(void);
+
+/*
  * mp_step_noalloc -- one moment-propagation + sorption step of one propagated field of one
  * species, on caller-owned dense device arrays, that allocates no memory of any kind (no
  * cudaMalloc, no cudaFree, no allocating library routine). It serves callers that cannot

@@ -117,8 +117,17 @@ int build_geometry(const mp_geometry* g, cudaStream_t stream, bool stream_ordere
                    bool want_list, Geometry* out);
 void free_geometry(Geometry* g, cudaStream_t stream, bool stream_ordered);
 
-// Largest connected cluster of fluid nodes (D3Q19 links, periodic) into g->cluster and
-// g->n_cluster; ties go to the cluster holding the smallest node index. Synchronises.
-int build_cluster(Geometry* g, cudaStream_t stream, bool stream_ordered);
+// Largest connected cluster of fluid nodes (D3Q19 links, periodic) into g->cluster; ties go to
+// the cluster holding the smallest node index. With `want_count` also g->n_cluster, which
+// synchronises.
+int build_cluster(Geometry* g, cudaStream_t stream, bool stream_ordered, bool want_count);
+
+// Stream-ordered device scratch from the library's pool (freed with cudaFreeAsync); pool_trim
+// gives the memory that the pool keeps between calls back to the system.
+cudaError_t pool_malloc(void** p, size_t bytes, cudaStream_t stream);
+void pool_trim();
+
+// unique id of the calling thread's current context; 0 if none or not available
+unsigned long long current_ctx_id();
 
 }  // namespace mp

@@ -226,7 +226,7 @@ extern "C" int lb_steady(const mp_geometry* geom, const double force[3], double 
     if (rc != MP_OK) return rc;
     // the body force acts on the largest connected fluid cluster: in a sealed pocket a
     // uniform force is balanced by pressure and the steady velocity is zero
-    rc = build_cluster(&G, s, true);
+    rc = build_cluster(&G, s, true, false);
     if (rc != MP_OK) {
         free_geometry(&G, s, true);
         cudaStreamSynchronize(s);
@@ -238,12 +238,12 @@ extern "C" int lb_steady(const mp_geometry* geom, const double force[3], double 
     uint32_t* omask = nullptr;
     uint2* fw = nullptr;
     unsigned long long* res_d = nullptr;
-    cudaError_t e = cudaMallocAsync((void**)&g0, sizeof(float) * kQ * NF, s);
-    if (e == cudaSuccess) e = cudaMallocAsync((void**)&omask, sizeof(uint32_t) * NF, s);
-    if (e == cudaSuccess) e = cudaMallocAsync((void**)&fw, sizeof(uint2) * (size_t)(G.W > 0 ? G.W : 1), s);
-    if (e == cudaSuccess) e = cudaMallocAsync((void**)&g1, sizeof(float) * kQ * NF, s);
-    if (e == cudaSuccess) e = cudaMallocAsync((void**)&uprev, sizeof(float) * 3 * NF, s);
-    if (e == cudaSuccess) e = cudaMallocAsync((void**)&res_d, sizeof(unsigned long long), s);
+    cudaError_t e = pool_malloc((void**)&g0, sizeof(float) * kQ * NF, s);
+    if (e == cudaSuccess) e = pool_malloc((void**)&omask, sizeof(uint32_t) * NF, s);
+    if (e == cudaSuccess) e = pool_malloc((void**)&fw, sizeof(uint2) * (size_t)(G.W > 0 ? G.W : 1), s);
+    if (e == cudaSuccess) e = pool_malloc((void**)&g1, sizeof(float) * kQ * NF, s);
+    if (e == cudaSuccess) e = pool_malloc((void**)&uprev, sizeof(float) * 3 * NF, s);
+    if (e == cudaSuccess) e = pool_malloc((void**)&res_d, sizeof(unsigned long long), s);
     // solid entries of the dense outputs stay zero; fluid entries are written at every check
     if (e == cudaSuccess) e = cudaMemsetAsync(u_out, 0, sizeof(float) * 3 * N, s);
     if (e == cudaSuccess && rho_out) e = cudaMemsetAsync(rho_out, 0, sizeof(float) * N, s);

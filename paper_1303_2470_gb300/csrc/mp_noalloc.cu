@@ -135,41 +135,13 @@ __global__ void __launch_bounds__(kNaThreads)
 // stand-in, so the address is looked up with cudaGetSymbolAddress (with the device current)
 // and remembered per device together with the unique id of the context it belongs to. A
 // cudaDeviceReset ends that context and the next call runs in a new one, whose module copy
-// of the array lives elsewhere: a changed context id triggers a fresh lookup. The driver's
-// context queries are resolved through the runtime, so the library needs no link to libcuda.
-typedef int (*CtxGetCurrentFn)(void**);
-typedef int (*CtxGetIdFn)(void*, unsigned long long*);
-
+// of the array lives elsewhere: a changed context id triggers a fresh lookup.
 std::mutex g_scratch_mu;
 struct ScratchSlot {
     unsigned char* ptr = nullptr;
     unsigned long long ctx_id = 0;
 };
 ScratchSlot g_scratch[128];
-CtxGetCurrentFn g_ctx_current = nullptr;
-CtxGetIdFn g_ctx_id = nullptr;
-bool g_ctx_fns_tried = false;
-
-// unique id of the calling thread's current context; 0 if none or not available
-unsigned long long current_ctx_id()
-{
-    if (!g_ctx_fns_tried) {
-        g_ctx_fns_tried = true;
-        void* f = nullptr;
-        cudaDriverEntryPointQueryResult q;
-        if (cudaGetDriverEntryPointByVersion("cuCtxGetCurrent", &f, 12000, cudaEnableDefault, &q) == cudaSuccess &&
-            q == cudaDriverEntryPointSuccess)
-            g_ctx_current = reinterpret_cast<CtxGetCurrentFn>(f);
-        f = nullptr;
-        if (cudaGetDriverEntryPointByVersion("cuCtxGetId", &f, 12000, cudaEnableDefault, &q) == cudaSuccess &&
-            q == cudaDriverEntryPointSuccess)
-            g_ctx_id = reinterpret_cast<CtxGetIdFn>(f);
-    }
-    void* ctx = nullptr;
-    unsigned long long id = 0;
-    if (!g_ctx_current || !g_ctx_id || g_ctx_current(&ctx) != 0 || !ctx || g_ctx_id(ctx, &id) != 0) return 0;
-    return id;
-}
 
 int scratch_address(unsigned char** out)
 {

@@ -1366,38 +1366,62 @@ __device__ __forceinline__ int net_voxel(int axis, int n, int nx, int ny, int nz
     return (r * Q + q) * P + p;
 }
 
-__global__ void k_pack_input(const uint8_t* __restrict__ cls, bf16* __restrict__ x, int nx, int ny, int nz, int axis)
+__global__ void k_pack_input(const uint8_t* __restrict__ cls, bf16* __restrict__ x, int nx, int ny, int nz, int axis,
+                             int vec)
 {
     const int n = blockIdx.x * blockDim.x + threadIdx.x;
     const int N = nx * ny * nz;
     if (n >= N) return;
     const int v = net_voxel(axis, n, nx, ny, nz);
     const uint8_t c = cls[n];
+    const uint32_t one = 0x3f80u;  // BF16 1
+    const uint32_t w0 = ((c & 3) != 0 ? one : 0u) | ((c & 4) != 0 ? one << 16 : 0u);
     bf16* o = x + (size_t)v * 16;
-    const bf16 zero = __float2bfloat16_rn(0.0f);
-    o[0] = __float2bfloat16_rn((c & 3) != 0 ? 1.0f : 0.0f);
-    o[1] = __float2bfloat16_rn((c & 4) != 0 ? 1.0f : 0.0f);
-    for (int k = 2; k < 16; ++k) o[k] = zero;
+    if (vec) {
+        reinterpret_cast<uint4*>(o)[0] = make_uint4(w0, 0u, 0u, 0u);
+        reinterpret_cast<uint4*>(o)[1] = make_uint4(0u, 0u, 0u, 0u);
+    } else {
+        unsigned short* h = reinterpret_cast<unsigned short*>(o);
+        h[0] = (unsigned short)w0;
+        h[1] = (unsigned short)(w0 >> 16);
+        for (int k = 2; k < 16; ++k) h[k] = 0;
+    }
 }
 
 // sum and count of y[.][3] over the forced cluster (FP64)
-__global__ void k_cluster_mean(const float* __restrict__ y, int ldy, const uint8_t* __restrict__ cls, int nx, int ny,
+__global__ void __launch_bounds__(256) k_cluster_mean(const float* __restrict__ y, int ldy, const uint8_t* __restrict__ cls, int nx, int ny,
                                int nz, int axis, double* __restrict__ acc)
 {
-    const int n = blockIdx.x * blockDim.x + threadIdx.x;
     const int N = nx * ny * nz;
-    double s = 0.0, c = 0.0;
-    if (n < N && (cls[n] & 4)) {
-        s = y[(size_t)net_voxel(axis, n, nx, ny, nz) * ldy + 3];
-        c = 1.0;
+    double s = 0.0;
+    int c = 0;
+    for (long long n = (long long)blockIdx.x * 256 + threadIdx.x; n < N; n += (long long)gridDim.x * 256) {
+        if (cls[n] & 4) {
+            s += y[(size_t)net_voxel(axis, (int)n, nx, ny, nz) * ldy + 3];
+            ++c;
+        }
     }
-    for (int o = 16; o > 0; o >>= 1) {
-        s += __shfl_xor_sync(0xffffffffu, s, o);
-        c += __shfl_xor_sync(0xffffffffu, c, o);
+    // the block's sum, so that few atomic additions meet at the two totals
+    __shared__ double part[8];
+    for (int o = 16; o > 0; o >>= 1) s += __shfl_xor_sync(0xffffffffu, s, o);
+    const int cw = __reduce_add_sync(0xffffffffu, c);
+    __shared__ int cnt[8];
+    if ((threadIdx.x & 31) == 0) {
+        part[threadIdx.x >> 5] = s;
+        cnt[threadIdx.x >> 5] = cw;
     }
-    if ((threadIdx.x & 31) == 0 && c > 0.0) {
-        atomicAdd(acc, s);
-        atomicAdd(acc + 1, c);
+    __syncthreads();
+    if (threadIdx.x == 0) {
+        double t = 0.0;
+        int k = 0;
+        for (int w = 0; w < 8; ++w) {
+            t += part[w];
+            k += cnt[w];
+        }
+        if (k > 0) {
+            atomicAdd(acc, t);
+            atomicAdd(acc + 1, (double)k);
+        }
     }
 }
 
@@ -1931,7 +1955,7 @@ int sg_pack_input(const uint8_t* cls, void* x, int nx, int ny, int nz, int axis,
         return MP_EINVAL;
     }
     const int N = nx * ny * nz;
-    k_pack_input<<<grid1(N, 256), 256, 0, (cudaStream_t)stream>>>(cls, (bf16*)x, nx, ny, nz, axis);
+    k_pack_input<<<grid1(N, 256), 256, 0, (cudaStream_t)stream>>>(cls, (bf16*)x, nx, ny, nz, axis, aligned16(x));
     MP_CUDA(cudaGetLastError());
     return MP_OK;
 }
@@ -1948,10 +1972,10 @@ int sg_unpack_output(const float* y, int ldy, const uint8_t* cls, float* u, floa
     const int N = nx * ny * nz;
     double* acc = nullptr;
     if (rho) {
-        MP_CUDA(cudaMallocAsync((void**)&acc, 2 * sizeof(double), s));
+        MP_CUDA(pool_malloc((void**)&acc, 2 * sizeof(double), s));
         cudaError_t e = cudaMemsetAsync(acc, 0, 2 * sizeof(double), s);
         if (e == cudaSuccess) {
-            k_cluster_mean<<<grid1(N, 256), 256, 0, s>>>(y, ldy, cls, nx, ny, nz, axis, acc);
+            k_cluster_mean<<<std::min(grid1(N, 256), 152 * 8), 256, 0, s>>>(y, ldy, cls, nx, ny, nz, axis, acc);
             e = cudaGetLastError();
         }
         if (e != cudaSuccess) {

@@ -84,6 +84,9 @@ _lib.lb_steady.argtypes = [ctypes.POINTER(mp_geometry), _dp, _c_dbl, _c_dbl, _c_
                            _c_vp, _c_vp, ctypes.POINTER(_c_i64), _dp, _c_vp]
 _lib.mp_classify.argtypes = [ctypes.POINTER(mp_geometry), _c_vp, ctypes.POINTER(_c_i64),
                              ctypes.POINTER(_c_i64), ctypes.POINTER(_c_i64), _c_vp]
+_lib.mp_classify_device.argtypes = _lib.mp_classify.argtypes
+_lib.mp_release_cached.argtypes = []
+_lib.mp_release_cached.restype = None
 _lib.mp_step_noalloc.argtypes = [_c_int, _c_int, _c_int, _c_vp, _c_vp, _c_dbl, _c_dbl, _c_dbl, _c_int,
                                  _c_vp, _c_vp, _c_vp, _c_vp, _c_vp, _c_vp]
 _lib.mp_group_create.argtypes = [ctypes.POINTER(_c_vp), ctypes.POINTER(_c_vp), _c_int, _c_int, _c_int]
@@ -115,7 +118,7 @@ _lib.sg_pack_target.argtypes = [_vp, _vp, _vp, _c_i, _c_i, _c_i, _c_i, _f32, _f3
 _lib.sg_mse.argtypes = [_vp, _c_i, _vp, _c_i, _vp, _vp, _vp, _c_i, _c_i, _c_dbl, _vp]
 _lib.sg_adam.argtypes = [_vp, _vp, _vp, _vp, _c_i64, _f32, _f32, _f32, _f32, _c_i, _vp, _vp, _c_i, _c_i, _vp]
 for _f in ("mp_init", "mp_init_batch", "mp_step", "mp_vacf", "mp_mass", "mp_info", "mp_get_field",
-           "mp_set_field", "lb_steady", "mp_classify", "mp_step_noalloc", "mp_group_create", "mp_group_create_ex",
+           "mp_set_field", "lb_steady", "mp_classify", "mp_classify_device", "mp_step_noalloc", "mp_group_create", "mp_group_create_ex",
            "mp_grid_wait_selftest",
            "mp_group_step", "mp_group_block_size", "sg_conv3d", "sg_conv3d_wgrad", "sg_conv3d_ex",
            "sg_conv3d_wgrad_ex", "sg_up2_grad_relu", "sg_pool2_grad_relu", "sg_check", "sg_pool2",
@@ -345,6 +348,26 @@ def mp_classify(solid, stream=None):
                             ctypes.byref(nc), _stream(stream)))
     del keep
     return cls, (nf.value, ni.value, nc.value)
+
+
+def mp_classify_device(solid, cls, stream=None):
+    """Node classes of mp_classify written to `cls`, a contiguous CUDA uint8 tensor of at least
+    N elements; returns (n_fluid, n_interface)."""
+    g, keep = make_geometry(solid)
+    n = g.nx * g.ny * g.nz
+    if (not getattr(cls, "is_cuda", False) or str(cls.dtype) != "torch.uint8" or not cls.is_contiguous()
+            or cls.numel() < n):
+        raise MPBufferError(f"cls: needs a contiguous CUDA uint8 tensor of at least {n} elements")
+    nf, ni = _c_i64(), _c_i64()
+    _check(_lib.mp_classify_device(ctypes.byref(g), _addr(cls), ctypes.byref(nf), ctypes.byref(ni), None,
+                                   _stream(stream)))
+    del keep
+    return nf.value, ni.value
+
+
+def mp_release_cached():
+    """mp_release_cached of include/mp.h."""
+    _lib.mp_release_cached()
 
 
 def _device_of(buf):

@@ -267,8 +267,8 @@ def warm_start(solid, force, model=None):
     torch = _torch()
     from . import mp
     model = model or load()[0]
-    cls, _ = mp.mp_classify(solid)
-    cls_dev = torch.as_tensor(cls).cuda()
+    cls_dev = torch.empty(tuple(solid.shape), dtype=torch.uint8, device="cuda")
+    mp.mp_classify_device(solid, cls_dev)
     u = torch.zeros((3,) + tuple(solid.shape), dtype=torch.float32, device="cuda")
     rho = torch.ones(tuple(solid.shape), dtype=torch.float32, device="cuda")
     model.predict(cls_dev, solid.shape, force, u, rho)
