@@ -43,13 +43,19 @@ struct LbArgs {
     const uint32_t* fluid;
     const int32_t* fbase;    // fluid nodes before each 32-node word
     const int32_t* flist;    // lattice node of fluid index k
-    const uint32_t* omask;   // open-link mask of fluid index k (bit i-1: r - c_i is fluid)
+    const uint32_t* omask;   // fluid index k: bit i-1: r - c_i is fluid; kXlo, kXhi, kForced
+    const uint4* rows;       // fluid index k: eight 16-bit offsets of the row centres from k
     const uint2* fw;         // {fluid bits, fluid nodes before the word} per 32-node word
     const uint32_t* forced;  // the force acts on these nodes (the largest fluid cluster)
     float Fx, Fy, Fz;
     float inv_tau;
     float guo;  // 1 - 1/(2 tau)
 };
+
+// flags beside the 18 link bits: x - 1 and x + 1 lie in the node's row without wrapping, the
+// force acts on the node
+constexpr uint32_t kXlo = 1u << 18, kXhi = 1u << 19, kForced = 1u << 20;
+constexpr int kFarRow = -32768;  // a row centre out of the 16-bit offsets' reach
 
 __device__ __forceinline__ bool lb_bit(const uint32_t* __restrict__ w, int n)
 {
@@ -60,34 +66,76 @@ __device__ __forceinline__ bool lb_bit(const uint32_t* __restrict__ w, int n)
 // rho_out when given), fold max|u - u_prev| (FP64) into *res_bits (non-negative doubles
 // order like their bits), then store u into u_prev. u_prev is compact [3][N_F]; u_out and
 // rho_out are dense (their solid entries are zeroed once by the host).
+// Everything static (the sources' places) is worked out before griddepcontrol.wait, while the
+// previous step drains. kRows: the row centres come as 16-bit offsets from a table of 16 bytes
+// a node instead of eight lookups (about 100 of 870 instructions; the step issues 70 % of the
+// time); rows beyond their reach, where z wraps around, are looked up. kWide: populations
+// beyond 2^32 elements (a source's plane is then found at its load).
+template <bool kRows, bool kWide>
 __global__ void __launch_bounds__(kLbThreads, MP_LB_MIN_BLOCKS)
-    k_lb_step(const LbArgs a, const float* __restrict__ g, float* __restrict__ gn, int mode,
+    k_lb_step(const __grid_constant__ LbArgs a, const float* __restrict__ g, float* __restrict__ gn, int mode,
               float* __restrict__ u_prev, float* __restrict__ u_out, float* __restrict__ rho_out,
               unsigned long long* __restrict__ res_bits)
 {
-    pdl_enter();  // launched with programmatic dependent launch: the previous step's populations
+    cudaTriggerProgrammaticLaunchCompletion();
     const int k = blockIdx.x * kLbThreads + threadIdx.x;
     const size_t NF = (size_t)a.NF;
     double res = 0.0;
-    if (k < a.NF) {
-        const int n = __ldg(a.flist + k);
-        const uint32_t mask = __ldg(a.omask + k);
-        const Nbr b = nbrs_of(a.nx, a.ny, a.nz, a.dx, a.dxy, n);
+    const bool active = k < a.NF;
+    const uint32_t nf = (uint32_t)a.NF;
+    uint32_t at[kQ];  // element of g that link i is read from (kWide: without its plane)
+    uint32_t mask = 0;
+    if (active) {
+        mask = __ldg(a.omask + k);
         // fluid-list index of each source row's centre; sources in a row are consecutive
         int C[8];
+        if constexpr (kRows) {
+            const uint4 r = __ldg(a.rows + k);
+            const uint32_t w[4] = {r.x, r.y, r.z, r.w};
+            bool far = false;
 #pragma unroll
-        for (int j = 0; j < 8; ++j) C[j] = fluid_index(a.fw, src_of(b, row_centre(j)));
-        const bool xlo = b.oxm == -1, xhi = b.oxp == 1;
+            for (int j = 0; j < 8; ++j) {
+                const int o = (int)(short)(w[j >> 1] >> (16 * (j & 1)));
+                C[j] = k + o;
+                far |= o == kFarRow;
+            }
+            if (far) {
+                const Nbr b = nbrs_of(a.nx, a.ny, a.nz, a.dx, a.dxy, __ldg(a.flist + k));
+#pragma unroll
+                for (int j = 0; j < 8; ++j) C[j] = fluid_index(a.fw, src_of(b, row_centre(j)));
+            }
+        } else {
+            const Nbr b = nbrs_of(a.nx, a.ny, a.nz, a.dx, a.dxy, __ldg(a.flist + k));
+#pragma unroll
+            for (int j = 0; j < 8; ++j) C[j] = fluid_index(a.fw, src_of(b, row_centre(j)));
+        }
+        at[0] = (uint32_t)k;
+#pragma unroll
+        for (int i = 1; i < kQ; ++i) {
+            const int row = row_of(i);
+            const int base = row < 0 ? k : C[row < 0 ? 0 : row];
+            int s = base;
+            if (cx(i) > 0) s = base - 1;
+            if (cx(i) < 0) s = base + (row < 0 ? 1 : (int)((mask >> (row_centre(row < 0 ? 0 : row) - 1)) & 1u));
+            const bool open = (mask >> (i - 1)) & 1u;  // else halfway bounce-back
+            at[i] = (open ? (uint32_t)s : (uint32_t)k) + (kWide ? 0u : (open ? (uint32_t)i : (uint32_t)opposite(i)) * nf);
+        }
+        if ((mask & (kXlo | kXhi)) != (kXlo | kXhi)) {
+            // the sources beyond the wrap of x (rare) are looked up one by one
+            const Nbr b = nbrs_of(a.nx, a.ny, a.nz, a.dx, a.dxy, __ldg(a.flist + k));
+#pragma unroll
+            for (int i = 1; i < kQ; ++i)
+                if (cx(i) != 0 && !(mask & (cx(i) > 0 ? kXlo : kXhi)) && ((mask >> (i - 1)) & 1u))
+                    at[i] = (uint32_t)fluid_index(a.fw, src_of(b, i)) + (kWide ? 0u : (uint32_t)i * nf);
+        }
+    }
+    cudaGridDependencySynchronize();  // the previous step's populations and residual are visible
+    if (active) {
         float f[kQ];
 #pragma unroll
         for (int i = 0; i < kQ; ++i) {
-            if (i == 0) {
-                f[0] = g[k];
-            } else if ((mask >> (i - 1)) & 1u) {
-                f[i] = g[(size_t)i * NF + source_index(i, k, C, mask, xlo, xhi, b, a.fw)];
-            } else {
-                f[i] = g[(size_t)opposite(i) * NF + k];  // halfway bounce-back
-            }
+            const size_t plane = kWide ? (size_t)(i == 0 || ((mask >> (i > 0 ? i - 1 : 0)) & 1u) ? i : opposite(i)) * NF : 0;
+            f[i] = g[plane + at[i]];
         }
         float drho = 0.f, mx = 0.f, my = 0.f, mz = 0.f;
 #pragma unroll
@@ -97,7 +145,7 @@ __global__ void __launch_bounds__(kLbThreads, MP_LB_MIN_BLOCKS)
             my += float(cy(i)) * f[i];
             mz += float(cz(i)) * f[i];
         }
-        const bool on = lb_bit(a.forced, n);
+        const bool on = (mask & kForced) != 0;
         const float Fx = on ? a.Fx : 0.0f, Fy = on ? a.Fy : 0.0f, Fz = on ? a.Fz : 0.0f;
         const float rho = 1.0f + drho;
         const float inv_rho = 1.0f / rho;
@@ -136,6 +184,7 @@ __global__ void __launch_bounds__(kLbThreads, MP_LB_MIN_BLOCKS)
             u_prev[NF + k] = uy;
             u_prev[2 * NF + k] = uz;
         } else if (mode == 2) {
+            const int n = __ldg(a.flist + k);
             u_out[n] = ux;
             u_out[(size_t)a.N + n] = uy;
             u_out[2 * (size_t)a.N + n] = uz;
@@ -151,9 +200,18 @@ __global__ void __launch_bounds__(kLbThreads, MP_LB_MIN_BLOCKS)
         }
     }
     if (mode == 2) {
+        // one atomic maximum per block, and only where it still raises the total (every warp's
+        // met at one address: 110 us of a 128^3 step)
+        __shared__ double s_res[kLbThreads / 32];
 #pragma unroll
         for (int o = 16; o > 0; o >>= 1) res = fmax(res, __shfl_xor_sync(0xffffffffu, res, o));
-        if ((threadIdx.x & 31) == 0 && res > 0.0) atomicMax(res_bits, (unsigned long long)__double_as_longlong(res));
+        if ((threadIdx.x & 31) == 0) s_res[threadIdx.x >> 5] = res;
+        __syncthreads();
+        if (threadIdx.x == 0) {
+            for (int w = 1; w < kLbThreads / 32; ++w) res = fmax(res, s_res[w]);
+            const unsigned long long bits = (unsigned long long)__double_as_longlong(res);
+            if (bits > *(volatile unsigned long long*)res_bits) atomicMax(res_bits, bits);
+        }
     }
 }
 
@@ -193,21 +251,39 @@ __global__ void k_lb_init(const LbArgs a, const float* __restrict__ u0, const fl
 
 }  // namespace
 
-// Per lb_steady call: the open-link mask of every fluid node and the {fluid bits, prefix}
-// words that locate link sources in the fluid list.
-__global__ void k_lb_prep(const LbArgs a, int W, uint32_t* __restrict__ omask, uint2* __restrict__ fw)
+// Per lb_steady call: the {fluid bits, prefix} words that locate link sources in the fluid list,
+// then (k_lb_prep) the open-link mask and flags of every fluid node and, when `rows` is given,
+// its row offsets.
+__global__ void k_lb_words(const LbArgs a, int W, uint2* __restrict__ fw)
 {
     const int t = blockIdx.x * blockDim.x + threadIdx.x;
     if (t < W) fw[t] = make_uint2(a.fluid[t], (uint32_t)a.fbase[t]);
-    if (t < a.NF) {
-        const Nbr b = nbrs_of(a.nx, a.ny, a.nz, a.dx, a.dxy, a.flist[t]);
-        uint32_t m = 0;
+}
+__global__ void k_lb_prep(const LbArgs a, uint32_t* __restrict__ omask, uint4* __restrict__ rows)
+{
+    const int t = blockIdx.x * blockDim.x + threadIdx.x;
+    if (t >= a.NF) return;
+    const int n = a.flist[t];
+    const Nbr b = nbrs_of(a.nx, a.ny, a.nz, a.dx, a.dxy, n);
+    uint32_t m = 0;
 #pragma unroll
-        for (int i = 1; i < kQ; ++i) {
-            const int s = src_of(b, i);
-            if ((a.fluid[s >> 5] >> (s & 31)) & 1u) m |= 1u << (i - 1);
+    for (int i = 1; i < kQ; ++i) {
+        const int s = src_of(b, i);
+        if ((a.fluid[s >> 5] >> (s & 31)) & 1u) m |= 1u << (i - 1);
+    }
+    if (b.oxm == -1) m |= kXlo;
+    if (b.oxp == 1) m |= kXhi;
+    if (lb_bit(a.forced, n)) m |= kForced;
+    omask[t] = m;
+    if (rows) {
+        uint32_t w[4] = {0u, 0u, 0u, 0u};
+#pragma unroll
+        for (int j = 0; j < 8; ++j) {
+            const int o = fluid_index(a.fw, src_of(b, row_centre(j))) - t;
+            const int v = o > kFarRow && o < -kFarRow ? o : kFarRow;
+            w[j >> 1] |= (uint32_t)(v & 0xffff) << (16 * (j & 1));
         }
-        omask[t] = m;
+        rows[t] = make_uint4(w[0], w[1], w[2], w[3]);
     }
 }
 
@@ -237,10 +313,16 @@ extern "C" int lb_steady(const mp_geometry* geom, const double force[3], double 
     float *g0 = nullptr, *g1 = nullptr, *uprev = nullptr;
     uint32_t* omask = nullptr;
     uint2* fw = nullptr;
+    uint4* rows = nullptr;
+    // the row table where 16-bit offsets reach the neighbouring planes (at the fluid nodes of a
+    // plane on average)
+    const bool wide = kQ * (unsigned long long)NF >= (1ull << 32);
+    const bool use_rows = !wide && (double)G.n_fluid / G.nz * 1.2 + G.nx < 32000.0;
     unsigned long long* res_d = nullptr;
     cudaError_t e = pool_malloc((void**)&g0, sizeof(float) * kQ * NF, s);
     if (e == cudaSuccess) e = pool_malloc((void**)&omask, sizeof(uint32_t) * NF, s);
     if (e == cudaSuccess) e = pool_malloc((void**)&fw, sizeof(uint2) * (size_t)(G.W > 0 ? G.W : 1), s);
+    if (e == cudaSuccess && use_rows) e = pool_malloc((void**)&rows, sizeof(uint4) * NF, s);
     if (e == cudaSuccess) e = pool_malloc((void**)&g1, sizeof(float) * kQ * NF, s);
     if (e == cudaSuccess) e = pool_malloc((void**)&uprev, sizeof(float) * 3 * NF, s);
     if (e == cudaSuccess) e = pool_malloc((void**)&res_d, sizeof(unsigned long long), s);
@@ -253,6 +335,7 @@ extern "C" int lb_steady(const mp_geometry* geom, const double force[3], double 
         if (uprev) cudaFreeAsync(uprev, s);
         if (omask) cudaFreeAsync(omask, s);
         if (fw) cudaFreeAsync(fw, s);
+        if (rows) cudaFreeAsync(rows, s);
         if (res_d) cudaFreeAsync(res_d, s);
         free_geometry(&G, s, true);
         cudaStreamSynchronize(s);
@@ -274,6 +357,7 @@ extern "C" int lb_steady(const mp_geometry* geom, const double force[3], double 
     a.fbase = G.fbase;
     a.flist = G.flist;
     a.omask = omask;
+    a.rows = rows;
     a.fw = fw;
     a.forced = G.cluster;
     a.Fx = (float)force[0];
@@ -284,8 +368,8 @@ extern "C" int lb_steady(const mp_geometry* geom, const double force[3], double 
     // one thread per fluid node (at least one block, so that a medium without fluid still
     // runs its checks: its residual is 0)
     const int blocks = (int)((NF + kLbThreads - 1) / kLbThreads);
-    const size_t prep = std::max<size_t>(NF, (size_t)G.W);
-    k_lb_prep<<<(unsigned)((prep + 255) / 256), 256, 0, s>>>(a, G.W, omask, fw);
+    k_lb_words<<<(unsigned)((G.W + 255) / 256), 256, 0, s>>>(a, G.W, fw);
+    k_lb_prep<<<(unsigned)((NF + 255) / 256), 256, 0, s>>>(a, omask, rows);
     k_lb_init<<<blocks, kLbThreads, 0, s>>>(a, u_init, rho_init, g0, uprev);
     e = cudaGetLastError();
     int64_t t = 0;
@@ -300,7 +384,7 @@ extern "C" int lb_steady(const mp_geometry* geom, const double force[3], double 
             mode = 1;
         if (mode == 2) e = cudaMemsetAsync(res_d, 0, sizeof(unsigned long long), s);
         if (e == cudaSuccess)
-            e = launch_pdl(k_lb_step, dim3(blocks), dim3(kLbThreads), s, a, (const float*)g0, g1, mode, uprev, u_out,
+            e = launch_pdl(wide ? k_lb_step<false, true> : (use_rows ? k_lb_step<true, false> : k_lb_step<false, false>), dim3(blocks), dim3(kLbThreads), s, a, (const float*)g0, g1, mode, uprev, u_out,
                            rho_out, res_d);
         float* tmp = g0;
         g0 = g1;
