@@ -10,14 +10,15 @@
 // fluid list: g[i*N_F + k] for fluid node k (structure of arrays). One thread per fluid node;
 // the compact index of a neighbour s is prefix[s >> 5] + popc(fluid bits of s's word below
 // s), from two bit-sized arrays that stay cache-resident, so a warp's reads and writes cover
-// whole sectors of fluid data only. The steady criterion max|u(t) - u(t-1)| is evaluated in
-// FP64.
+// whole sectors of fluid data only. The steady criterion max|u(t) - u(t-1)| is evaluated
+// without rounding.
 // The body force acts on the largest connected fluid cluster only (sealed pockets stay at
 // rest, their steady Stokes velocity). At every failed residual check the state is replaced
 // by the mean of the last two iterates: the fixed point is unchanged, an error mode of
 // eigenvalue lambda is scaled by (1 + lambda)/2, and the undamped period-2 modes that
 // bounce-back sustains at nodes with few open links disappear (without it the residual of a
 // porous medium stalls near |F|).
+#include <cfloat>
 #include <cmath>
 #include <cstring>
 #include <string>
@@ -29,13 +30,14 @@ using namespace mp;
 
 namespace {
 
-constexpr int kLbThreads = 256;
-// 5 resident blocks per SM (48 registers a thread): with sources located by row (eight
-// prefix + popcount lookups a node) the step keeps its 19 gathers and the row centres in
-// registers; measured at 8, 6, 5 and 4 blocks (32 registers spill), 5 is fastest
-#ifndef MP_LB_MIN_BLOCKS
-#define MP_LB_MIN_BLOCKS 5
-#endif
+// Blocks of 128 threads, 10 per SM (48 registers a thread): the step keeps its 19 gathers and
+// their places in registers. Measured per step at 128^3 / 192^3 / 384^3: 26.5 / 80.8 / 645 us; 256 x 5
+// 26.7 / 81.7 / 656, 256 x 4 28.6 / 87.9 / 734, 512 x 2 30.4 / 92.0 / 781. Launches that a SM's share of
+// 1024 threads takes in one wave (kLbSmall nodes) run blocks of 64 with 64 registers: nothing
+// waits for a block slot, small blocks spread evenly (64^3: 4.2 us, 5.0 with 128 x 10).
+constexpr int kLbThreads = 128, kLbMinBlocks = 10;
+constexpr int kLbSmallThreads = 64, kLbSmallMinBlocks = 16;
+constexpr long long kLbSmall = 152LL * 1024;
 
 struct LbArgs {
     int nx, ny, nz, N, NF;
@@ -52,6 +54,29 @@ struct LbArgs {
     float guo;  // 1 - 1/(2 tau)
 };
 
+// |a - b| of two FP32 numbers without rounding, as a key that orders like the value: the FP32
+// difference s and its rounding error e (a - b = s + e exactly; Knuth's two-sum), the bits of |s|
+// above those of e towards |s| made to order as unsigned. In FP64 the same comparison took some
+// 35 operations of a pipe that does two per clock and SM (50 us of a 128^3 check).
+__device__ __forceinline__ unsigned long long diff_key(float a, float b)
+{
+    const float s = __fsub_rn(a, b), t = __fsub_rn(s, a);
+    float e = __fadd_rn(__fsub_rn(a, __fsub_rn(s, t)), __fsub_rn(-b, t));
+    if (s < 0.0f) e = -e;
+    const uint32_t w = __float_as_uint(e);
+    return ((unsigned long long)__float_as_uint(fabsf(s)) << 32) | (w ^ ((w >> 31) ? 0xffffffffu : 0x80000000u));
+}
+double key_value(unsigned long long key)
+{
+    const uint32_t sb = (uint32_t)(key >> 32);
+    uint32_t eb = (uint32_t)key;
+    eb = (eb >> 31) ? eb ^ 0x80000000u : ~eb;
+    float s, e;
+    memcpy(&s, &sb, 4);
+    memcpy(&e, &eb, 4);
+    return key == 0 ? 0.0 : (std::isfinite(s) ? (double)s + (double)e : (double)INFINITY);
+}
+
 // flags beside the 18 link bits: x - 1 and x + 1 lie in the node's row without wrapping, the
 // force acts on the node
 constexpr uint32_t kXlo = 1u << 18, kXhi = 1u << 19, kForced = 1u << 20;
@@ -63,24 +88,24 @@ __device__ __forceinline__ bool lb_bit(const uint32_t* __restrict__ w, int n)
 }
 
 // mode 0: plain step; 1: also store u into u_prev; 2: store u into u_out (and rho into
-// rho_out when given), fold max|u - u_prev| (FP64) into *res_bits (non-negative doubles
-// order like their bits), then store u into u_prev. u_prev is compact [3][N_F]; u_out and
-// rho_out are dense (their solid entries are zeroed once by the host).
+// rho_out when given), fold max|u - u_prev| into *res_key (diff_key), then store u into
+// u_prev. u_prev is compact [3][N_F]; u_out and rho_out are dense (their solid entries are
+// zeroed once by the host).
 // Everything static (the sources' places) is worked out before griddepcontrol.wait, while the
 // previous step drains. kRows: the row centres come as 16-bit offsets from a table of 16 bytes
 // a node instead of eight lookups (about 100 of 870 instructions; the step issues 70 % of the
 // time); rows beyond their reach, where z wraps around, are looked up. kWide: populations
 // beyond 2^32 elements (a source's plane is then found at its load).
-template <bool kRows, bool kWide>
-__global__ void __launch_bounds__(kLbThreads, MP_LB_MIN_BLOCKS)
+template <bool kRows, bool kWide, int kB, int kMinBlocks>
+__global__ void __launch_bounds__(kB, kMinBlocks)
     k_lb_step(const __grid_constant__ LbArgs a, const float* __restrict__ g, float* __restrict__ gn, int mode,
               float* __restrict__ u_prev, float* __restrict__ u_out, float* __restrict__ rho_out,
-              unsigned long long* __restrict__ res_bits)
+              unsigned long long* __restrict__ res_key)
 {
     cudaTriggerProgrammaticLaunchCompletion();
-    const int k = blockIdx.x * kLbThreads + threadIdx.x;
+    const int k = blockIdx.x * kB + threadIdx.x;
     const size_t NF = (size_t)a.NF;
-    double res = 0.0;
+    unsigned long long res = 0;
     const bool active = k < a.NF;
     const uint32_t nf = (uint32_t)a.NF;
     uint32_t at[kQ];  // element of g that link i is read from (kWide: without its plane)
@@ -137,6 +162,14 @@ __global__ void __launch_bounds__(kLbThreads, MP_LB_MIN_BLOCKS)
             const size_t plane = kWide ? (size_t)(i == 0 || ((mask >> (i > 0 ? i - 1 : 0)) & 1u) ? i : opposite(i)) * NF : 0;
             f[i] = g[plane + at[i]];
         }
+        // the reference of a check, read before the 19 stores: behind them the three loads waited
+        // for the stores to drain (135 us instead of 33 for a checked step of a 128^3 box)
+        float px = 0.f, py = 0.f, pz = 0.f;
+        if (mode == 2) {
+            px = u_prev[k];
+            py = u_prev[NF + k];
+            pz = u_prev[2 * NF + k];
+        }
         float drho = 0.f, mx = 0.f, my = 0.f, mz = 0.f;
 #pragma unroll
         for (int i = 0; i < kQ; ++i) {
@@ -189,10 +222,9 @@ __global__ void __launch_bounds__(kLbThreads, MP_LB_MIN_BLOCKS)
             u_out[(size_t)a.N + n] = uy;
             u_out[2 * (size_t)a.N + n] = uz;
             if (rho_out) rho_out[n] = rho;
-            res = fmax(fabs((double)ux - (double)u_prev[k]),
-                       fmax(fabs((double)uy - (double)u_prev[NF + k]), fabs((double)uz - (double)u_prev[2 * NF + k])));
-            // a non-finite velocity (fmax drops NaN) counts as an infinite residual
-            if (!(fabs((double)ux) + fabs((double)uy) + fabs((double)uz) <= 1.0e300)) res = INFINITY;
+            res = max(diff_key(ux, px), max(diff_key(uy, py), diff_key(uz, pz)));
+            // a non-finite velocity counts as an infinite residual
+            if (!(fabsf(ux) <= FLT_MAX && fabsf(uy) <= FLT_MAX && fabsf(uz) <= FLT_MAX)) res = 0x7f800000ull << 32;
             // this node's u(t) is the reference of the next check when it is due next step
             u_prev[k] = ux;
             u_prev[NF + k] = uy;
@@ -202,24 +234,35 @@ __global__ void __launch_bounds__(kLbThreads, MP_LB_MIN_BLOCKS)
     if (mode == 2) {
         // one atomic maximum per block, and only where it still raises the total (every warp's
         // met at one address: 110 us of a 128^3 step)
-        __shared__ double s_res[kLbThreads / 32];
+        __shared__ unsigned long long s_res[kB / 32];
 #pragma unroll
-        for (int o = 16; o > 0; o >>= 1) res = fmax(res, __shfl_xor_sync(0xffffffffu, res, o));
+        for (int o = 16; o > 0; o >>= 1) res = max(res, __shfl_xor_sync(0xffffffffu, res, o));
         if ((threadIdx.x & 31) == 0) s_res[threadIdx.x >> 5] = res;
         __syncthreads();
         if (threadIdx.x == 0) {
-            for (int w = 1; w < kLbThreads / 32; ++w) res = fmax(res, s_res[w]);
-            const unsigned long long bits = (unsigned long long)__double_as_longlong(res);
-            if (bits > *(volatile unsigned long long*)res_bits) atomicMax(res_bits, bits);
+            for (int w = 1; w < kB / 32; ++w) res = max(res, s_res[w]);
+            if (res > *(volatile unsigned long long*)res_key) atomicMax(res_key, res);
         }
     }
 }
 
-// g0 <- (g0 + g1) / 2 over all populations: the mean of the last two iterates
-__global__ void k_lb_mean(float* __restrict__ g0, const float* __restrict__ g1, size_t count)
+// g0 <- (g0 + g1) / 2 over all populations: the mean of the last two iterates (four a thread;
+// both arrays start on 256-byte boundaries)
+__global__ void __launch_bounds__(256) k_lb_mean(float* __restrict__ g0, const float* __restrict__ g1, size_t count)
 {
-    for (size_t k = blockIdx.x * (size_t)blockDim.x + threadIdx.x; k < count; k += (size_t)gridDim.x * blockDim.x)
+    const size_t i = blockIdx.x * (size_t)256 + threadIdx.x, n4 = count / 4;
+    if (i < n4) {
+        float4 a = reinterpret_cast<const float4*>(g0)[i];
+        const float4 b = reinterpret_cast<const float4*>(g1)[i];
+        a.x = 0.5f * (a.x + b.x);
+        a.y = 0.5f * (a.y + b.y);
+        a.z = 0.5f * (a.z + b.z);
+        a.w = 0.5f * (a.w + b.w);
+        reinterpret_cast<float4*>(g0)[i] = a;
+    } else if (i < n4 + count % 4) {
+        const size_t k = 4 * n4 + (i - n4);
         g0[k] = 0.5f * (g0[k] + g1[k]);
+    }
 }
 
 // f = f^eq(rho0, u0) as deviations (u0 = 0 and rho0 = 1 when NULL; both dense); u_prev = u0
@@ -367,10 +410,17 @@ extern "C" int lb_steady(const mp_geometry* geom, const double force[3], double 
     a.guo = (float)(1.0 - 0.5 / tau);
     // one thread per fluid node (at least one block, so that a medium without fluid still
     // runs its checks: its residual is 0)
-    const int blocks = (int)((NF + kLbThreads - 1) / kLbThreads);
+    const bool small = (long long)NF <= kLbSmall;
+    const int threads = small ? kLbSmallThreads : kLbThreads;
+    const int blocks = (int)((NF + threads - 1) / threads);
+    auto kern = wide ? k_lb_step<false, true, kLbThreads, kLbMinBlocks>
+                : small ? (use_rows ? k_lb_step<true, false, kLbSmallThreads, kLbSmallMinBlocks>
+                                    : k_lb_step<false, false, kLbSmallThreads, kLbSmallMinBlocks>)
+                        : (use_rows ? k_lb_step<true, false, kLbThreads, kLbMinBlocks>
+                                    : k_lb_step<false, false, kLbThreads, kLbMinBlocks>);
     k_lb_words<<<(unsigned)((G.W + 255) / 256), 256, 0, s>>>(a, G.W, fw);
     k_lb_prep<<<(unsigned)((NF + 255) / 256), 256, 0, s>>>(a, omask, rows);
-    k_lb_init<<<blocks, kLbThreads, 0, s>>>(a, u_init, rho_init, g0, uprev);
+    k_lb_init<<<blocks, threads, 0, s>>>(a, u_init, rho_init, g0, uprev);
     e = cudaGetLastError();
     int64_t t = 0;
     double res = INFINITY;
@@ -384,7 +434,7 @@ extern "C" int lb_steady(const mp_geometry* geom, const double force[3], double 
             mode = 1;
         if (mode == 2) e = cudaMemsetAsync(res_d, 0, sizeof(unsigned long long), s);
         if (e == cudaSuccess)
-            e = launch_pdl(wide ? k_lb_step<false, true> : (use_rows ? k_lb_step<true, false> : k_lb_step<false, false>), dim3(blocks), dim3(kLbThreads), s, a, (const float*)g0, g1, mode, uprev, u_out,
+            e = launch_pdl(kern, dim3(blocks), dim3(threads), s, a, (const float*)g0, g1, mode, uprev, u_out,
                            rho_out, res_d);
         float* tmp = g0;
         g0 = g1;
@@ -394,7 +444,7 @@ extern "C" int lb_steady(const mp_geometry* geom, const double force[3], double 
             unsigned long long bits = 0;
             e = cudaMemcpyAsync(&bits, res_d, sizeof(bits), cudaMemcpyDeviceToHost, s);
             if (e == cudaSuccess) e = cudaStreamSynchronize(s);
-            memcpy(&res, &bits, sizeof(res));
+            res = key_value(bits);
             if (res < tol) {
                 converged = true;
                 break;
@@ -403,7 +453,8 @@ extern "C" int lb_steady(const mp_geometry* geom, const double force[3], double 
             // the mean of the last two iterates (g0 = t, g1 = t-1): same fixed point, and the
             // undamped period-2 modes that bounce-back sustains at confined nodes vanish
             if (t < max_steps) {
-                k_lb_mean<<<2 * 152 * 4, 256, 0, s>>>(g0, g1, (size_t)kQ * NF);
+                const size_t count = (size_t)kQ * NF;
+                k_lb_mean<<<(unsigned)((count / 4 + count % 4 + 255) / 256), 256, 0, s>>>(g0, g1, count);
                 e = cudaGetLastError();
             }
         }
