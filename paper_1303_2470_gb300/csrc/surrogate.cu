@@ -385,8 +385,8 @@ __global__ void __launch_bounds__(kTThreads) k_conv_tc(const ConvArgs a)
 }
 
 // ---------------------------------------------------------------------------------------
-// The same convolution marching along y (W a multiple of 8, K = 16, 32, 64, 96 or 128): the
-// kernel of the network's layers. Measured, forward on one box (tap by tap -> marching): 128^3,
+// The same convolution marching along y (W >= 3, K = 16, 32, 64, 96 or 128): the kernel of the
+// network's layers. Measured, forward on one box (tap by tap -> marching): 128^3,
 // 32 -> 32 channels 463 -> 167 us, 64 -> 32 643 -> 238 us; 64^3, 64 -> 64 171 -> 60 us (960
 // TFLOP/s); 32^3, 96 -> 96 60 -> 29 us; 16^3, 128 -> 128 59 -> 15 us.
 //
@@ -405,7 +405,7 @@ __global__ void __launch_bounds__(kTThreads) k_conv_tc(const ConvArgs a)
 // The column of 128 voxels is any 16 groups of 8 x-neighbours (b, z, x / 8): each group is
 // staged as 10 rows of 128 bytes, its voxels with their left and right neighbour (periodic),
 // and the descriptor's stride between 8-row groups is 1280 bytes. So a box of any W that is a
-// multiple of 8 fills the MMA's 128 rows.
+// multiple of 8 fills the MMA's 128 rows (other widths end each row with a short group).
 // Per accumulator the products are added in the order of k_conv_tc (taps ascending, then
 // channels): source rows ascend for sign = +1 and descend for sign = -1, and outputs are
 // bitwise the same.
@@ -543,8 +543,8 @@ __global__ void __launch_bounds__(kMThreads, 1) k_conv_march(const __grid_consta
                     if (g < m.NG) {
                         const int xg = g % m.GX, r = g / m.GX;
                         const int z = r % m.c.D, b = r / m.c.D;
-                        const int x = wrap(8 * xg - 1 + row % 10, W);
-                        off = x_voxel(m.c.up, m.c.D, H, W, b, wrap(z + sign * (d - 1), m.c.D), 0, x);
+                        const int x = 8 * xg - 1 + row % 10;  // beyond W: past the row's last neighbour
+                        if (x <= W) off = x_voxel(m.c.up, m.c.D, H, W, b, wrap(z + sign * (d - 1), m.c.D), 0, wrap(x, W));
                     }
                     s_off[row] = off;
                 }
@@ -711,7 +711,8 @@ __global__ void __launch_bounds__(kMThreads, 1) k_conv_march(const __grid_consta
             const int use = m.bufs == 2 ? nu >> 1 : nu;
             const int g = tc * 16 + tid / 8;
             const int xg = g % m.GX, r = g / m.GX;   // r = b D + z
-            const long long v0 = g < m.NG ? ((long long)r * H + y0) * W + 8 * xg + (tid & 7) : -1;
+            const int x = 8 * xg + (tid & 7);
+            const long long v0 = g < m.NG && x < W ? ((long long)r * H + y0) * W + x : -1;
             ok = mbar_wait_or(smem_u32(&s_afull[buf]), (uint32_t)use & 1u, fail);
             if (!__all_sync(0xffffffffu, ok)) break;
             asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
@@ -731,7 +732,7 @@ __global__ void __launch_bounds__(kMThreads, 1) k_conv_march(const __grid_consta
 }
 
 // ---------------------------------------------------------------------------------------
-// Weight gradient on the 5th-generation tensor cores (W a multiple of 8): dW[tap][ci][co] is a
+// Weight gradient on the 5th-generation tensor cores (W >= 3): dW[tap][ci][co] is a
 // product over voxels of x rows and dy rows, both channels-last, i.e. both operands with the
 // reduction index (voxels) as rows of shared memory: MN-major operands. What bounds a
 // tap-by-tap kernel is reading x and dy once per tap (27 times); here a unit takes one dz, a
@@ -751,7 +752,7 @@ __global__ void __launch_bounds__(kMThreads, 1) k_conv_march(const __grid_consta
 // dw with one reduction per element, 32 consecutive output channels per warp.
 // Measured (tap by tap with mma.sync -> this): one 128^3 box 32 -> 32 channels 2266 -> 157 us,
 // 64 -> 32 2297 -> 208 us (1117 TFLOP/s); 64^3 64 -> 64 365 -> 60 us; 16^3 128 -> 128 56 -> 13 us.
-// 13 warps: 4 epilogue, 1 MMA, 8 copies (cp.async, zero-filled for groups beyond the batch).
+// 13 warps: 4 epilogue, 1 MMA, 8 copies (cp.async, zero-filled beyond the row or batch).
 // Waits are bounded as in k_conv_march.
 // ---------------------------------------------------------------------------------------
 constexpr int kGThreads = 160 + kMCopy;
@@ -852,8 +853,9 @@ __global__ void __launch_bounds__(kGThreads, 1) k_wgrad_tc(const __grid_constant
                 if (g < m.NG) {
                     const int xg = g % m.GX, l = g / m.GX;
                     const int z = l % m.D, b = l / m.D;
-                    const int x = isx ? wrap(8 * xg - 1 + r % 10, W) : 8 * xg + r % 8;
-                    off = isx ? x_voxel(m.up, m.D, H, W, b, wrap(z + d - 1, m.D), 0, x) : ((b * m.D + z) * H) * W + x;
+                    const int x = isx ? 8 * xg - 1 + r % 10 : 8 * xg + r % 8;
+                    if (isx && x <= W) off = x_voxel(m.up, m.D, H, W, b, wrap(z + d - 1, m.D), 0, wrap(x, W));
+                    if (!isx && x < W) off = ((b * m.D + z) * H) * W + x;
                 }
                 if (isx)
                     s_xoff[r] = off;
@@ -1556,6 +1558,11 @@ bool weight_map(const ConvArgs& a, int NB, CUtensorMap* map)
                   CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) == CUDA_SUCCESS;
 }
 
+// x-rows are cut into groups of 8 voxels; the last one of a row may be short, and what it lacks
+// is work done for nothing. Rows of one or two voxels (an eighth, a quarter of a group) stay with
+// the tap-by-tap kernels, which the marching ones beat by about three.
+bool fills_groups(int W) { return W >= 3; }
+
 // Shape of the marching kernel for one layer, or false where it does not apply. The channel
 // block NB and the strip length T are those with the least estimated time: waves of one unit
 // per SM times the clocks of a unit, where a staged row costs the larger of its MMAs (products
@@ -1564,7 +1571,7 @@ bool weight_map(const ConvArgs& a, int NB, CUtensorMap* map)
 bool march_plan(const ConvArgs& a, int B, int sms, MarchArgs* out, size_t* smem)
 {
     const int K = a.K, N = a.N;
-    if (a.W % 8 || !(K == 16 || K == 32 || K == 64 || K == 96 || K == 128) || (long long)B * a.V >= (1LL << 31)) return false;
+    if (!fills_groups(a.W) || !(K == 16 || K == 32 || K == 64 || K == 96 || K == 128) || (long long)B * a.V >= (1LL << 31)) return false;
     const int kch = (K + 63) / 64;
     const size_t abytes = (size_t)kch * kMChunk;
     MarchArgs best{};
@@ -1581,7 +1588,7 @@ bool march_plan(const ConvArgs& a, int B, int sms, MarchArgs* out, size_t* smem)
         const int nA = (int)std::min<size_t>(kMStages, ((size_t)kMSmem - 1024 - bsm) / abytes);
         for (int T = 1; T <= a.H && T <= 16 && T * NB <= 512; T = T < 4 ? T + 1 : T + 2) {
             const int bufs = 2 * T * NB <= 512 ? 2 : 1;
-            const int GX = a.W / 8, NG = B * a.D * GX;
+            const int GX = (a.W + 7) / 8, NG = B * a.D * GX;
             const long long units = (long long)((NG + 15) / 16) * ((a.H + T - 1) / T) * nblk;
             if (units > (1LL << 30)) continue;
             double rows = 0.0;
@@ -1625,7 +1632,7 @@ int channel_block(int c) { return c % 64 == 0 ? 64 : (c % 32 == 0 ? 32 : 16); }
 // unit within 16 rows.
 bool wgrad_plan(const WgradArgs& a, int B, int sms, WgradTcArgs* m, size_t* smem)
 {
-    if (a.W % 8 || a.total >= (1LL << 31)) return false;
+    if (!fills_groups(a.W) || a.total >= (1LL << 31)) return false;
     const int ci = channel_block(a.Cin), co = channel_block(a.Cout);
     const size_t xb = (size_t)kMRows * 2 * ci, yb = (size_t)kTM * 2 * co;
     const int tiles = co == 64 ? 2 : 1, n = 3 * ci;
@@ -1643,7 +1650,7 @@ bool wgrad_plan(const WgradArgs& a, int B, int sms, WgradTcArgs* m, size_t* smem
     m->Cin = a.Cin;
     m->Cout = a.Cout;
     m->up = a.up;
-    m->GX = a.W / 8;
+    m->GX = (a.W + 7) / 8;
     m->NG = B * a.D * m->GX;
     m->nci = a.Cin / ci;
     m->nco = a.Cout / co;

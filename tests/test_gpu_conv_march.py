@@ -1,7 +1,7 @@
 """The tensor-core convolutions at the edges of the marching kernel's tiles: a column of 128
 voxels that the box does not fill, strips of rows that do not divide H, one-row boxes whose
 neighbours are the row itself, several channel blocks, both signs, every compiled channel
-count and the general kernel beside it (W not a multiple of 8). Operands are small integers,
+count, rows with a short last group, and the general kernel (W < 3). Operands are small integers,
 so every sum is exact in FP32 and the comparison has no tolerance; BF16 outputs are the
 exact sums rounded once."""
 import pytest
@@ -14,7 +14,9 @@ pytestmark = pytest.mark.gpu
     (1, 1, 1, 8, 16, 16), (1, 2, 3, 8, 16, 32), (2, 3, 5, 16, 32, 32), (1, 3, 2, 24, 96, 48), (2, 2, 4, 8, 64, 32),
     (1, 3, 7, 40, 128, 32), (1, 2, 1, 136, 16, 16), (1, 5, 17, 64, 64, 64), (3, 8, 8, 8, 128, 128),
     (1, 4, 33, 128, 32, 64), (1, 6, 19, 32, 96, 96), (1, 2, 9, 72, 64, 96), (2, 40, 40, 40, 32, 16),
-    (1, 1, 2, 256, 128, 96), (1, 3, 4, 16, 48, 32), (1, 3, 5, 12, 32, 32), (1, 2, 3, 16, 64, 272)])
+    (1, 1, 2, 256, 128, 96), (1, 3, 4, 16, 48, 32), (1, 3, 5, 12, 32, 32), (1, 2, 3, 16, 64, 272),
+    (2, 5, 6, 1, 32, 32), (1, 4, 5, 2, 16, 32), (2, 3, 7, 3, 32, 64), (1, 5, 4, 7, 64, 32), (1, 3, 9, 9, 96, 64),
+    (2, 4, 11, 31, 128, 96), (1, 2, 5, 127, 64, 64)])
 def test_conv_exact_on_integers(B, D, H, W, K, N):
     if not torch.cuda.is_available():
         pytest.skip("no CUDA device")

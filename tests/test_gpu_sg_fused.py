@@ -1,6 +1,6 @@
 """The fused forms of the network's passes (upsampled input, skip sum, ReLU mask, masked pool and
-upsampling gradients) against the separate calls: the same values bit for bit. Boxes whose
-width is and is not a multiple of 8 (the two convolution kernels), channel counts that the
+upsampling gradients) against the separate calls: the same values bit for bit. Boxes of
+widths and channel counts that the marching and the general convolution take, channel counts that the
 16-byte passes do and do not take, buffers off a 16-byte boundary, and the loss gradient with
 and without its vector form."""
 import pytest
@@ -23,7 +23,8 @@ def _rand(g, *shape):
 
 
 @pytest.mark.parametrize("B,D,H,W,K,N", [(1, 2, 4, 8, 16, 32), (2, 4, 6, 16, 64, 32), (2, 4, 2, 12, 32, 16),
-                                         (1, 6, 10, 24, 96, 64)])
+                                         (1, 6, 10, 24, 96, 64), (1, 4, 6, 2, 64, 32),
+                                         (1, 2, 4, 10, 48, 32)])
 def test_fused_convolution_equals_separate_calls(mp, B, D, H, W, K, N):
     g = torch.Generator(device="cuda")
     g.manual_seed(K + N)
