@@ -307,7 +307,7 @@ void mp_release_cached(void);
  *
  *  nx, ny, nz    lattice (each >= 3); N = nx*ny*nz must not exceed 2,097,152 nodes: the
  *                step's FP64 reduction uses a fixed scratch array of 8192 block partials
- *                (64 KiB plus a counter, a __device__ array that every GPU using this entry
+ *                (64 KiB, a __device__ array that every GPU using this entry
  *                point keeps until the library is unloaded). Larger N returns MP_EINVAL.
  *  solid         device, N bytes, nonzero = solid.
  *  u             device, FP32 3*N SoA, or NULL (rest).
@@ -325,7 +325,7 @@ void mp_release_cached(void);
  * current) and remembers it with the id of the device's context; make that first call before
  * any stream capture. After a cudaDeviceReset the next call finds a new context and looks the
  * address up again (so it is again a first call). Every call shares the
- * one scratch array and leaves its contents behind: the counter is cleared by each call, so
+ * one scratch array and leaves its contents behind, so
  * calls that overlap on the GPU (different streams, concurrent host threads) race and must
  * be serialised by the caller.
  * Errors: MP_EINVAL, MP_ECUDA.

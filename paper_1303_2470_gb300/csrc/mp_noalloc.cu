@@ -4,130 +4,168 @@
 // its own pool, where a stray cudaMalloc would fail or break its accounting), or code that
 // must not trigger the implicit device synchronisation of cudaMalloc / cudaFree.
 //
-// The only scratch the step needs -- the per-block partial sums of its FP64 reduction and a
-// completion counter -- lives in a file-scope __device__ array of fixed size. Every GPU that
-// runs this entry point keeps that array until the library is unloaded.
+// The only scratch the step needs -- the per-block partial sums of its FP64 reduction -- lives
+// in a file-scope __device__ array of fixed size. Every GPU that runs this entry point keeps
+// that array until the library is unloaded.
 #include <mutex>
 
 #include "internal.cuh"
+#include "lattice.cuh"
 #include "link_arith.cuh"
 
 using namespace mp;
 
 namespace {
 
-constexpr int kNaThreads = 256;
-constexpr int kNaWarps = kNaThreads / 32;
-constexpr int kNaMaxBlocks = 8192;  // one thread per node: at most 2,097,152 nodes per call
-constexpr long long kNaMaxNodes = (long long)kNaThreads * kNaMaxBlocks;
-constexpr size_t kNaTicketOffset = kNaMaxBlocks * sizeof(double);
+constexpr int kNaThreads = 128;
+constexpr int kNaNodes = 256;       // nodes per block
+constexpr int kNaMaxBlocks = 8192;  // at most 2,097,152 nodes per call
+constexpr long long kNaMaxNodes = (long long)kNaNodes * kNaMaxBlocks;
 
-// [0, kNaTicketOffset): one FP64 partial sum per block; then the completion counter.
-static __device__ __align__(256) unsigned char g_noalloc_scratch[kNaTicketOffset + 256];
+// one FP64 partial sum per block
+static __device__ __align__(256) unsigned char g_noalloc_scratch[kNaMaxBlocks * sizeof(double)];
 
 struct NaArgs {
     int nx, ny, nz, N;
     int g;  // direction of the velocity weight of the sum, -1 for the plain sum
     float hl, pa, pd;
+    Div dx, dxy;  // division by nx and by nx*ny
 };
-
-__device__ __forceinline__ int na_wrap(int v, int n) { return v < 0 ? v + n : (v >= n ? v - n : v); }
 
 // Same update as the library's step kernel, read from dense arrays: X(r) + sum of net link
 // fluxes, then the sorption exchange on interfacial nodes (paper Sec. "Algorithm",
 // Eqs. propagated_quantity, Pads, newP), and sum_r X'(r) u*_g(r) in FP64.
-__global__ void __launch_bounds__(kNaThreads)
-    k_step_noalloc(const NaArgs a, const uint8_t* __restrict__ solid, const float* __restrict__ u,
+// Everything is recomputed from the mask and the flow, about a thousand instructions a fluid
+// node, and issuing them is what bounds it: in a porous medium most lanes of a warp of
+// consecutive nodes are solid. So a block packs the fluid nodes of its 256 onto its 128 threads
+// (in one or two rounds), with 64 registers and no branch around a link, so that the loads of
+// several links are in flight; the sums are taken over the nodes in their own order all the
+// same. A call on 64^3 spheres (porosity 0.4) takes 14.3 us (one thread a node, a branch a link:
+// 20.8), on 127^3 51 us (93).
+template <bool kFlow>
+__global__ void __launch_bounds__(kNaThreads, 8)
+    k_step_noalloc(const __grid_constant__ NaArgs a, const uint8_t* __restrict__ solid, const float* __restrict__ u,
                    const float* __restrict__ X, const float* __restrict__ Xa, float* __restrict__ Xn,
-                   float* __restrict__ Xan, double* __restrict__ z_out, unsigned char* __restrict__ scratch)
+                   float* __restrict__ Xan, unsigned char* __restrict__ scratch)
 {
     double* partials = reinterpret_cast<double*>(scratch);
-    unsigned int* ticket = reinterpret_cast<unsigned int*>(scratch + kNaTicketOffset);
-    const int n = blockIdx.x * kNaThreads + threadIdx.x;
-    float zp = 0.0f;
-    if (n < a.N) {
-        if (solid[n]) {
+    cudaTriggerProgrammaticLaunchCompletion();
+    constexpr int kRounds = kNaNodes / kNaThreads;
+    __shared__ float s_z[kNaNodes];
+    __shared__ unsigned char s_list[kNaNodes];  // the block's fluid nodes, ascending
+    __shared__ int s_count[kNaNodes / 32];
+    const int base = blockIdx.x * kNaNodes;
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    bool fl[kRounds];
+    uint32_t bits[kRounds];
+#pragma unroll
+    for (int r = 0; r < kRounds; ++r) {
+        const int l = r * kNaThreads + threadIdx.x, n = base + l;
+        fl[r] = n < a.N && solid[n] == 0;
+        bits[r] = __ballot_sync(0xffffffffu, fl[r]);
+        if (lane == 0) s_count[r * (kNaThreads / 32) + warp] = __popc(bits[r]);
+        s_z[l] = 0.0f;
+        if (n < a.N && !fl[r]) {
             Xn[n] = 0.0f;
             Xan[n] = 0.0f;
-        } else {
-            const int x = n % a.nx, y = (n / a.nx) % a.ny, z = n / (a.nx * a.ny);
-            float ux = 0.f, uy = 0.f, uz = 0.f;
-            if (u) {
-                ux = u[n];
-                uy = u[a.N + n];
-                uz = u[2 * a.N + n];
-            }
-            const float ar = rn_mul(-1.5f, rn_add(rn_add(rn_mul(ux, ux), rn_mul(uy, uy)), rn_mul(uz, uz)));
-            const float whl_face = rn_mul(weight<float>(1), a.hl), whl_edge = rn_mul(weight<float>(5), a.hl);
-            const float xr = X[n];
-            float delta = 0.0f, us = 0.0f;
-            bool itf = false;
+        }
+    }
+    __syncthreads();
+    int total = 0;
 #pragma unroll
-            for (int i = 1; i < kQ; ++i) {
-                const int s = na_wrap(x - cx(i), a.nx) +
-                              a.nx * (na_wrap(y - cy(i), a.ny) + a.ny * na_wrap(z - cz(i), a.nz));
-                if (solid[s]) {
-                    itf = true;
-                    continue;
-                }
+    for (int w = 0; w < kNaNodes / 32; ++w) total += s_count[w];
+#pragma unroll
+    for (int r = 0; r < kRounds; ++r) {
+        int before = 0;
+        for (int w = 0; w < r * (kNaThreads / 32) + warp; ++w) before += s_count[w];
+        if (fl[r]) s_list[before + __popc(bits[r] & ((1u << lane) - 1u))] = (unsigned char)(r * kNaThreads + threadIdx.x);
+    }
+    __syncthreads();
+    for (int j = threadIdx.x; j < total; j += kNaThreads) {
+        const int l = s_list[j], n = base + l;
+        const Nbr b = nbrs_of(a.nx, a.ny, a.nz, a.dx, a.dxy, n);
+        float ux = 0.f, uy = 0.f, uz = 0.f;
+        if (kFlow) {
+            ux = u[n];
+            uy = u[a.N + n];
+            uz = u[2 * a.N + n];
+        }
+        const float ar = rn_mul(-1.5f, rn_add(rn_add(rn_mul(ux, ux), rn_mul(uy, uy)), rn_mul(uz, uz)));
+        const float whl_face = rn_mul(weight<float>(1), a.hl), whl_edge = rn_mul(weight<float>(5), a.hl);
+        const float xr = X[n];
+        float delta = 0.0f, us = 0.0f;
+        uint32_t mask = 0;
+#pragma unroll
+        for (int i = 1; i < kQ; ++i) mask |= (__ldg(solid + src_of(b, i)) == 0 ? 1u : 0u) << (i - 1);
+#pragma unroll
+        for (int i = 1; i < kQ; ++i) {
+            const int s = src_of(b, i);
+            const bool open = (mask >> (i - 1)) & 1u;
                 float sx = 0.f, sy = 0.f, sz = 0.f;
-                if (u) {
-                    sx = u[s];
-                    sy = u[a.N + s];
-                    sz = u[2 * a.N + s];
+                if (kFlow) {
+                    sx = (open ? __ldg(u + s) : 0.0f);
+                    sy = (open ? __ldg(u + a.N + s) : 0.0f);
+                    sz = (open ? __ldg(u + 2 * a.N + s) : 0.0f);
                 }
+                const float xs = (open ? __ldg(X + s) : 0.0f);
                 const float as = rn_mul(-1.5f, rn_add(rn_add(rn_mul(sx, sx), rn_mul(sy, sy)), rn_mul(sz, sz)));
                 const float whl = is_face(i) ? whl_face : whl_edge;
                 const float pin = rn_fma(weight<float>(i), qlink(edot<float>(i, sx, sy, sz), as), whl);
                 const float pout = rn_fma(weight<float>(i), qlink(edot<float>(opposite(i), ux, uy, uz), ar), whl);
-                delta = rn_add(delta, rn_sub(rn_mul(pin, X[s]), rn_mul(pout, xr)));
+                const float d = rn_add(delta, rn_sub(rn_mul(pin, xs), rn_mul(pout, xr)));
+                delta = open ? d : delta;
                 if (a.g >= 0) {
                     const int c = ci(opposite(i), a.g);
-                    if (c != 0) us += float(c) * pout;
+                    if (c != 0) us += open ? float(c) * pout : 0.0f;
                 }
-            }
-            if (itf) {
-                const float xa = Xa[n];
-                const float js = rn_sub(rn_mul(a.pa, xr), rn_mul(a.pd, xa));
-                delta = rn_sub(delta, js);
-                Xan[n] = rn_add(xa, js);
-            } else {
-                Xan[n] = 0.0f;
-            }
-            const float xn = rn_add(xr, delta);
-            Xn[n] = xn;
-            zp = a.g >= 0 ? xn * us : xn;
         }
+        if (mask != (1u << (kQ - 1)) - 1u) {
+            const float xa = Xa[n];
+            const float js = rn_sub(rn_mul(a.pa, xr), rn_mul(a.pd, xa));
+            delta = rn_sub(delta, js);
+            Xan[n] = rn_add(xa, js);
+        } else {
+            Xan[n] = 0.0f;
+        }
+        const float xn = rn_add(xr, delta);
+        Xn[n] = xn;
+        s_z[l] = a.g >= 0 ? xn * us : xn;
     }
-    // FP32 within the warp, FP64 across warps and blocks, in a fixed order
-    __shared__ double s_red[kNaWarps];
-    __shared__ unsigned int s_last;
+    __syncthreads();
+    // FP32 within 32 consecutive nodes, FP64 across them and blocks, in a fixed order
+    __shared__ double s_red[kNaNodes / 32];
 #pragma unroll
-    for (int o = 16; o > 0; o >>= 1) zp += __shfl_xor_sync(0xffffffffu, zp, o);
-    if ((threadIdx.x & 31) == 0) s_red[threadIdx.x >> 5] = (double)zp;
+    for (int r = 0; r < kRounds; ++r) {
+        float zp = s_z[r * kNaThreads + threadIdx.x];
+#pragma unroll
+        for (int o = 16; o > 0; o >>= 1) zp += __shfl_xor_sync(0xffffffffu, zp, o);
+        if (lane == 0) s_red[r * (kNaThreads / 32) + warp] = (double)zp;
+    }
     __syncthreads();
     if (threadIdx.x == 0) {
         double t = 0.0;
-        for (int w = 0; w < kNaWarps; ++w) t += s_red[w];
+        for (int w = 0; w < kNaNodes / 32; ++w) t += s_red[w];
         partials[blockIdx.x] = t;
-        __threadfence();
-        s_last = (atomicAdd(ticket, 1u) == gridDim.x - 1) ? 1u : 0u;
     }
-    __syncthreads();
-    if (!s_last) return;
-    __threadfence();
+}
+
+// The sum of the block partials, in a fixed order. A launch of its own (programmatic dependent
+// launch: resident by the time the step ends) in place of a completion counter, which had to be
+// cleared by a launch before the step and made its last block work alone.
+__global__ void __launch_bounds__(256) k_sum_noalloc(const double* __restrict__ partials, int blocks,
+                                                     double* __restrict__ z_out)
+{
+    __shared__ double s_w[8];
+    cudaGridDependencySynchronize();
     double v = 0.0;
-    for (int b = threadIdx.x; b < (int)gridDim.x; b += kNaThreads) v += __ldcg(partials + b);
-#pragma unroll
-    for (int o = 16; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
-    __syncthreads();
-    if ((threadIdx.x & 31) == 0) s_red[threadIdx.x >> 5] = v;
+    for (int b = threadIdx.x; b < blocks; b += 256) v += __ldcg(partials + b);
+    v = warp_sum(v);
+    if ((threadIdx.x & 31) == 0) s_w[threadIdx.x >> 5] = v;
     __syncthreads();
     if (threadIdx.x == 0) {
         double t = 0.0;
-        for (int w = 0; w < kNaWarps; ++w) t += s_red[w];
+        for (int w = 0; w < 8; ++w) t += s_w[w];
         *z_out = t;
-        *ticket = 0u;
     }
 }
 
@@ -219,8 +257,6 @@ extern "C" int mp_step_noalloc(int nx, int ny, int nz, const uint8_t* solid, con
     int rc = scratch_address(&scratch);
     if (rc != MP_OK) return rc;
     cudaStream_t s = (cudaStream_t)stream;
-    // the completion counter must start at zero (the previous call may have been cut short)
-    MP_CUDA(cudaMemsetAsync(scratch + kNaTicketOffset, 0, sizeof(unsigned int), s));
     NaArgs a;
     a.nx = nx;
     a.ny = ny;
@@ -230,8 +266,12 @@ extern "C" int mp_step_noalloc(int nx, int ny, int nz, const uint8_t* solid, con
     a.hl = (float)(6.0 * D_b);  // lambda/2 = 12 D_b / 2
     a.pa = (float)k_a;
     a.pd = (float)k_d;
-    const int blocks = (int)((N + kNaThreads - 1) / kNaThreads);
-    k_step_noalloc<<<blocks, kNaThreads, 0, s>>>(a, solid, u, X, X_ads, X_out, X_ads_out, Z_out, scratch);
+    const int blocks = (int)((N + kNaNodes - 1) / kNaNodes);
+    a.dx = make_div((unsigned)nx);
+    a.dxy = make_div((unsigned)(nx * ny));
+    auto kern = u ? k_step_noalloc<true> : k_step_noalloc<false>;
+    kern<<<blocks, kNaThreads, 0, s>>>(a, solid, u, X, X_ads, X_out, X_ads_out, scratch);
     MP_CUDA(cudaGetLastError());
+    MP_CUDA(launch_pdl(k_sum_noalloc, dim3(1), dim3(256), s, (const double*)scratch, blocks, Z_out));
     return MP_OK;
 }

@@ -10,6 +10,7 @@ from __future__ import annotations
 
 import ctypes
 import os
+import sys
 
 import numpy as np
 
@@ -374,6 +375,29 @@ def _device_of(buf):
     return str(getattr(buf, "device", "?"))
 
 
+def _noalloc_device(torch, solid, u, *fields):
+    """The device index of mp_step_noalloc's buffers when each is a tensor of the documented
+    layout on one device, else None (the checks that name what is wrong follow). One pass of
+    cheap tests: the step of a small lattice takes less time than the full checks."""
+    tensor, f32 = torch.Tensor, torch.float32
+    if not (isinstance(solid, tensor) and solid.is_cuda and solid.dim() == 3
+            and (solid.dtype is torch.uint8 or solid.dtype is torch.bool) and solid.is_contiguous()):
+        return None
+    n, index = solid.numel(), solid.get_device()
+    if u is not None and not (isinstance(u, tensor) and u.is_cuda and u.dtype is f32 and u.is_contiguous()
+                              and u.numel() >= 3 * n and u.get_device() == index):
+        return None
+    for t in fields[:-1]:
+        if not (isinstance(t, tensor) and t.is_cuda and t.dtype is f32 and t.is_contiguous() and t.numel() >= n
+                and t.get_device() == index):
+            return None
+    z = fields[-1]
+    if not (isinstance(z, tensor) and z.is_cuda and z.dtype is torch.float64 and z.numel() >= 1
+            and z.get_device() == index):
+        return None
+    return index
+
+
 def mp_step_noalloc(solid, u, D_b, k_a, k_d, direction, X, X_ads, X_out, X_ads_out, Z_out,
                     stream=None):
     """mp_step_noalloc of include/mp.h: one step of one field on caller-owned device arrays
@@ -381,6 +405,15 @@ def mp_step_noalloc(solid, u, D_b, k_a, k_d, direction, X, X_ads, X_out, X_ads_o
     nx) or None; X, X_ads, X_out, X_ads_out: FP32 (nz, ny, nx); Z_out: one FP64 element.
     Every tensor is checked against that layout (CUDA, dtype, contiguity, size, one device)
     before the call, which then runs with that device current."""
+    torch = sys.modules.get("torch")
+    if torch is not None:
+        index = _noalloc_device(torch, solid, u, X, X_ads, X_out, X_ads_out, Z_out)
+        if index is not None and index == torch.cuda.current_device():
+            nz, ny, nx = solid.shape
+            _check(_lib.mp_step_noalloc(nx, ny, nz, solid.data_ptr(), None if u is None else u.data_ptr(), D_b, k_a,
+                                        k_d, direction, X.data_ptr(), X_ads.data_ptr(), X_out.data_ptr(),
+                                        X_ads_out.data_ptr(), Z_out.data_ptr(), _stream(stream)))
+            return
     if not (hasattr(solid, "data_ptr") and getattr(solid, "is_cuda", False) and len(solid.shape) == 3
             and str(solid.dtype) in ("torch.uint8", "torch.bool") and solid.is_contiguous()):
         raise MPBufferError(f"solid: needs a contiguous CUDA uint8 tensor (nz, ny, nx), got "
