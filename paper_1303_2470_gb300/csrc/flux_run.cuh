@@ -1,0 +1,58 @@
+// flux_run.cuh -- how the flux steps of one context are launched (not part of the C ABI): one
+// launch per step and one that closes a run, runs of kFluxGraph steps replayed from a CUDA graph
+// captured once per starting buffer on streams that can be captured.
+#pragma once
+
+#include "internal.cuh"
+#include "mp_ctx.cuh"
+
+namespace mp {
+
+constexpr int kFluxGraph = 64;  // even: a replay ends on the buffer it started from
+
+// launch(pending): the step from buffer c->cur; pending: the previous launch was a step whose
+// series is not appended yet. finish(parity): appends the series of the last step, which read
+// buffer `parity`.
+template <typename Launch, typename Finish>
+int run_flux(mp_ctx* c, long long n, Launch launch, Finish finish)
+{
+    cudaError_t le = cudaSuccess;  // first failed launch, if any
+    auto run = [&](long long count) {
+        for (long long k = 0; k < count; ++k) {
+            const cudaError_t e = launch(k > 0 ? 1 : 0);
+            if (e != cudaSuccess && le == cudaSuccess) le = e;
+            c->cur = 1 - c->cur;
+        }
+        if (count > 0) {
+            const cudaError_t e = finish(1 - c->cur);
+            if (e != cudaSuccess && le == cudaSuccess) le = e;
+        }
+    };
+    const bool capturable =
+        c->stream != nullptr && c->stream != cudaStreamLegacy && c->stream != cudaStreamPerThread;
+    if (capturable && n >= 2 * kFluxGraph) {
+        const int b = c->cur;
+        if (!c->exec[b]) {
+            cudaError_t e = cudaStreamBeginCapture(c->stream, cudaStreamCaptureModeThreadLocal);
+            if (e == cudaSuccess) {
+                run(kFluxGraph);
+                e = cudaStreamEndCapture(c->stream, &c->graph[b]);
+            }
+            c->cur = b;
+            if (e == cudaSuccess && le != cudaSuccess) e = le;
+            if (e == cudaSuccess) e = cudaGraphInstantiate(&c->exec[b], c->graph[b], 0);
+            if (e != cudaSuccess) return cuda_fail(e, "mp_step: graph capture");
+        }
+        for (; n >= kFluxGraph; n -= kFluxGraph) {
+            MP_CUDA(cudaGraphLaunch(c->exec[b], c->stream));
+            c->t += kFluxGraph;
+        }
+    }
+    run(n);
+    c->t += n;
+    if (le != cudaSuccess) return cuda_fail(le, "mp_step: launch");
+    MP_CUDA(cudaGetLastError());
+    return MP_OK;
+}
+
+}  // namespace mp

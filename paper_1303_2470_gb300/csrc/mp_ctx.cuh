@@ -15,6 +15,7 @@ struct mp_group;
 namespace mp {
 struct DirectTables;
 struct DirectState;
+struct Flux32;
 struct Flux64;
 }  // namespace mp
 
@@ -61,6 +62,10 @@ struct mp_ctx {
     mp::DirectState* dstate = nullptr;
     // FP64 flux contexts: link tables of the tabulated step (NULL: terms recomputed)
     mp::Flux64* flux64 = nullptr;
+    // FP32 and FP16 flux contexts stepped on their own; series_moved: a group (or mp_init) has moved
+    // the series position since their last step
+    mp::Flux32* flux32 = nullptr;
+    bool series_moved = false;
 };
 
 namespace mp {
@@ -80,6 +85,12 @@ void direct_free(mp_ctx* c);
 int flux64_setup(mp_ctx* c);
 int flux64_step(mp_ctx* c, long long n);
 void flux64_free(mp_ctx* c);
+
+// The flux step of one FP32 or FP16 context (mp_flux32.cu): tables after the fields are
+// initialised, n steps, release.
+int flux32_setup(mp_ctx* c);
+int flux32_step(mp_ctx* c, long long n);
+void flux32_free(mp_ctx* c);
 
 // A set of direct-scheme contexts stepped together (groups): created over n contexts, run on
 // `stream`, stepped n steps; variant and block size are autotuned when `tune` is nonzero.

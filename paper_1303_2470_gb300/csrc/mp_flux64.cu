@@ -26,6 +26,7 @@
 #include <cstring>
 #include <string>
 
+#include "flux_run.cuh"
 #include "internal.cuh"
 #include "lattice.cuh"
 #include "link_arith.cuh"
@@ -81,7 +82,6 @@ constexpr uint32_t face_links()
     return m;
 }
 constexpr uint32_t kFaceLinks = face_links();
-constexpr int kFlux64Graph = 64;                    // steps per captured graph (even)
 
 // series of the step whose partials have parity `parity`: warp w adds series w, w + warps, ...
 // over the blocks (FP64, fixed order) and appends Z and D at t + 1
@@ -392,48 +392,11 @@ int flux64_setup(mp_ctx* c)
     return MP_OK;
 }
 
-// n steps: one launch per step and one that appends the last step's series; runs of
-// kFlux64Graph replayed from a graph (captured once per starting buffer) where the stream can
-// be captured.
 int flux64_step(mp_ctx* c, long long n)
 {
-    cudaError_t le = cudaSuccess;
-    auto run = [&](long long count) {
-        for (long long k = 0; k < count; ++k) {
-            const cudaError_t e = launch64(c, k > 0 ? 1 : 0);
-            if (e != cudaSuccess && le == cudaSuccess) le = e;
-            c->cur = 1 - c->cur;
-        }
-        if (count > 0) {
-            const cudaError_t e = launch_pdl(k_finish64, dim3(1), dim3(256), c->stream, c->flux64->a, 1 - c->cur);
-            if (e != cudaSuccess && le == cudaSuccess) le = e;
-        }
-    };
-    const bool capturable =
-        c->stream != nullptr && c->stream != cudaStreamLegacy && c->stream != cudaStreamPerThread;
-    if (capturable && n >= 2 * kFlux64Graph) {
-        const int b = c->cur;
-        if (!c->exec[b]) {
-            cudaError_t e = cudaStreamBeginCapture(c->stream, cudaStreamCaptureModeThreadLocal);
-            if (e == cudaSuccess) {
-                run(kFlux64Graph);
-                e = cudaStreamEndCapture(c->stream, &c->graph[b]);
-            }
-            c->cur = b;
-            if (e == cudaSuccess && le != cudaSuccess) e = le;
-            if (e == cudaSuccess) e = cudaGraphInstantiate(&c->exec[b], c->graph[b], 0);
-            if (e != cudaSuccess) return cuda_fail(e, "mp_step: graph capture");
-        }
-        for (; n >= kFlux64Graph; n -= kFlux64Graph) {
-            MP_CUDA(cudaGraphLaunch(c->exec[b], c->stream));
-            c->t += kFlux64Graph;
-        }
-    }
-    run(n);
-    c->t += n;
-    if (le != cudaSuccess) return cuda_fail(le, "mp_step: launch");
-    MP_CUDA(cudaGetLastError());
-    return MP_OK;
+    return run_flux(
+        c, n, [&](int pending) { return launch64(c, pending); },
+        [&](int parity) { return launch_pdl(k_finish64, dim3(1), dim3(256), c->stream, c->flux64->a, parity); });
 }
 
 }  // namespace mp
