@@ -99,6 +99,16 @@ __device__ __forceinline__ void pdl_enter()
     cudaGridDependencySynchronize();
 }
 
+// Pointer to data that the previous grid writes, for use after cudaGridDependencySynchronize():
+// loads through it cannot be moved above the wait (an address that is known earlier, a
+// __restrict__ parameter or a non-volatile load instruction would allow it).
+template <typename T>
+__device__ __forceinline__ T* after_wait(T* p)
+{
+    asm volatile("" : "+l"(p) : : "memory");
+    return p;
+}
+
 // Error reporting: the thread-local last-error text behind mp_last_error().
 void set_error(const std::string& msg);
 void clear_error();

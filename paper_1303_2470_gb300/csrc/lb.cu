@@ -98,8 +98,8 @@ __device__ __forceinline__ bool lb_bit(const uint32_t* __restrict__ w, int n)
 // beyond 2^32 elements (a source's plane is then found at its load).
 template <bool kRows, bool kWide, int kB, int kMinBlocks>
 __global__ void __launch_bounds__(kB, kMinBlocks)
-    k_lb_step(const __grid_constant__ LbArgs a, const float* __restrict__ g, float* __restrict__ gn, int mode,
-              float* __restrict__ u_prev, float* __restrict__ u_out, float* __restrict__ rho_out,
+    k_lb_step(const __grid_constant__ LbArgs a, const float* g_in, float* __restrict__ gn, int mode, float* u_prev_in,
+              float* __restrict__ u_out, float* __restrict__ rho_out,
               unsigned long long* __restrict__ res_key)
 {
     cudaTriggerProgrammaticLaunchCompletion();
@@ -155,6 +155,8 @@ __global__ void __launch_bounds__(kB, kMinBlocks)
         }
     }
     cudaGridDependencySynchronize();  // the previous step's populations and residual are visible
+    const float* g = after_wait(g_in);
+    float* u_prev = after_wait(u_prev_in);
     if (active) {
         float f[kQ];
 #pragma unroll

@@ -110,8 +110,8 @@ constexpr int kB = 256, kSingleBlocks = 6, kMultiBlocks = 3;
 // of species per pass of the link loop (0: one species)
 template <typename TS, int FP, int kCP>
 __global__ void __launch_bounds__(kB, kCP == 0 ? kSingleBlocks : kMultiBlocks)
-    k_step32(const __grid_constant__ F32Args a, const TS* __restrict__ P, TS* __restrict__ Pn, const TS* __restrict__ A,
-             TS* __restrict__ An, int parity, int pending)
+    k_step32(const __grid_constant__ F32Args a, const TS* P_in, TS* __restrict__ Pn, const TS* A_in, TS* __restrict__ An,
+             int parity, int pending)
 {
     cudaTriggerProgrammaticLaunchCompletion();
     if ((int)blockIdx.x < a.napp) {
@@ -134,6 +134,8 @@ __global__ void __launch_bounds__(kB, kCP == 0 ? kSingleBlocks : kMultiBlocks)
         ur = a.u4[n];
     }
     cudaGridDependencySynchronize();  // the previous step's fields, series and counts are visible
+    const TS* P = after_wait(P_in);
+    const TS* A = after_wait(A_in);
     // binary16 storage: rounding keys from the time index after this step, then array and element
     uint32_t tkey = 0;
     if constexpr (!std::is_same<float, TS>::value)
@@ -202,9 +204,9 @@ __global__ void __launch_bounds__(kB, kCP == 0 ? kSingleBlocks : kMultiBlocks)
         constexpr int kMaxPass = kCP == 1 ? 1 : MP_MAX_SPECIES / (kCP * kSC);  // kCP 1: one chunk in all
         using VC = FieldVec<float, 8>;
         using VCS = FieldVec<TS, 8>;
-        const VCS* __restrict__ Pc = reinterpret_cast<const VCS*>(P);
+        const VCS* Pc = reinterpret_cast<const VCS*>(P);
         VCS* __restrict__ Pnc = reinterpret_cast<VCS*>(Pn);
-        const VCS* __restrict__ Ac = reinterpret_cast<const VCS*>(A);
+        const VCS* Ac = reinterpret_cast<const VCS*>(A);
         VCS* __restrict__ Anc = reinterpret_cast<VCS*>(An);
 #pragma unroll
         for (int pass = 0; pass < kMaxPass; ++pass) {

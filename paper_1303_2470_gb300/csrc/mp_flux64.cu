@@ -124,8 +124,8 @@ __device__ __forceinline__ void st_rec64(double* p, const double (&v)[FP])
 // block (x, y): nodes x kB/kLanes .. of species y; block (nblk, 0) appends the previous step
 template <int FP, bool kSingle, int kLanes, int kB>
 __global__ void __launch_bounds__(kB)
-    k_step64(const __grid_constant__ F64Args a, const double* __restrict__ P, double* __restrict__ Pn,
-             const double* __restrict__ A, double* __restrict__ An, int parity, int pending)
+    k_step64(const __grid_constant__ F64Args a, const double* P, double* Pn, const double* A_in, double* An, int parity,
+             int pending)
 {
     cudaTriggerProgrammaticLaunchCompletion();
     const int sp = (int)blockIdx.y;
@@ -167,7 +167,6 @@ __global__ void __launch_bounds__(kB)
     const size_t stride = kSingle ? FP : (size_t)a.SC * FP;
     const size_t off = kSingle ? 0 : (size_t)(sp % a.SC) * FP;
     const size_t base = kSingle ? 0 : (size_t)(sp / a.SC) * a.N * stride + off;
-    const double* Ps = P + base;
     if constexpr (!kSingle) {
         const double whf = a.whf[sp], whe = a.whe[sp];
 #pragma unroll
@@ -181,6 +180,8 @@ __global__ void __launch_bounds__(kB)
         }
     }
     cudaGridDependencySynchronize();  // the previous step's fields and series are visible
+    const double* Ps = after_wait(P) + base;
+    const double* A = after_wait(A_in);
     double xr[FP], delta[FP];
 #pragma unroll
     for (int f = 0; f < FP; ++f) xr[f] = delta[f] = 0.0;
