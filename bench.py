@@ -98,10 +98,10 @@ TRAFFIC = {
 }
 
 
-# One-off kernels of one job on this medium, counted in an ncu launch list of the job:
-# geometry preparation for the LB and for the MP, cluster labelling (24 sweeps on this
-# medium), and the LB and MP initialisation.
-JOB_FIXED_LAUNCHES = 42
+# One-off kernels of one job, counted in an ncu launch list of the job's calls: geometry
+# preparation for the LB and for the MP (6 each), cluster labelling (5), and the LB and MP
+# initialisation (3 and 4); their number does not depend on the medium.
+JOB_FIXED_LAUNCHES = 24
 
 
 def _src_sha(name):
@@ -235,15 +235,15 @@ def run_hbm_probe(mp, peak, peak_kind, scheme_opts):
 
 
 def mp_kernel_launches(variant, steps, tuned):
-    """Kernels of mp_step(steps) and of the direct scheme's set-up: the flux scheme launches one
-    kernel per step; the direct scheme one per step plus one that appends the last step's
-    series per run (graphs of 64 steps are runs), or one persistent launch; its set-up adds
-    the table kernel and, when tuned, 20 + 2 steps of each of the six one-step candidates (with
-    their closing launches) and two launches of each of the six persistent ones."""
+    """Kernels of mp_step(steps) and of the scheme's set-up: one launch per step plus one that
+    appends the last step's series per run (graphs of 64 steps are runs), or one persistent
+    launch. The set-up adds the table kernel; the direct scheme's, when tuned, 20 + 2 steps of
+    each of the six one-step candidates (with their closing launches and the one that sets
+    their counts) and two launches of each of the six persistent ones."""
     if variant == "flux":
-        return steps
+        return steps + -(-steps // 64) + 1
     run = 1 if variant.startswith("persistent") else steps + -(-steps // 64)
-    return run + 1 + (6 * (22 + 2) + 6 * 2 if tuned else 0)
+    return run + 1 + (6 * (22 + 3) + 6 * 2 if tuned else 0)
 
 
 def make_medium():

@@ -62,9 +62,10 @@ struct mp_ctx {
     mp::DirectState* dstate = nullptr;
     // FP64 flux contexts: link tables of the tabulated step (NULL: terms recomputed)
     mp::Flux64* flux64 = nullptr;
-    // FP32 and FP16 flux contexts stepped on their own; series_moved: a group (or mp_init) has moved
-    // the series position since their last step
+    // FP32 and FP16 flux contexts stepped on their own
     mp::Flux32* flux32 = nullptr;
+    // the series position has been moved by launches that do not keep the counts by which the
+    // one-step launches (flux32, direct) find it: they are to be set before the next run
     bool series_moved = false;
 };
 

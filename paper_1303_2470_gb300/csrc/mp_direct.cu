@@ -14,7 +14,7 @@
 // (mp.cu). One species keeps dense fields: links into solid nodes meet zero fields (solid
 // entries are never written), so that inflow needs no open-link test. Several species keep
 // their fields for the fluid nodes only and locate each open link's source in the fluid list
-// (lattice.cuh); closed links are skipped. A variant recomputes q_i from the flow vector of
+// (lattice.cuh); a closed link adds 0 x (table) or is skipped (recomputed). A variant recomputes q_i from the flow vector of
 // the source instead of reading the table (less memory traffic, more arithmetic), and for
 // several species a tiled variant stages planes of the medium in shared memory.
 //
@@ -28,10 +28,14 @@
 // gives up sets an error flag that the host reports as MP_ETIMEOUT). Several contexts
 // (media of any size, each with its own species) can share one launch: work is cut into
 // virtual blocks of `block` fluid nodes, numbered context after context.
+// One launch per step is the faster form on every medium measured (one species, table, us a step,
+// before -> now: 32^3 3.7 -> 2.4, 128^3 20.3 -> 18.5, 256^3 167 -> 160; four species: 160^3
+// 136 -> 105, 256^3 530 -> 415; persistent, one species: 20.5 at 128^3, 164 at 256^3).
 #include <algorithm>
 #include <climits>
 #include <cstring>
 #include <string>
+#include <type_traits>
 #include <vector>
 
 #include "internal.cuh"
@@ -53,6 +57,7 @@ struct DirectTables {
     uint2* fw = nullptr;
     uint2* iw = nullptr;  // {interface bits, interfacial nodes before the word} per word
     Flow4<float>* uc = nullptr;
+    long long* count = nullptr;  // [2], see DArgs
 };
 
 namespace {
@@ -73,9 +78,6 @@ constexpr long long kWaitNs = 2000000000LL;   // a grid barrier wait gives up af
 #endif
 #ifndef MP_DIRECT_MULTI_THREADS
 #define MP_DIRECT_MULTI_THREADS 1024
-#endif
-#ifndef MP_DIRECT_CP
-#define MP_DIRECT_CP 1
 #endif
 
 struct DArgs {
@@ -98,7 +100,13 @@ struct DArgs {
     float* P[2];
     float* A[2];
     float whf[MP_MAX_SPECIES], whe[MP_MAX_SPECIES], pa[MP_MAX_SPECIES], pd[MP_MAX_SPECIES];
-    double* part;  // [2][slots][K] partial sums of the K = S*M series, by step parity
+    // partial sums of the K = S*M series, by step parity: [2][slots][K] (persistent and tiled
+    // launches), or one per warp of work items, [2][K][nw] (one launch per step)
+    double* part;
+    int nw, napp;  // one launch per step: warps of work items, blocks that append the series
+    // time index of the last appended step that read buffer 0 and 1. A step that reads buffer b
+    // ends at time count[b] + 2; count[b] is written by the launch before it, never by its own.
+    long long* count;
     double* Z;
     double* D;
     long long* tdev;
@@ -108,7 +116,17 @@ struct DArgs {
 struct DLaunch {
     const DArgs* args;          // [n], device
     int vbofs[kMaxCtx + 1];     // virtual-block prefix over the contexts
+    int apofs[kMaxCtx + 1];     // the same of the appending blocks (one launch per step)
     int n;
+};
+
+// One-step launches carry the arguments of their contexts by value: pointers, sizes and species
+// constants then come from the constant bank as operands, neither loaded from global memory at the
+// start of every block nor held in registers or shared memory (4 species, 160^3: 123 -> 100 us a step)
+template <int kN>
+struct DStepArgs {
+    DLaunch L;
+    DArgs a[kN];
 };
 
 // Link table layout: the 18 values of 32 consecutive work items are stored together, link
@@ -119,8 +137,9 @@ __host__ __device__ __forceinline__ size_t tab_at(int k, int i)
     return ((size_t)(k >> 5) * 18 + (size_t)(i - 1)) * 32 + (size_t)(k & 31);
 }
 
-// ---- field loads: read-only (non-coherent path) inside a one-step launch; plain loads in
-// the persistent kernel, where the fields read in a step were written earlier in the launch
+// ---- field loads: inside a one-step launch the fields don't change after its wait (pointers
+// through after_wait), so the loads may be reordered; in the persistent kernel the fields read in
+// a step were written earlier in the launch
 template <bool kCoherent, int W>
 __device__ __forceinline__ FieldVec<float, W> ld_field(const FieldVec<float, W>* p)
 {
@@ -129,7 +148,7 @@ __device__ __forceinline__ FieldVec<float, W> ld_field(const FieldVec<float, W>*
         if constexpr (kCoherent)
             asm volatile("ld.global.v2.f32 {%0,%1}, [%2];" : "=f"(r.v[0]), "=f"(r.v[1]) : "l"(p) : "memory");
         else
-            asm("ld.global.nc.v2.f32 {%0,%1}, [%2];" : "=f"(r.v[0]), "=f"(r.v[1]) : "l"(p));
+            asm("ld.global.v2.f32 {%0,%1}, [%2];" : "=f"(r.v[0]), "=f"(r.v[1]) : "l"(p));
     } else if constexpr (W == 4) {
         if constexpr (kCoherent)
             asm volatile("ld.global.v4.f32 {%0,%1,%2,%3}, [%4];"
@@ -137,7 +156,7 @@ __device__ __forceinline__ FieldVec<float, W> ld_field(const FieldVec<float, W>*
                          : "l"(p)
                          : "memory");
         else
-            asm("ld.global.nc.v4.f32 {%0,%1,%2,%3}, [%4];"
+            asm("ld.global.v4.f32 {%0,%1,%2,%3}, [%4];"
                 : "=f"(r.v[0]), "=f"(r.v[1]), "=f"(r.v[2]), "=f"(r.v[3])
                 : "l"(p));
     } else {
@@ -149,7 +168,7 @@ __device__ __forceinline__ FieldVec<float, W> ld_field(const FieldVec<float, W>*
                          : "l"(p)
                          : "memory");
         else
-            asm("ld.global.nc.v8.f32 {%0,%1,%2,%3,%4,%5,%6,%7}, [%8];"
+            asm("ld.global.v8.f32 {%0,%1,%2,%3,%4,%5,%6,%7}, [%8];"
                 : "=f"(r.v[0]), "=f"(r.v[1]), "=f"(r.v[2]), "=f"(r.v[3]), "=f"(r.v[4]), "=f"(r.v[5]),
                   "=f"(r.v[6]), "=f"(r.v[7])
                 : "l"(p));
@@ -239,7 +258,9 @@ __device__ __forceinline__ float4 ld_stream(const float4* p)
 // Reads buffer `in`, writes 1 - in. One species: each thread adds its node's Z terms to
 // zacc (FP32, reduced over the block by the caller); links into solid nodes are skipped.
 // ---------------------------------------------------------------------------------------
-template <int FP, bool kTable, bool kCoherent, int kB>
+// kWait: a launch of one step, which waits for the previous one once its static loads are issued;
+// kPre: the link table's among them (see launch_step_t).
+template <int FP, bool kTable, bool kCoherent, int kB, bool kWait, bool kPre>
 __device__ __forceinline__ void vblock_single(const DArgs& a, int vb, int in, float (&zacc)[3])
 {
     using V = FieldVec<float, FP>;
@@ -249,6 +270,7 @@ __device__ __forceinline__ void vblock_single(const DArgs& a, int vb, int in, fl
     V* Aout = reinterpret_cast<V*>(a.A[1 - in]);
     const int k = vb * kB + threadIdx.x;
     const int M = a.M;
+    if (kWait && k >= a.NF) cudaGridDependencySynchronize();
     if (k < a.NF) {
         const int n = ld_stream(a.flist + k);
         const uint32_t mask = kTable ? kAll : ld_stream(a.fmask + k);
@@ -268,6 +290,16 @@ __device__ __forceinline__ void vblock_single(const DArgs& a, int vb, int in, fl
         }
         const Nbr b = nbrs_of(a.nx, a.ny, a.nz, a.dx, a.dxy, n);
         const float whf = a.whf[0], whe = a.whe[0];
+        float pt[kQ];
+        if constexpr (kTable && kPre) {
+#pragma unroll
+            for (int i = 1; i < kQ; ++i) pt[i] = ld_stream(a.tab + tab_at(k, i));
+        }
+        if (kWait) {
+            cudaGridDependencySynchronize();
+            Pin = after_wait(Pin);
+            Ain = after_wait(Ain);
+        }
         float acc[FP];
 #pragma unroll
         for (int f = 0; f < FP; ++f) acc[f] = 0.f;
@@ -279,7 +311,7 @@ __device__ __forceinline__ void vblock_single(const DArgs& a, int vb, int in, fl
                 const int s = src_of(b, i);
                 float p;
                 if constexpr (kTable) {
-                    p = ld_stream(a.tab + tab_at(k, i));
+                    p = kPre ? pt[i] : ld_stream(a.tab + tab_at(k, i));
                 } else {
                     const Flow4<float> uf = ld_flow(a.u4 + s);
                     p = rn_fma(weight<float>(i), qlink(edot<float>(i, uf.x, uf.y, uf.z), uf.w), is_face(i) ? whf : whe);
@@ -321,18 +353,34 @@ __device__ __forceinline__ void reduce_zacc(double (*s_red)[kMaxSeries], int M, 
     block_store<kB>(s_red, M, out, accumulate);
 }
 
+// the five rows that hold sources at x - 1 and x + 1, numbered (links with c_x != 0)
+__host__ __device__ constexpr int wrap_slot(int i)
+{
+    int n = 0;
+    for (int r = -1; r < row_of(i); ++r)
+        for (int j = 1; j < kQ; ++j)
+            if (cx(j) > 0 && row_of(j) == r) ++n;
+    return n;
+}
+
 // Several species: fields chunk-major over the fluid list, [chunk][k][8 floats] with 8/FP
-// species per chunk (k = index in the sorted fluid list = work item). The link loop is
-// outermost within a pass of up to two chunks: q_i is read (or recomputed) once per link and
-// serves every species of both chunks. Sources are located in the fluid list by row (above).
-template <int FP, bool kTable, bool kCoherent, int kB>
+// species per chunk (k = index in the sorted fluid list = work item), one pass of the links per
+// chunk; q_i is read (or recomputed) once per link and pass and serves the chunk's species (two
+// chunks a pass needed more registers than it saved table reads: 160^3 with 16 species 4-40% slower).
+// Sources are located in the fluid list by row (above).
+// Bound: the L1 gathers of 32-byte records (77% of its rate at 160^3) and latency. With the table the
+// loop has no branch, so that the loads of several links are in flight; a closed link reads the
+// node's own record and adds 0 x (160^3 with 4 species 165 -> 100 us a step, from 186 before both this
+// and the arguments in the constant bank). Recomputing, the flow of the source is needed first and
+// closed links are skipped (121 us without branches, 106 with).
+// kWait: as for vblock_single, with one partial sum per warp and series (part: [K][nw]) and the
+// species constants in the launch's arguments; otherwise they are in shared memory.
+template <int FP, bool kTable, bool kCoherent, int kB, bool kWait>
 __device__ __forceinline__ void vblock_multi(const DArgs& a, int vb, int in, double* part, bool acc_part,
-                                             double (*s_red)[kMaxSeries], const float* s_whf, const float* s_whe,
-                                             const float* s_pa, const float* s_pd)
+                                             double (*s_red)[kMaxSeries], const float* c_whf, const float* c_whe,
+                                             const float* c_pa, const float* c_pd)
 {
     constexpr int kSC = 8 / FP;
-    constexpr int kCP = MP_DIRECT_CP;
-    constexpr int kMaxPass = MP_MAX_SPECIES / (kCP * kSC);
     constexpr int kOW4 = FP == 2 ? 2 : 4;  // float4s per node record
     using VC = FieldVec<float, 8>;
     const VC* Pin = reinterpret_cast<const VC*>(a.P[in]);
@@ -343,140 +391,138 @@ __device__ __forceinline__ void vblock_multi(const DArgs& a, int vb, int in, dou
     const bool active = k < a.NF;
     const int M = a.M, K = a.K;
     const size_t NF = (size_t)a.NF, NI = (size_t)a.NI;
-    int ai = -1, n = 0;
+    int ai = -1;
     uint32_t mask = 0;
+    __shared__ int s_wrap[5][kB];  // written and read by the same thread
     int C[8];  // fluid-list index of each row centre (or of the first fluid node after it)
     bool xlo = true, xhi = true;  // x - 1 and x + 1 lie in r's row without wrapping
     const float4* o = reinterpret_cast<const float4*>(a.own) + (size_t)(active ? k : 0) * kOW4;
     if (active) {
-        n = ld_stream(a.flist + k);
         mask = ld_stream(a.fmask + k);
         ai = ld_stream(a.aidx + k);
-        const Nbr b = nbrs_of(a.nx, a.ny, a.nz, a.dx, a.dxy, n);
+        const Nbr b = nbrs_of(a.nx, a.ny, a.nz, a.dx, a.dxy, ld_stream(a.flist + k));
 #pragma unroll
         for (int j = 0; j < 8; ++j) C[j] = fluid_index(a.fw, src_of(b, row_centre(j)));
         xlo = b.oxm == -1;
         xhi = b.oxp == 1;
+        // rare: x - 1 or x + 1 wraps around the box (never both: nx >= 3). The
+        // sources there go to shared memory: looked up in the link loop they doubled its code.
+#pragma unroll
+        for (int i = 1; i < kQ; ++i)
+            if ((cx(i) > 0 && !xlo) || (cx(i) < 0 && !xhi))
+                s_wrap[wrap_slot(i)][threadIdx.x] = fluid_index(a.fw, src_of(b, i));
     }
-    // the source of link i where x - 1 or x + 1 wraps around the box (rare): the periodic
-    // neighbourhood is rebuilt from n there, so that it is not kept live through the loop
-    auto wrapped_source = [&](int i) {
-        const Nbr b = nbrs_of(a.nx, a.ny, a.nz, a.dx, a.dxy, n);
-        return fluid_index(a.fw, src_of(b, i));
-    };
+    if (kWait) {
+        cudaGridDependencySynchronize();
+        Pin = after_wait(Pin);
+        Ain = after_wait(Ain);
+    }
     const int cpn = a.SP / kSC;
 #pragma unroll 1
-    for (int pass = 0; pass < kMaxPass; ++pass) {
-        const int c0 = pass * kCP;
-        if (c0 >= cpn) break;
-        const int nc = cpn - c0 < kCP ? cpn - c0 : kCP;
-        float acc[kCP][8];
+    for (int ch = 0; ch < cpn; ++ch) {
+        float acc[8];
 #pragma unroll
-        for (int cc = 0; cc < kCP; ++cc)
-#pragma unroll
-            for (int j = 0; j < 8; ++j) acc[cc][j] = 0.f;
+        for (int j = 0; j < 8; ++j) acc[j] = 0.f;
+        const VC* Pc = Pin + (size_t)ch * NF;
         if (active) {
 #pragma unroll
             for (int i = 1; i < kQ; ++i) {
-                if (!((mask >> (i - 1)) & 1u)) continue;
+                const bool open = (mask >> (i - 1)) & 1u;
+                if (!kTable && !open) continue;
                 const int row = row_of(i);
                 const int base = row < 0 ? k : C[row < 0 ? 0 : row];
                 int s;
                 if (cx(i) == 0)
                     s = base;
                 else if (cx(i) > 0)
-                    s = xlo ? base - 1 : wrapped_source(i);
+                    s = xlo ? base - 1 : s_wrap[wrap_slot(i)][threadIdx.x];
                 else
                     s = xhi ? base + (row < 0 ? 1 : (int)((mask >> (row_centre(row < 0 ? 0 : row) - 1)) & 1u))
-                            : wrapped_source(i);
+                            : s_wrap[wrap_slot(i)][threadIdx.x];
                 float q;
                 if constexpr (kTable) {
+                    if (!open) s = k;
                     q = ld_stream(a.tab + tab_at(k, i));
                 } else {
                     const Flow4<float> uf = ld_flow(a.uc + s);
                     q = qlink(edot<float>(i, uf.x, uf.y, uf.z), uf.w);
                 }
+                const VC xs = ld_field<kCoherent, 8>(Pc + s);
 #pragma unroll
-                for (int cc = 0; cc < kCP; ++cc) {
-                    if (cc < nc) {
-                        const VC xs = ld_field<kCoherent, 8>(Pin + (size_t)(c0 + cc) * NF + s);
+                for (int qq = 0; qq < kSC; ++qq) {
+                    const float wh = (is_face(i) ? c_whf : c_whe)[ch * kSC + qq];  // w lambda/2
+                    const float p = kTable && !open ? 0.f : rn_fma(weight<float>(i), q, wh);
 #pragma unroll
-                        for (int qq = 0; qq < kSC; ++qq) {
-                            const int sp = (c0 + cc) * kSC + qq;
-                            const float p = rn_fma(weight<float>(i), q, is_face(i) ? s_whf[sp] : s_whe[sp]);
+                    for (int f = 0; f < FP; ++f) acc[qq * FP + f] = __fmaf_rn(p, xs.v[qq * FP + f], acc[qq * FP + f]);
+                }
+            }
+        }
+        float zv[kSC * 3];
 #pragma unroll
-                            for (int f = 0; f < FP; ++f)
-                                acc[cc][qq * FP + f] = __fmaf_rn(p, xs.v[qq * FP + f], acc[cc][qq * FP + f]);
-                        }
+        for (int j = 0; j < kSC * 3; ++j) zv[j] = 0.f;
+        if (active) {
+            const VC xr = ld_field<kCoherent, 8>(Pc + k);
+            const float4 o0 = __ldg(o);
+            VC xn;
+#pragma unroll
+            for (int qq = 0; qq < kSC; ++qq) {
+                const int sp = ch * kSC + qq;
+                // out = sum_i (w_i q_i + w_i lambda/2) + p_a 1_I: the flow part A, the open
+                // face and edge link counts times w lambda/2, the interface flag times p_a
+                const float out =
+                    __fmaf_rn(o0.w, c_pa[sp], __fmaf_rn(o0.z, c_whe[sp], __fmaf_rn(o0.y, c_whf[sp], o0.x)));
+#pragma unroll
+                for (int f = 0; f < FP; ++f) {
+                    const int j = qq * FP + f;
+                    xn.v[j] = __fadd_rn(__fmaf_rn(-out, xr.v[j], acc[j]), xr.v[j]);
+                }
+            }
+            if (ai >= 0) {
+                const size_t ia = (size_t)ch * NI + ai;
+                const VC xa = ld_field<kCoherent, 8>(Ain + ia);
+                VC xan;
+#pragma unroll
+                for (int qq = 0; qq < kSC; ++qq) {
+                    const int sp = ch * kSC + qq;
+                    const float pa = c_pa[sp], pd = c_pd[sp];
+#pragma unroll
+                    for (int f = 0; f < FP; ++f) {
+                        const int j = qq * FP + f;
+                        const float x0 = xr.v[j];
+                        xn.v[j] = __fmaf_rn(pd, xa.v[j], xn.v[j]);
+                        xan.v[j] = __fmaf_rn(pa, x0, __fmaf_rn(-pd, xa.v[j], xa.v[j]));
+                    }
+                }
+                st_field<8>(Aout + ia, xan);
+            }
+            st_field<8>(Pout + (size_t)ch * NF + k, xn);
+#pragma unroll
+            for (int qq = 0; qq < kSC; ++qq) {
+                const int sp = ch * kSC + qq;
+#pragma unroll
+                for (int m = 0; m < 3; ++m) {
+                    if (m < M && 1 + m < FP) {
+                        // u*_g = UA_g + (face sum of c_g) w_f lambda/2 + (edge sum) w_e lambda/2
+                        const float4 om = __ldg(o + 1 + m);
+                        const float us = __fmaf_rn(om.z, c_whe[sp], __fmaf_rn(om.y, c_whf[sp], om.x));
+                        zv[qq * 3 + m] = xn.v[qq * FP + ((1 + m) < FP ? 1 + m : 0)] * us;
                     }
                 }
             }
         }
+        // warp sums of this chunk's series
+        const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
 #pragma unroll
-        for (int cc = 0; cc < kCP; ++cc) {
-            float zv[kSC * 3];
+        for (int qq = 0; qq < kSC; ++qq) {
+            const int sp = ch * kSC + qq;
+            if (sp < a.S) {
 #pragma unroll
-            for (int j = 0; j < kSC * 3; ++j) zv[j] = 0.f;
-            if (active && cc < nc) {
-                const VC xr = ld_field<kCoherent, 8>(Pin + (size_t)(c0 + cc) * NF + k);
-                const float4 o0 = __ldg(o);
-                VC xn;
-#pragma unroll
-                for (int qq = 0; qq < kSC; ++qq) {
-                    const int sp = (c0 + cc) * kSC + qq;
-                    // out = sum_i (w_i q_i + w_i lambda/2) + p_a 1_I: the flow part A, the open
-                    // face and edge link counts times w lambda/2, the interface flag times p_a
-                    const float out =
-                        __fmaf_rn(o0.w, s_pa[sp], __fmaf_rn(o0.z, s_whe[sp], __fmaf_rn(o0.y, s_whf[sp], o0.x)));
-#pragma unroll
-                    for (int f = 0; f < FP; ++f) {
-                        const int j = qq * FP + f;
-                        xn.v[j] = __fadd_rn(__fmaf_rn(-out, xr.v[j], acc[cc][j]), xr.v[j]);
-                    }
-                }
-                if (ai >= 0) {
-                    const size_t ia = (size_t)(c0 + cc) * NI + ai;
-                    const VC xa = ld_field<kCoherent, 8>(Ain + ia);
-                    VC xan;
-#pragma unroll
-                    for (int qq = 0; qq < kSC; ++qq) {
-                        const int sp = (c0 + cc) * kSC + qq;
-                        const float pa = s_pa[sp], pd = s_pd[sp];
-#pragma unroll
-                        for (int f = 0; f < FP; ++f) {
-                            const int j = qq * FP + f;
-                            const float x0 = xr.v[j];
-                            xn.v[j] = __fmaf_rn(pd, xa.v[j], xn.v[j]);
-                            xan.v[j] = __fmaf_rn(pa, x0, __fmaf_rn(-pd, xa.v[j], xa.v[j]));
-                        }
-                    }
-                    st_field<8>(Aout + ia, xan);
-                }
-                st_field<8>(Pout + (size_t)(c0 + cc) * NF + k, xn);
-#pragma unroll
-                for (int qq = 0; qq < kSC; ++qq) {
-                    const int sp = (c0 + cc) * kSC + qq;
-#pragma unroll
-                    for (int m = 0; m < 3; ++m) {
-                        if (m < M && 1 + m < FP) {
-                            // u*_g = UA_g + (face sum of c_g) w_f lambda/2 + (edge sum) w_e lambda/2
-                            const float4 om = __ldg(o + 1 + m);
-                            const float us = __fmaf_rn(om.z, s_whe[sp], __fmaf_rn(om.y, s_whf[sp], om.x));
-                            zv[qq * 3 + m] = xn.v[qq * FP + ((1 + m) < FP ? 1 + m : 0)] * us;
-                        }
-                    }
-                }
-            }
-            // warp sums of this chunk's series into the block's shared partials
-            const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-#pragma unroll
-            for (int qq = 0; qq < kSC; ++qq) {
-                const int sp = (c0 + cc) * kSC + qq;
-                if (cc < nc && sp < a.S) {
-#pragma unroll
-                    for (int m = 0; m < 3; ++m) {
-                        if (m < M) {
-                            const float w = warp_sum(zv[qq * 3 + m]);
+                for (int m = 0; m < 3; ++m) {
+                    if (m < M) {
+                        const float w = warp_sum(zv[qq * 3 + m]);
+                        if constexpr (kWait) {
+                            if (lane == 0 && k < a.NF) part[(size_t)(sp * M + m) * a.nw + (k >> 5)] = (double)w;
+                        } else {
                             if (lane == 0) s_red[warp][sp * M + m] = (double)w;
                         }
                     }
@@ -484,7 +530,7 @@ __device__ __forceinline__ void vblock_multi(const DArgs& a, int vb, int in, dou
             }
         }
     }
-    block_store<kB>(s_red, K, part, acc_part);
+    if constexpr (!kWait) block_store<kB>(s_red, K, part, acc_part);
 }
 
 // ---------------------------------------------------------------------------------------
@@ -782,7 +828,7 @@ __device__ __forceinline__ void vblock_tiled(const DArgs& a, int vb, int in, dou
 
 // Several species: stage the per-species constants in shared memory (uniform across the
 // block) and run the body; block sums to part[0..K) (stored, or added when acc_part).
-template <int FP, bool kTable, bool kCoherent, int kB>
+template <int FP, bool kTable, bool kCoherent, int kB, bool kWait>
 __device__ __forceinline__ void run_multi(const DArgs& a, int vb, int in, double* part, bool acc_part,
                                           double (*s_red)[kMaxSeries], float* s_c)
 {
@@ -793,7 +839,7 @@ __device__ __forceinline__ void run_multi(const DArgs& a, int vb, int in, double
         s_c[3 * MP_MAX_SPECIES + j] = a.pd[j];
     }
     __syncthreads();
-    vblock_multi<FP, kTable, kCoherent, kB>(a, vb, in, part, acc_part, s_red, s_c, s_c + MP_MAX_SPECIES,
+    vblock_multi<FP, kTable, kCoherent, kB, kWait>(a, vb, in, part, acc_part, s_red, s_c, s_c + MP_MAX_SPECIES,
                                             s_c + 2 * MP_MAX_SPECIES, s_c + 3 * MP_MAX_SPECIES);
 }
 
@@ -824,17 +870,25 @@ __device__ __forceinline__ int ctx_of(const DLaunch& L, int v)
 template <int kB>
 __device__ __forceinline__ double ctx_series_total(const double* part, int nvb, int K, int j, double* s_tmp)
 {
-    // four independent chains of loads, added in a fixed order
-    double v0 = 0.0, v1 = 0.0, v2 = 0.0, v3 = 0.0;
+    // up to 16 independent loads in flight a thread, added in a fixed order to four sums (FP64 adds
+    // are dear: sixteen sums with their tail cost a persistent step of 32^3 nodes 1.9 us of 5.1)
+    double acc[4] = {0.0, 0.0, 0.0, 0.0};
     int b = threadIdx.x;
-    for (; b + 3 * kB < nvb; b += 4 * kB) {
-        v0 += __ldcg(part + (size_t)b * K + j);
-        v1 += __ldcg(part + (size_t)(b + kB) * K + j);
-        v2 += __ldcg(part + (size_t)(b + 2 * kB) * K + j);
-        v3 += __ldcg(part + (size_t)(b + 3 * kB) * K + j);
+    for (; b + 15 * kB < nvb; b += 16 * kB) {
+        double x[16];
+#pragma unroll
+        for (int e = 0; e < 16; ++e) x[e] = __ldcg(part + (size_t)(b + e * kB) * K + j);
+#pragma unroll
+        for (int e = 0; e < 16; ++e) acc[e & 3] += x[e];
     }
-    for (; b < nvb; b += kB) v0 += __ldcg(part + (size_t)b * K + j);
-    double v = (v0 + v1) + (v2 + v3);
+    for (; b < nvb; b += 4 * kB) {
+        double x[4];
+#pragma unroll
+        for (int e = 0; e < 4; ++e) x[e] = b + e * kB < nvb ? __ldcg(part + (size_t)(b + e * kB) * K + j) : 0.0;
+#pragma unroll
+        for (int e = 0; e < 4; ++e) acc[e] += x[e];
+    }
+    double v = (acc[0] + acc[1]) + (acc[2] + acc[3]);
     v = warp_sum(v);
     if ((threadIdx.x & 31) == 0) s_tmp[threadIdx.x >> 5] = v;
     __syncthreads();
@@ -871,18 +925,94 @@ __device__ __forceinline__ void append_series(const DArgs& a, const double* part
     if (threadIdx.x == 0) *a.tdev = t1;
 }
 
-// ---------------------------------------------------------------------------------------
-// One step of every context in the launch; block partials to the half of the partials array
-// of this step's parity (`phase`). The series of the previous step are appended here, by
-// block c for context c while the other blocks work (`pending`: the previous launch was a
-// step whose partials are not yet added), so no block waits for the others at the end; the
-// last step of a run is appended by k_direct_finish.
-// ---------------------------------------------------------------------------------------
-template <int FP, bool kSingle, bool kTable, int kB, bool kTiled>
-__global__ void __launch_bounds__(kB, min_blocks_direct<FP, kSingle, kTiled>(kB))
-    k_direct_step(const __grid_constant__ DLaunch L, int phase, int pending)
+// Appends Z, D of the series j0, j0 + napp, ... of context a for the step of parity `phase`, from
+// its warps' partial sums (FP64, fixed order); called by one whole block.
+template <int kB>
+__device__ __forceinline__ void append_warps(const DArgs& a, int j0, int phase, double* s_tmp)
 {
-    extern __shared__ __align__(16) unsigned char tsm[];  // tiled variant's ring
+    const int in = (a.in0 + phase) & 1;  // the buffer that step read
+    const long long t1 = *((volatile long long*)(a.count + (in ^ 1))) + 1;
+    for (int j = j0; j < a.K; j += a.napp) {
+        const double z = ctx_series_total<kB>(a.part + ((size_t)phase * a.K + j) * a.nw, a.nw, 1, 0, s_tmp);
+        if (threadIdx.x == 0) {
+            a.Z[(size_t)j * a.cap + t1] = z;
+            a.D[(size_t)j * a.cap + t1] = a.D[(size_t)j * a.cap + t1 - 1] + z;
+        }
+    }
+    if (j0 == 0 && threadIdx.x == 0) {
+        a.count[in] = t1;
+        *a.tdev = t1;
+    }
+}
+
+// ---------------------------------------------------------------------------------------
+// One step of every context in the launch. The first blocks append the series of the previous
+// step (`pending`: the previous launch was a step whose partials are not yet added); the others
+// load everything static of their nodes, wait for the previous step, and store one partial sum
+// per warp and series: no block waits for another, and no warp for its block (a block barrier
+// before a reduction cost an eighth to a quarter of the stall cycles). The last step of a run is
+// appended by k_direct_finish.
+// ---------------------------------------------------------------------------------------
+template <int FP, bool kSingle, bool kTable, int kB, bool kPre>
+__device__ __forceinline__ void step_body(const DArgs& a, int vb, int phase)
+{
+    const int in = (a.in0 + phase) & 1;
+    double* part = a.part + (size_t)phase * a.K * a.nw;
+    if (kSingle || a.S == 1) {
+        // one partial sum per block: with few series the appending blocks are few as well
+        __shared__ double s_z[kB / 32][3];
+        float zacc[3] = {0.f, 0.f, 0.f};
+        vblock_single<FP, kTable, false, kB, true, kPre>(a, vb, in, zacc);
+#pragma unroll
+        for (int m = 0; m < 3; ++m) {
+            if (m < a.M) {
+                const float w = warp_sum(zacc[m]);
+                if ((threadIdx.x & 31) == 0) s_z[threadIdx.x >> 5][m] = (double)w;
+            }
+        }
+        __syncthreads();
+        if ((int)threadIdx.x < a.M) {
+            double t = 0.0;
+#pragma unroll
+            for (int w = 0; w < kB / 32; ++w) t += s_z[w][threadIdx.x];
+            part[(size_t)threadIdx.x * a.nw + vb] = t;
+        }
+    } else {
+        vblock_multi<FP, kTable, false, kB, true>(a, vb, in, part, false, nullptr, a.whf, a.whe, a.pa, a.pd);
+    }
+}
+
+// kN: contexts in the launch, at most. kThreads: the threads per SM that registers are budgeted for.
+template <int FP, bool kSingle, bool kTable, int kB, bool kPre, int kN, int kThreads>
+__global__ void __launch_bounds__(kB, kThreads / kB > 1 ? kThreads / kB : 1)
+    k_direct_step(const __grid_constant__ DStepArgs<kN> g, int phase, int pending)
+{
+    cudaTriggerProgrammaticLaunchCompletion();
+    const int nap = g.L.apofs[kN == 1 ? 1 : g.L.n];
+    if ((int)blockIdx.x < nap) {
+        __shared__ double s_tmp[kB / 32];
+        int c = 0;
+        if constexpr (kN > 1) {
+#pragma unroll
+            for (int j = 1; j < kN; ++j)
+                if (j < g.L.n && (int)blockIdx.x >= g.L.apofs[j]) c = j;
+        }
+        cudaGridDependencySynchronize();
+        if (pending) append_warps<kB>(g.a[c], (int)blockIdx.x - g.L.apofs[c], phase ^ 1, s_tmp);
+        return;
+    }
+    const int v = (int)blockIdx.x - nap;
+    const int c = kN == 1 ? 0 : ctx_of(g.L, v);
+    step_body<FP, kSingle, kTable, kB, kPre>(g.a[c], v - g.L.vbofs[c], phase);
+}
+
+// One step of every context by tiles (several species): block partials, the series of the
+// previous step appended by block c for context c while the other blocks work.
+template <int FP, int kB>
+__global__ void __launch_bounds__(kB, min_blocks_direct<FP, false, true>(kB))
+    k_direct_step_tiled(const __grid_constant__ DLaunch L, int phase, int pending)
+{
+    extern __shared__ __align__(16) unsigned char tsm[];  // the ring
     __shared__ double s_red[kB / 32][kMaxSeries];
     __shared__ float s_c[4 * MP_MAX_SPECIES];
     __shared__ double s_tmp[kB / 32];
@@ -896,26 +1026,44 @@ __global__ void __launch_bounds__(kB, min_blocks_direct<FP, kSingle, kTiled>(kB)
     const int vb = (int)blockIdx.x - L.vbofs[c];
     const int in = (a.in0 + phase) & 1;
     double* part = a.part + ((size_t)phase * a.nvb + vb) * a.K;
-    if (kSingle || a.S == 1) {
+    if (a.S == 1) {
         float zacc[3] = {0.f, 0.f, 0.f};
-        vblock_single<FP, kTable, false, kB>(a, vb, in, zacc);
+        vblock_single<FP, false, false, kB, false, false>(a, vb, in, zacc);
         reduce_zacc<kB>(s_red, a.M, zacc, part, false);
-    } else if constexpr (kTiled) {
-        run_tiled<FP, false, kB>(a, vb, in, part, false, s_red, s_c, tsm);
     } else {
-        run_multi<FP, kTable, false, kB>(a, vb, in, part, false, s_red, s_c);
+        run_tiled<FP, false, kB>(a, vb, in, part, false, s_red, s_c, tsm);
     }
 }
 
-// appends the series of the step of parity `phase` (the last step of a run), block c for
-// context c
-template <int kB>
+// appends the series of the step of parity `phase` (the last step of a run): the appending blocks
+// of every context, or (tiled) block c for context c
+template <int kB, bool kTiled>
 __global__ void __launch_bounds__(kB) k_direct_finish(const __grid_constant__ DLaunch L, int phase)
 {
     __shared__ double s_tmp[kB / 32];
     pdl_enter();
-    const DArgs& r = L.args[blockIdx.x];
-    append_series<kB>(r, r.part + (size_t)phase * r.nvb * r.K, r.nvb, s_tmp);
+    if constexpr (kTiled) {
+        const DArgs& r = L.args[blockIdx.x];
+        append_series<kB>(r, r.part + (size_t)phase * r.nvb * r.K, r.nvb, s_tmp);
+    } else {
+        int c = 0;
+#pragma unroll
+        for (int j = 1; j < kMaxCtx; ++j)
+            if (j < L.n && (int)blockIdx.x >= L.apofs[j]) c = j;
+        append_warps<kB>(L.args[c], (int)blockIdx.x - L.apofs[c], phase, s_tmp);
+    }
+}
+
+// the counts of every context from its series position, after launches of another kind have moved
+// it (phase: of the next step)
+__global__ void k_direct_counts(const DArgs* args, int n, int phase)
+{
+    if ((int)threadIdx.x >= n) return;
+    const DArgs& a = args[threadIdx.x];
+    const int in = (a.in0 + phase) & 1;
+    const long long t = *a.tdev;
+    a.count[in] = t - 1;
+    a.count[in ^ 1] = t;
 }
 
 // ---------------------------------------------------------------------------------------
@@ -979,11 +1127,19 @@ __device__ __forceinline__ bool grid_wait(unsigned int* count, unsigned int targ
 #endif
 constexpr bool kRoundRobin = MP_DIRECT_RR != 0;
 
-template <int FP, bool kSingle, bool kTable, int kB, bool kTiled>
+// kOne: the launch of one context of several species, with its arguments by value (as for the
+// one-step launches: 256^3 with 4 species, recomputed: 594 -> 442 us a step).
+__device__ __forceinline__ const DLaunch& launch_of(const DLaunch& L) { return L; }
+__device__ __forceinline__ const DLaunch& launch_of(const DStepArgs<1>& g) { return g.L; }
+__device__ __forceinline__ const DArgs& args_of(const DLaunch& L, int c) { return L.args[c]; }
+__device__ __forceinline__ const DArgs& args_of(const DStepArgs<1>& g, int) { return g.a[0]; }
+
+template <int FP, bool kSingle, bool kTable, int kB, bool kTiled, bool kOne>
 __global__ void __launch_bounds__(kB, min_blocks_direct<FP, kSingle, kTiled>(kB))
-    k_direct_persistent(const __grid_constant__ DLaunch L, int phase0, int nsteps, unsigned int* bar, int* err,
-                        long long timeout_ns)
+    k_direct_persistent(const __grid_constant__ std::conditional_t<kOne, DStepArgs<1>, DLaunch> g, int phase0, int nsteps,
+                        unsigned int* bar, int* err, long long timeout_ns)
 {
+    const DLaunch& L = launch_of(g);
     extern __shared__ __align__(16) unsigned char tsm[];  // tiled variant's ring
     __shared__ double s_red[kB / 32][kMaxSeries];
     __shared__ double s_acc[kMaxSeries];
@@ -1004,7 +1160,7 @@ __global__ void __launch_bounds__(kB, min_blocks_direct<FP, kSingle, kTiled>(kB)
     // the block's sums of context c for step st into its slot: per-thread sums (one species)
     // or the shared accumulator (several)
     auto flush = [&](int c, int st) {
-        const DArgs& a = L.args[c];
+        const DArgs& a = args_of(g, c);
         const int slot = kRoundRobin ? (((int)blockIdx.x - L.vbofs[c]) % G + G) % G
                                      : (int)blockIdx.x - owner(L.vbofs[c]);
         double* dst = a.part + ((size_t)(st & 1) * slots_of(c) + slot) * a.K;
@@ -1020,26 +1176,28 @@ __global__ void __launch_bounds__(kB, min_blocks_direct<FP, kSingle, kTiled>(kB)
         const int phase = (phase0 + st) & 1;
         int cur = -1;
         for (int v = v_lo; v < v_hi; v += v_step) {
-            const int c = ctx_of(L, v);
+            const int c = kOne ? 0 : ctx_of(L, v);
             if (c != cur) {
                 if (cur >= 0) flush(cur, st);
                 for (int j = threadIdx.x; j < kMaxSeries; j += kB) s_acc[j] = 0.0;
                 zacc[0] = zacc[1] = zacc[2] = 0.f;
                 cur = c;
             }
-            const DArgs& a = L.args[c];
+            const DArgs& a = args_of(g, c);
             const int in = (a.in0 + phase) & 1;
             if (kSingle || a.S == 1)
-                vblock_single<FP, kTable, true, kB>(a, v - L.vbofs[c], in, zacc);
+                vblock_single<FP, kTable, true, kB, false, false>(a, v - L.vbofs[c], in, zacc);
             else if constexpr (kTiled)
                 run_tiled<FP, true, kB>(a, v - L.vbofs[c], in, s_acc, true, s_red, s_c, tsm);
+            else if constexpr (kOne)
+                vblock_multi<FP, kTable, true, kB, false>(a, v - L.vbofs[c], in, s_acc, true, s_red, a.whf, a.whe, a.pa, a.pd);
             else
-                run_multi<FP, kTable, true, kB>(a, v - L.vbofs[c], in, s_acc, true, s_red, s_c);
+                run_multi<FP, kTable, true, kB, false>(a, v - L.vbofs[c], in, s_acc, true, s_red, s_c);
         }
         if (cur >= 0) flush(cur, st);
         if (!grid_wait(bar, (unsigned int)(st + 1) * G, err, timeout_ns)) return;
         if ((int)blockIdx.x < L.n) {
-            const DArgs& a = L.args[blockIdx.x];
+            const DArgs& a = args_of(g, (int)blockIdx.x);
             const int slots = slots_of((int)blockIdx.x);
             append_series<kB>(a, a.part + (size_t)(st & 1) * slots * a.K, slots, s_tmp);
         }
@@ -1179,10 +1337,10 @@ void set_tiles(DArgs& a, int sms)
     a.tz = (int)tz;
 }
 int tiles_of(const DArgs& a) { return a.ntx * a.nty * ((a.nz + a.tz - 1) / a.tz); }
-// virtual blocks of the untiled variants at the smallest block (128), or tiles
+// partial sums per series and parity, at most: warps of work items, or tiles
 size_t part_rows(const DArgs& a)
 {
-    const size_t rows = (size_t)((a.NF + 127) / 128);
+    const size_t rows = (size_t)((a.NF + 31) / 32);
     return a.S > 1 ? std::max(rows, (size_t)tiles_of(a)) : rows;
 }
 
@@ -1207,6 +1365,7 @@ struct DirectState {
     unsigned int* bar = nullptr;
     int* err = nullptr;
     int pgrid = 0;  // blocks of the persistent launch
+    int sms = 0;
     cudaGraphExec_t exec[2] = {nullptr, nullptr};
     std::string variant;
 };
@@ -1223,7 +1382,7 @@ template <int FP, bool kSingle, bool kTable, int kB, bool kTiled>
 cudaError_t launch_step_t(DirectState* d, int pending)
 {
     cudaLaunchConfig_t cfg = {};
-    cfg.gridDim = dim3(d->L.vbofs[d->L.n]);
+    cfg.gridDim = dim3(d->L.vbofs[d->L.n] + (kTiled ? 0 : d->L.apofs[d->L.n]));
     cfg.blockDim = dim3(kB);
     cfg.dynamicSmemBytes = dyn_smem<kTiled, kB>();
     cfg.stream = d->stream;
@@ -1232,13 +1391,52 @@ cudaError_t launch_step_t(DirectState* d, int pending)
     attr[0].val.programmaticStreamSerializationAllowed = 1;
     cfg.attrs = attr;
     cfg.numAttrs = 1;
-    return cudaLaunchKernelEx(&cfg, k_direct_step<FP, kSingle, kTable, kB, kTiled>, d->L, d->phase, pending);
+    if constexpr (kTiled)
+        return cudaLaunchKernelEx(&cfg, k_direct_step_tiled<FP, kB>, d->L, d->phase, pending);
+    else
+    {
+        const long long threads = (long long)cfg.gridDim.x * kB;
+        auto wave = [&](int t) { return threads <= (long long)t * d->sms; };  // at t threads per SM
+        auto launch = [&](auto kn) {
+            constexpr int kN = decltype(kn)::value;
+            DStepArgs<kN> g;
+            g.L = d->L;
+            for (int c = 0; c < d->L.n; ++c) g.a[c] = d->h_args[c];
+            if constexpr (kSingle) {
+                // the table's loads go before the wait where one wave of blocks takes the whole launch
+                // (32^3: 3.6 -> 2.4 us; 256^3: 161 -> 307 us, the fields of a block's successor only
+                // start when its table is read)
+                constexpr int kT = MP_DIRECT_SINGLE_THREADS;
+                if constexpr (kTable)
+                    if (wave(kT))
+                        return cudaLaunchKernelEx(&cfg, k_direct_step<FP, true, true, kB, true, kN, kT>, g, d->phase, pending);
+                return cudaLaunchKernelEx(&cfg, k_direct_step<FP, true, kTable, kB, false, kN, kT>, g, d->phase, pending);
+            } else {
+                // More registers a thread keep more of its gathers in flight and hold the link loop
+                // without spills, as long as one wave takes the launch: 512, 768 or 1024 threads per SM
+                // (48^3 with 16 species and two moments 33.7, 47.9, 57.7 us; 64^3 with 4: 10.2, 7.2,
+                // 8.5; 72^3 with 4: 11.4, 12.7, 9.0). Beyond a wave more warps win (160^3 with 4: 129
+                // at 640, 131 at 768, 100 at 1024). Groups, whose several contexts fill the device
+                // sooner, have the last form only.
+                if constexpr (kN == 1) {
+                    if (wave(512))
+                        return cudaLaunchKernelEx(&cfg, k_direct_step<FP, false, kTable, kB, false, kN, 512>, g, d->phase, pending);
+                    if constexpr (kB < 512)
+                        if (wave(768))
+                            return cudaLaunchKernelEx(&cfg, k_direct_step<FP, false, kTable, kB, false, kN, 768>, g, d->phase, pending);
+                }
+                return cudaLaunchKernelEx(&cfg, k_direct_step<FP, false, kTable, kB, false, kN, MP_DIRECT_MULTI_THREADS>, g, d->phase, pending);
+            }
+        };
+        return d->L.n == 1 ? launch(std::integral_constant<int, 1>{}) : launch(std::integral_constant<int, kMaxCtx>{});
+    }
 }
 
 // appends the series of the last step (parity `phase`) of a run of one-step launches
 cudaError_t launch_finish(DirectState* d, int phase)
 {
-    return launch_pdl(k_direct_finish<256>, dim3(d->L.n), dim3(256), d->stream, d->L, phase);
+    if (d->tiled) return launch_pdl(k_direct_finish<256, true>, dim3(d->L.n), dim3(256), d->stream, d->L, phase);
+    return launch_pdl(k_direct_finish<256, false>, dim3(d->L.apofs[d->L.n]), dim3(256), d->stream, d->L, phase);
 }
 
 template <int FP, bool kSingle, bool kTable, int kB, bool kTiled>
@@ -1256,24 +1454,37 @@ cudaError_t launch_persistent_t(DirectState* d, int nsteps)
     attr[0].val.cooperative = 1;
     cfg.attrs = attr;
     cfg.numAttrs = 1;
-    return cudaLaunchKernelEx(&cfg, k_direct_persistent<FP, kSingle, kTable, kB, kTiled>, d->L, d->phase, nsteps,
+    if constexpr (!kSingle && !kTiled)
+        if (d->L.n == 1) {
+            DStepArgs<1> g;
+            g.L = d->L;
+            g.a[0] = d->h_args[0];
+            return cudaLaunchKernelEx(&cfg, k_direct_persistent<FP, kSingle, kTable, kB, kTiled, true>, g, d->phase,
+                                      nsteps, d->bar, d->err, kWaitNs);
+        }
+    return cudaLaunchKernelEx(&cfg, k_direct_persistent<FP, kSingle, kTable, kB, kTiled, false>, d->L, d->phase, nsteps,
                               d->bar, d->err, kWaitNs);
 }
 
 // allows the tiled instances their dynamic shared memory; the persistent grid's blocks per SM
 template <int FP, bool kSingle, bool kTable, int kB, bool kTiled>
-int occupancy_t(int* blocks_per_sm)
+int occupancy_t(int* blocks_per_sm, bool one)
 {
-    if (kTiled) {
+    if constexpr (kTiled) {
         const int bytes = (int)dyn_smem<kTiled, kB>();
-        if (cudaFuncSetAttribute(k_direct_step<FP, kSingle, kTable, kB, kTiled>,
-                                 cudaFuncAttributeMaxDynamicSharedMemorySize, bytes) != cudaSuccess ||
-            cudaFuncSetAttribute(k_direct_persistent<FP, kSingle, kTable, kB, kTiled>,
+        if (cudaFuncSetAttribute(k_direct_step_tiled<FP, kB>, cudaFuncAttributeMaxDynamicSharedMemorySize, bytes) != cudaSuccess ||
+            cudaFuncSetAttribute(k_direct_persistent<FP, kSingle, kTable, kB, kTiled, false>,
                                  cudaFuncAttributeMaxDynamicSharedMemorySize, bytes) != cudaSuccess)
             return MP_ECUDA;
     }
+    if constexpr (!kSingle && !kTiled)
+        if (one)
+            return cudaOccupancyMaxActiveBlocksPerMultiprocessor(
+                       blocks_per_sm, k_direct_persistent<FP, kSingle, kTable, kB, kTiled, true>, kB, 0) == cudaSuccess
+                       ? MP_OK
+                       : MP_ECUDA;
     return cudaOccupancyMaxActiveBlocksPerMultiprocessor(blocks_per_sm,
-                                                         k_direct_persistent<FP, kSingle, kTable, kB, kTiled>, kB,
+                                                         k_direct_persistent<FP, kSingle, kTable, kB, kTiled, false>, kB,
                                                          dyn_smem<kTiled, kB>()) == cudaSuccess
                ? MP_OK
                : MP_ECUDA;
@@ -1325,7 +1536,7 @@ int persistent_grid(DirectState* d)
     int per_sm = 0;
     int rc = dispatch(d, [&](auto fp, auto single, auto table, auto kb, auto tiled) {
         return occupancy_t<decltype(fp)::value, decltype(single)::value, decltype(table)::value, decltype(kb)::value,
-                           decltype(tiled)::value>(&per_sm);
+                           decltype(tiled)::value>(&per_sm, d->L.n == 1);
     });
     if (rc != MP_OK) return rc;
     int dev = 0, sms = 0;
@@ -1351,14 +1562,17 @@ int upload_args(DirectState* d)
 {
     const int n = (int)d->ctx.size();
     d->L.n = n;
-    d->L.vbofs[0] = 0;
+    d->L.vbofs[0] = d->L.apofs[0] = 0;
     for (int c = 0; c < n; ++c) {
         DArgs& a = d->h_args[c];
         const int blk = d->tiled ? 128 : d->block;  // the launch's block size
         a.nvb = d->tiled && a.S > 1 ? tiles_of(a) : (int)((d->ctx[c]->geo.n_fluid + blk - 1) / blk);
         d->L.vbofs[c + 1] = d->L.vbofs[c] + a.nvb;
+        a.nw = a.S > 1 ? (int)((d->ctx[c]->geo.n_fluid + 31) / 32) : a.nvb;
+        a.napp = std::min(a.K, 16);
+        d->L.apofs[c + 1] = d->L.apofs[c] + a.napp;
     }
-    // partials: [2][nvb][K] per context, sized for the most virtual blocks of any variant
+    // partials per context, sized for the most of any variant
     size_t off = 0;
     for (int c = 0; c < n; ++c) {
         DArgs& a = d->h_args[c];
@@ -1412,8 +1626,18 @@ int run_steps(DirectState* d, long long n)
             ph = (ph + m) & 1;
             n -= m;
         }
+        for (mp_ctx* c : d->ctx) c->series_moved = true;
         return MP_OK;
     }
+    if (!d->tiled) {
+        bool moved = false;
+        for (mp_ctx* c : d->ctx) moved = moved || c->series_moved;
+        if (moved) {
+            k_direct_counts<<<1, kMaxCtx, 0, d->stream>>>(d->d_args, d->L.n, d->phase);
+            MP_CUDA(cudaGetLastError());
+        }
+    }
+    for (mp_ctx* c : d->ctx) c->series_moved = d->tiled;
     const int ph0 = d->phase;
     int ph = ph0;
     cudaError_t le = cudaSuccess;
@@ -1531,6 +1755,7 @@ int autotune(DirectState* d, int steps)
             if (e == cudaSuccess) e = cudaMemcpyAsync(x->A[x->cur], bA[c], nA[c], cudaMemcpyDeviceToDevice, d->stream);
             if (e == cudaSuccess)
                 e = cudaMemcpyAsync(x->tdev, &t0[c], sizeof(long long), cudaMemcpyHostToDevice, d->stream);
+            x->series_moved = true;
         }
         if (e == cudaSuccess) e = cudaStreamSynchronize(d->stream);
         if (rc == MP_OK && e != cudaSuccess) rc = cuda_fail(e, "autotune");
@@ -1582,6 +1807,7 @@ DArgs make_dargs(mp_ctx* c)
     a.fw = c->dtab->fw;
     a.iw = c->dtab->iw;
     a.uc = c->dtab->uc;
+    a.count = c->dtab->count;
     for (int b = 0; b < 2; ++b) {
         a.P[b] = (float*)c->P[b];
         a.A[b] = (float*)c->A[b];
@@ -1632,6 +1858,7 @@ int direct_state_create(mp_ctx* const* ctxs, int n, cudaStream_t stream, int tun
         set_error("direct scheme: device query failed");
         return MP_ECUDA;
     }
+    d->sms = sms;
     size_t part_elems = 0;
     for (mp_ctx* c : d->ctx) {
         d->h_args.push_back(make_dargs(c));
@@ -1738,6 +1965,8 @@ int direct_setup(mp_ctx* c, int tune, int variant)
     MP_CUDA(cudaMalloc(&t->aidx, sizeof(int32_t) * NF));
     MP_CUDA(cudaMalloc(&t->tab, sizeof(float) * 18 * ((NF + 31) / 32 * 32)));
     MP_CUDA(cudaMalloc(&t->own, sizeof(float) * t->OW * NF));
+    MP_CUDA(cudaMalloc(&t->count, 2 * sizeof(long long)));
+    c->series_moved = true;
     const float hl = (float)(6.0 * c->Db[0]);
     const float whf = (float)((double)weight<float>(1) * (double)hl);
     const float whe = (float)((double)weight<float>(5) * (double)hl);
@@ -1779,6 +2008,7 @@ void direct_free(mp_ctx* c)
         cudaFree(c->dtab->fw);
         cudaFree(c->dtab->iw);
         cudaFree(c->dtab->uc);
+        cudaFree(c->dtab->count);
         delete c->dtab;
     }
     c->dtab = nullptr;
