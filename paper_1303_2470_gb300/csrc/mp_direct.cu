@@ -373,8 +373,8 @@ __host__ __device__ constexpr int wrap_slot(int i)
 // node's own record and adds 0 x (160^3 with 4 species 165 -> 100 us a step, from 186 before both this
 // and the arguments in the constant bank). Recomputing, the flow of the source is needed first and
 // closed links are skipped (121 us without branches, 106 with).
-// kWait: as for vblock_single, with one partial sum per warp and series (part: [K][nw]) and the
-// species constants in the launch's arguments; otherwise they are in shared memory.
+// kWait: as for vblock_single, with one partial sum per warp and series (part: [K][nw]). c_*: the
+// species constants, in the launch's arguments or staged in shared memory by the caller.
 template <int FP, bool kTable, bool kCoherent, int kB, bool kWait>
 __device__ __forceinline__ void vblock_multi(const DArgs& a, int vb, int in, double* part, bool acc_part,
                                              double (*s_red)[kMaxSeries], const float* c_whf, const float* c_whe,
