@@ -11,6 +11,7 @@
 
 #include "../../include/surrogate.h"
 #include "internal.cuh"
+#include "wgrad_plan.cuh"
 
 using namespace mp;
 
@@ -421,10 +422,10 @@ __global__ void __launch_bounds__(kTThreads) k_conv_tc(const ConvArgs a)
 // ---------------------------------------------------------------------------------------
 constexpr int kMCopy = 256;              // copying threads
 constexpr int kMThreads = 192 + kMCopy;
-constexpr int kMRows = 160;      // staged rows: 16 groups of 8 voxels with two neighbours
+constexpr int kMRows = kColumnRows;      // staged rows: 16 groups of 8 voxels with two neighbours
 constexpr int kMChunk = kMRows * 128;  // bytes of 64 channels of a staged row
 constexpr int kMStages = 8;      // most ring stages
-constexpr int kMSmem = 232448 - 1024;  // dynamic shared memory a block may use (227 KB less static)
+constexpr int kMSmem = kBlockSmem;
 
 struct MarchArgs {
     ConvArgs c;
@@ -746,6 +747,8 @@ __global__ void __launch_bounds__(kMThreads, 1) k_conv_march(const __grid_consta
 //    one slot. The ring's first two slots are copied a second time behind its end, so that
 //    three consecutive rows are always consecutive slots; rows of M beyond 3 CO read whatever
 //    the next slots hold and are dropped.
+// A copy waits until both the x slot and the dy slots that it overwrites have been read
+// (WgradUnits in wgrad_plan.cuh, with the plan).
 // So x and dy are read three times in all (once per dz), and an MMA of K = 16 voxels serves
 // nine taps. Rows of 128, 64 or 32 bytes use the swizzle of that width. A unit's sums (T rows,
 // at most 2048 voxels: partial sums stay as short as those of the kernel below) are added to
@@ -756,7 +759,6 @@ __global__ void __launch_bounds__(kMThreads, 1) k_conv_march(const __grid_consta
 // Waits are bounded as in k_conv_march.
 // ---------------------------------------------------------------------------------------
 constexpr int kGThreads = 160 + kMCopy;
-constexpr int kGStages = 8;
 
 struct WgradTcArgs {
     const bf16* x;
@@ -764,12 +766,7 @@ struct WgradTcArgs {
     float* dw;
     int D, H, W, Cin, Cout;
     int up;              // x is the coarse grid, read as its nearest upsampling
-    int GX, NG;          // groups per x-row, groups over the batch
-    int T, nstrip;       // x rows per unit, strips along y
-    int nci, nco, units;
-    int nX;              // ring stages (x rows); the dy ring has nX + 4 slots
-    int bufs;            // accumulator sets
-    uint32_t ncols;      // tensor-memory columns
+    WgradPlan p;
 };
 
 // MN-major descriptor: `lbo` bytes between channel blocks of one swizzle width, `sbo` between
@@ -802,8 +799,8 @@ __global__ void __launch_bounds__(kGThreads, 1) k_wgrad_tc(const __grid_constant
     __shared__ int s_xoff[kMRows], s_yoff[kTM];  // voxels of the staged rows at y = 0 (-1: none)
     const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
     const uint32_t base = (smem_u32(tc_smem_raw) + kTAtom - 1) & ~(uint32_t)(kTAtom - 1);
-    const int R = m.nX + 4;
-    const uint32_t sX = base, sY = base + (uint32_t)m.nX * kXB;
+    const int R = m.p.slots();
+    const uint32_t sX = base, sY = base + (uint32_t)m.p.nX * kXB;
     if (tid == 0) {
         for (int s = 0; s < kGStages; ++s) {
             asm volatile("mbarrier.init.shared::cta.b64 [%0], %1;" ::"r"(smem_u32(&s_full[s])), "n"(kMCopy));
@@ -819,7 +816,7 @@ __global__ void __launch_bounds__(kGThreads, 1) k_wgrad_tc(const __grid_constant
     }
     if (warp == 0) {
         asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(smem_u32(&s_tmem)),
-                     "r"(m.ncols));
+                     "r"(m.p.ncols));
         asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;");
     }
     asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
@@ -828,7 +825,7 @@ __global__ void __launch_bounds__(kGThreads, 1) k_wgrad_tc(const __grid_constant
     const uint32_t tmem = s_tmem;
     volatile int* fail = &s_fail;
     const int H = m.H, W = m.W, step = (int)gridDim.x;
-    const int combos = 3 * m.nci * m.nco;
+    const int combos = m.p.combos();
 
     if (warp >= 5) {
         // ---- copies ----
@@ -837,12 +834,14 @@ __global__ void __launch_bounds__(kGThreads, 1) k_wgrad_tc(const __grid_constant
         const int pt = tid - 160;
         int slot = 0, ys = 0;  // x slot of the next stage, dy slot of the next dy row
         uint32_t round = 0;
+        int stage = 0;  // the next stage, over all units
+        WgradUnits units;
         bool ok = true, all = true;
-        for (int u = blockIdx.x; u < m.units && all; u += step) {
+        for (int u = blockIdx.x; u < m.p.units && all; u += step) {
             const int combo = u % combos, q = u / combos;
-            const int d = combo % 3, ci0 = (combo / 3) % m.nci * kCI, co0 = combo / (3 * m.nci) * kCO;
-            const int strip = q % m.nstrip, tc = q / m.nstrip;
-            const int y0 = strip * m.T, te = min(m.T, H - y0);
+            const int d = combo % 3, ci0 = (combo / 3) % m.p.nci * kCI, co0 = combo / (3 * m.p.nci) * kCO;
+            const int strip = q % m.p.nstrip, tc = q / m.p.nstrip;
+            const int y0 = strip * m.p.T, te = m.p.rows(u);
             all = bar_and(ok);
             if (!all) break;
             for (int row = pt; row < kMRows + kTM; row += kMCopy) {
@@ -850,8 +849,8 @@ __global__ void __launch_bounds__(kGThreads, 1) k_wgrad_tc(const __grid_constant
                 const int r = isx ? row : row - kMRows;
                 const int g = tc * 16 + (isx ? r / 10 : r / 8);
                 int off = -1;
-                if (g < m.NG) {
-                    const int xg = g % m.GX, l = g / m.GX;
+                if (g < m.p.NG) {
+                    const int xg = g % m.p.GX, l = g / m.p.GX;
                     const int z = l % m.D, b = l / m.D;
                     const int x = isx ? 8 * xg - 1 + r % 10 : 8 * xg + r % 8;
                     if (isx && x <= W) off = x_voxel(m.up, m.D, H, W, b, wrap(z + d - 1, m.D), 0, wrap(x, W));
@@ -884,8 +883,10 @@ __global__ void __launch_bounds__(kGThreads, 1) k_wgrad_tc(const __grid_constant
                 }
                 ys = ys + 1 == R ? 0 : ys + 1;
             };
+            const int w = units.first_waits_for(m.p, stage);
+            if (w >= 0) ok = mbar_wait_or(smem_u32(&s_empty[w % m.p.nX]), (uint32_t)(w / m.p.nX) & 1u, fail);
             for (int i = 0; i < te; ++i) {
-                if (round > 0) ok = mbar_wait_or(smem_u32(&s_empty[slot]), (round - 1) & 1u, fail);
+                if (ok && round > 0) ok = mbar_wait_or(smem_u32(&s_empty[slot]), (round - 1) & 1u, fail);
                 if (!ok) break;
                 if (i == 0) {
                     load_y(wrap(y0 - 1, H));
@@ -902,11 +903,13 @@ __global__ void __launch_bounds__(kGThreads, 1) k_wgrad_tc(const __grid_constant
                 }
                 asm volatile("cp.async.mbarrier.arrive.noinc.shared::cta.b64 [%0];" ::"r"(smem_u32(&s_full[slot]))
                              : "memory");
-                if (++slot == m.nX) {
+                if (++slot == m.p.nX) {
                     slot = 0;
                     ++round;
                 }
             }
+            stage += te;
+            units.ended(stage);
         }
         asm volatile("cp.async.wait_all;" ::: "memory");
     } else if (warp == 4) {
@@ -916,11 +919,10 @@ __global__ void __launch_bounds__(kGThreads, 1) k_wgrad_tc(const __grid_constant
         int slot = 0, ys = 0, nu = 0;
         uint32_t round = 0;
         bool ok = true;
-        for (int u = blockIdx.x; u < m.units && ok; u += step, ++nu) {
-            const int strip = (u / combos) % m.nstrip;
-            const int te = min(m.T, H - strip * m.T);
-            const int buf = m.bufs == 2 ? nu & 1 : 0;
-            const int use = m.bufs == 2 ? nu >> 1 : nu;
+        for (int u = blockIdx.x; u < m.p.units && ok; u += step, ++nu) {
+            const int te = m.p.rows(u);
+            const int buf = m.p.bufs == 2 ? nu & 1 : 0;
+            const int use = m.p.bufs == 2 ? nu >> 1 : nu;
             const uint32_t acc = tmem + (uint32_t)(buf * kTiles * kN);
             if (use > 0) ok = mbar_wait_or(smem_u32(&s_aempty[buf]), (uint32_t)(use - 1) & 1u, fail);
             ok = __all_sync(0xffffffffu, ok);
@@ -944,7 +946,7 @@ __global__ void __launch_bounds__(kGThreads, 1) k_wgrad_tc(const __grid_constant
                     tc_commit(smem_u32(&s_empty[slot]));
                 }
                 ys = ys + 1 == R ? 0 : ys + 1;
-                if (++slot == m.nX) {
+                if (++slot == m.p.nX) {
                     slot = 0;
                     ++round;
                 }
@@ -961,11 +963,11 @@ __global__ void __launch_bounds__(kGThreads, 1) k_wgrad_tc(const __grid_constant
     } else {
         // ---- epilogue: accumulator row = (dy block, output channel), column = (dx, input channel) ----
         int nu = 0;
-        for (int u = blockIdx.x; u < m.units; u += step, ++nu) {
+        for (int u = blockIdx.x; u < m.p.units; u += step, ++nu) {
             const int combo = u % combos;
-            const int d = combo % 3, ci0 = (combo / 3) % m.nci * kCI, co0 = combo / (3 * m.nci) * kCO;
-            const int buf = m.bufs == 2 ? nu & 1 : 0;
-            const int use = m.bufs == 2 ? nu >> 1 : nu;
+            const int d = combo % 3, ci0 = (combo / 3) % m.p.nci * kCI, co0 = combo / (3 * m.p.nci) * kCO;
+            const int buf = m.p.bufs == 2 ? nu & 1 : 0;
+            const int use = m.p.bufs == 2 ? nu >> 1 : nu;
             const bool ok = mbar_wait_or(smem_u32(&s_afull[buf]), (uint32_t)use & 1u, fail);
             if (!__all_sync(0xffffffffu, ok)) break;
             asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
@@ -1005,7 +1007,7 @@ __global__ void __launch_bounds__(kGThreads, 1) k_wgrad_tc(const __grid_constant
     __syncthreads();
     if (tid == 0 && s_fail) atomicExch(&g_sg_tc_fail, 1);
     if (warp == 0)
-        asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(tmem), "r"(m.ncols));
+        asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(tmem), "r"(m.p.ncols));
 }
 
 struct WgradArgs {
@@ -1558,11 +1560,6 @@ bool weight_map(const ConvArgs& a, int NB, CUtensorMap* map)
                   CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) == CUDA_SUCCESS;
 }
 
-// x-rows are cut into groups of 8 voxels; the last one of a row may be short, and what it lacks
-// is work done for nothing. Rows of one or two voxels (an eighth, a quarter of a group) stay with
-// the tap-by-tap kernels, which the marching ones beat by about three.
-bool fills_groups(int W) { return W >= 3; }
-
 // Shape of the marching kernel for one layer, or false where it does not apply. The channel
 // block NB and the strip length T are those with the least estimated time: waves of one unit
 // per SM times the clocks of a unit, where a staged row costs the larger of its MMAs (products
@@ -1623,59 +1620,6 @@ bool march_plan(const ConvArgs& a, int B, int sms, MarchArgs* out, size_t* smem)
     *out = best;
     *smem = best_smem;
     return true;
-}
-
-int channel_block(int c) { return c % 64 == 0 ? 64 : (c % 32 == 0 ? 32 : 16); }
-
-// Shape of k_wgrad_tc for one layer, or false where it does not apply. T is the one with the
-// least estimated time (waves of units x clocks of a unit, as in march_plan) that keeps a
-// unit within 16 rows.
-bool wgrad_plan(const WgradArgs& a, int B, int sms, WgradTcArgs* m, size_t* smem)
-{
-    if (!fills_groups(a.W) || a.total >= (1LL << 31)) return false;
-    const int ci = channel_block(a.Cin), co = channel_block(a.Cout);
-    const size_t xb = (size_t)kMRows * 2 * ci, yb = (size_t)kTM * 2 * co;
-    const int tiles = co == 64 ? 2 : 1, n = 3 * ci;
-    // dy slots: the ring, two copies and what the padding rows of M read beyond a window
-    const int pad = tiles * 128 / co - 1;
-    int nX = kGStages;
-    while (nX > 1 && nX * xb + (nX + 4 + pad) * yb > (size_t)kMSmem - 2048) --nX;
-    if (nX < 2) return false;
-    m->x = a.x;
-    m->dy = a.dy;
-    m->dw = a.dw;
-    m->D = a.D;
-    m->H = a.H;
-    m->W = a.W;
-    m->Cin = a.Cin;
-    m->Cout = a.Cout;
-    m->up = a.up;
-    m->GX = (a.W + 7) / 8;
-    m->NG = B * a.D * m->GX;
-    m->nci = a.Cin / ci;
-    m->nco = a.Cout / co;
-    m->nX = nX;
-    m->bufs = 2 * tiles * n <= 512 ? 2 : 1;
-    m->ncols = 32;
-    while ((int)m->ncols < m->bufs * tiles * n) m->ncols <<= 1;
-    const double row = std::max(std::max(8.0 * tiles * std::max(n / 2.0, 32.0 + n / 4.0), (xb + yb) / 40.0), 300.0);
-    const double flush = 12.0 * tiles * n;
-    const long long per_row = (long long)3 * m->nci * m->nco * ((m->NG + 15) / 16);
-    double best = 0.0;
-    for (int T = 1; T <= a.H && T <= 16; ++T) {
-        const long long units = per_row * ((a.H + T - 1) / T);
-        if (units > (1LL << 30)) continue;
-        const double unit = std::max(T * row + 2.0 * yb / 40.0 + (m->bufs == 1 ? flush : 0.0), flush) + 500.0;
-        const double cost = (double)((units + sms - 1) / sms) * unit + flush;
-        if (best == 0.0 || cost < best) {
-            best = cost;
-            m->T = T;
-            m->nstrip = (a.H + T - 1) / T;
-            m->units = (int)units;
-        }
-    }
-    *smem = nX * xb + (nX + 4 + pad) * yb + 1024;
-    return best > 0.0;
 }
 
 template <int kCI>
@@ -1799,9 +1743,8 @@ int sg_conv3d_wgrad_ex(const void* x, const void* dy, float* dw, float* dbias, i
     int dev = 0, sms = 0;
     MP_CUDA(cudaGetDevice(&dev));
     MP_CUDA(cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev));
-    WgradTcArgs m;
-    size_t smem = 0;
-    const bool tc = wgrad_plan(a, B, sms, &m, &smem);
+    WgradTcArgs m{a.x, a.dy, a.dw, D, H, W, Cin, Cout, a.up, {}};
+    const bool tc = wgrad_plan(B, D, H, W, Cin, Cout, sms, &m.p);
     if (nchunk * 27 > 2147483647LL || ci_tiles * co_tiles > 65535) {
         set_error("sg_conv3d_wgrad: too many voxels or channels");
         return MP_EINVAL;
@@ -1810,7 +1753,7 @@ int sg_conv3d_wgrad_ex(const void* x, const void* dy, float* dw, float* dbias, i
         const int ci = channel_block(Cin), co = channel_block(Cout);
         auto kern = ci == 64 ? wgrad_kernel<64>(co) : (ci == 32 ? wgrad_kernel<32>(co) : wgrad_kernel<16>(co));
         MP_CUDA(cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, kMSmem - 1024));
-        kern<<<std::min(m.units, sms), kGThreads, smem, cs>>>(m);
+        kern<<<std::min(m.p.units, sms), kGThreads, m.p.smem, cs>>>(m);
     } else {
         dim3 grid((unsigned)(nchunk * 27), (unsigned)(ci_tiles * co_tiles));
         k_wgrad<<<grid, kWThreads, 0, cs>>>(a);
