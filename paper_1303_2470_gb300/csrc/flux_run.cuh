@@ -10,16 +10,21 @@ namespace mp {
 
 constexpr int kFluxGraph = 64;  // even: a replay ends on the buffer it started from
 
-// launch(pending): the step from buffer c->cur; pending: the previous launch was a step whose
-// series is not appended yet. finish(parity): appends the series of the last step, which read
-// buffer `parity`.
+// launch(pending, programmatic): the step from buffer c->cur; pending: the previous launch was a
+// step whose series is not appended yet. finish(parity): appends the series of the last step, which
+// read buffer `parity`.
+// A step reads its tables before griddepcontrol.wait. What is read there has to be finished and
+// visible when the launch before it has merely started, and a programmatic launch may start,
+// before its wait, while the table kernel's writes are still on their way. So the first step after
+// set-up is an ordinary launch (or the first node of a graph), and every later one follows it.
 template <typename Launch, typename Finish>
 int run_flux(mp_ctx* c, long long n, Launch launch, Finish finish)
 {
     cudaError_t le = cudaSuccess;  // first failed launch, if any
     auto run = [&](long long count) {
         for (long long k = 0; k < count; ++k) {
-            const cudaError_t e = launch(k > 0 ? 1 : 0);
+            const cudaError_t e = launch(k > 0 ? 1 : 0, !c->tables_new);
+            c->tables_new = false;
             if (e != cudaSuccess && le == cudaSuccess) le = e;
             c->cur = 1 - c->cur;
         }
@@ -32,6 +37,7 @@ int run_flux(mp_ctx* c, long long n, Launch launch, Finish finish)
         c->stream != nullptr && c->stream != cudaStreamLegacy && c->stream != cudaStreamPerThread;
     if (capturable && n >= 2 * kFluxGraph) {
         const int b = c->cur;
+        c->tables_new = false;  // a graph starts when all work before it is done
         if (!c->exec[b]) {
             cudaError_t e = cudaStreamBeginCapture(c->stream, cudaStreamCaptureModeThreadLocal);
             if (e == cudaSuccess) {

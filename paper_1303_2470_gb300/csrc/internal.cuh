@@ -76,9 +76,14 @@ struct Geometry {
 // Launch with programmatic dependent launch allowed: on the same stream the kernel may start
 // while the previous kernel drains (its blocks become resident and wait). Such a kernel calls
 // pdl_enter() first: it lets its own dependents start, then waits until the previous grid has
-// finished and its writes are visible, so nothing it reads or writes can race with it.
+// finished and its writes are visible, so nothing it reads or writes can race with it. What a
+// kernel reads before that wait has to come from work that an ordinary launch, copy or graph between
+// them has waited for.
+// launch_dependent: the same, or (not `programmatic`) an ordinary launch, which starts when all work
+// before it on the stream is done and visible.
 template <typename... KArgs, typename... Args>
-cudaError_t launch_pdl(void (*kern)(KArgs...), dim3 grid, dim3 block, cudaStream_t s, Args&&... args)
+cudaError_t launch_dependent(bool programmatic, void (*kern)(KArgs...), dim3 grid, dim3 block, cudaStream_t s,
+                             Args&&... args)
 {
     cudaLaunchConfig_t cfg = {};
     cfg.gridDim = grid;
@@ -89,8 +94,13 @@ cudaError_t launch_pdl(void (*kern)(KArgs...), dim3 grid, dim3 block, cudaStream
     attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
     attr[0].val.programmaticStreamSerializationAllowed = 1;
     cfg.attrs = attr;
-    cfg.numAttrs = 1;
+    cfg.numAttrs = programmatic ? 1 : 0;
     return cudaLaunchKernelEx(&cfg, kern, std::forward<Args>(args)...);
+}
+template <typename... KArgs, typename... Args>
+cudaError_t launch_pdl(void (*kern)(KArgs...), dim3 grid, dim3 block, cudaStream_t s, Args&&... args)
+{
+    return launch_dependent(true, kern, grid, block, s, std::forward<Args>(args)...);
 }
 
 __device__ __forceinline__ void pdl_enter()

@@ -67,6 +67,8 @@ struct mp_ctx {
     // the series position has been moved by launches that do not keep the counts by which the
     // one-step launches (flux32, direct) find it: they are to be set before the next run
     bool series_moved = false;
+    // the flux tables have been built and no step has been launched since (run_flux)
+    bool tables_new = false;
 };
 
 namespace mp {

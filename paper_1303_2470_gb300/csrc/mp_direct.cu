@@ -1632,6 +1632,9 @@ int run_steps(DirectState* d, long long n)
     if (!d->tiled) {
         bool moved = false;
         for (mp_ctx* c : d->ctx) moved = moved || c->series_moved;
+        // also an ordinary launch between the tables, which a step reads before its wait, and the
+        // first step after set-up (c->series_moved is set there): a programmatic one right behind the
+        // table kernel could read them before they are visible
         if (moved) {
             k_direct_counts<<<1, kMaxCtx, 0, d->stream>>>(d->d_args, d->L.n, d->phase);
             MP_CUDA(cudaGetLastError());

@@ -375,10 +375,10 @@ int step32(mp_ctx* c, long long n)
     const int blocks = a.napp + (a.NF + kB - 1) / kB;
     return run_flux(
         c, n,
-        [&](int pending) {
+        [&](int pending, bool programmatic) {
             const int s = c->cur;
-            return launch_pdl(kern, dim3(blocks), dim3(kB), c->stream, a, (const TS*)c->P[s], (TS*)c->P[1 - s],
-                              (const TS*)c->A[s], (TS*)c->A[1 - s], s, pending);
+            return launch_dependent(programmatic, kern, dim3(blocks), dim3(kB), c->stream, a, (const TS*)c->P[s],
+                                    (TS*)c->P[1 - s], (const TS*)c->A[s], (TS*)c->A[1 - s], s, pending);
         },
         [&](int parity) {
             return launch_pdl(k_finish32, dim3(a.napp), dim3(kAppendThreads), c->stream, a, parity);
@@ -455,6 +455,7 @@ int flux32_setup(mp_ctx* c)
                                                                     c->dir[2], f->aidx, f->ust);
     MP_CUDA(cudaGetLastError());
     c->series_moved = true;
+    c->tables_new = true;
     return MP_OK;
 }
 

@@ -294,23 +294,24 @@ __global__ void k_tables64(const F64Args a, const uint32_t* __restrict__ fmask, 
 }
 
 template <int FP, bool kSingle, int kLanes, int kB>
-cudaError_t launch64_t(mp_ctx* c, int pending)
+cudaError_t launch64_t(mp_ctx* c, int pending, bool programmatic)
 {
     const F64Args& a = c->flux64->a;
     const int s = c->cur;
-    return launch_pdl(k_step64<FP, kSingle, kLanes, kB>, dim3(a.nblk + 1, a.S), dim3(kB), c->stream, a, (const double*)c->P[s],
-                      (double*)c->P[1 - s], (const double*)c->A[s], (double*)c->A[1 - s], s, pending);
+    return launch_dependent(programmatic, k_step64<FP, kSingle, kLanes, kB>, dim3(a.nblk + 1, a.S), dim3(kB), c->stream, a,
+                            (const double*)c->P[s], (double*)c->P[1 - s], (const double*)c->A[s],
+                            (double*)c->A[1 - s], s, pending);
 }
 
-cudaError_t launch64(mp_ctx* c, int pending)
+cudaError_t launch64(mp_ctx* c, int pending, bool prog)
 {
     const bool small = c->flux64->lanes == 4;
     if (c->FP == 2) {
-        if (c->S == 1) return small ? launch64_t<2, true, 4, 64>(c, pending) : launch64_t<2, true, 1, 128>(c, pending);
-        return small ? launch64_t<2, false, 4, 64>(c, pending) : launch64_t<2, false, 1, 128>(c, pending);
+        if (c->S == 1) return small ? launch64_t<2, true, 4, 64>(c, pending, prog) : launch64_t<2, true, 1, 128>(c, pending, prog);
+        return small ? launch64_t<2, false, 4, 64>(c, pending, prog) : launch64_t<2, false, 1, 128>(c, pending, prog);
     }
-    if (c->S == 1) return small ? launch64_t<4, true, 4, 64>(c, pending) : launch64_t<4, true, 2, 128>(c, pending);
-    return small ? launch64_t<4, false, 4, 64>(c, pending) : launch64_t<4, false, 2, 128>(c, pending);
+    if (c->S == 1) return small ? launch64_t<4, true, 4, 64>(c, pending, prog) : launch64_t<4, true, 2, 128>(c, pending, prog);
+    return small ? launch64_t<4, false, 4, 64>(c, pending, prog) : launch64_t<4, false, 2, 128>(c, pending, prog);
 }
 
 }  // namespace
@@ -390,13 +391,14 @@ int flux64_setup(mp_ctx* c)
         make_div((unsigned)c->geo.nx), make_div((unsigned)(c->geo.nx * c->geo.ny)), c->dir[0], c->dir[1], c->dir[2],
         f->aidx, f->src, f->tab, f->ust, f->lanes > 1);
     MP_CUDA(cudaGetLastError());
+    c->tables_new = true;
     return MP_OK;
 }
 
 int flux64_step(mp_ctx* c, long long n)
 {
     return run_flux(
-        c, n, [&](int pending) { return launch64(c, pending); },
+        c, n, [&](int pending, bool programmatic) { return launch64(c, pending, programmatic); },
         [&](int parity) { return launch_pdl(k_finish64, dim3(1), dim3(256), c->stream, c->flux64->a, parity); });
 }
 
