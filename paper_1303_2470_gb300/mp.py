@@ -410,9 +410,9 @@ def mp_step_noalloc(solid, u, D_b, k_a, k_d, direction, X, X_ads, X_out, X_ads_o
         index = _noalloc_device(torch, solid, u, X, X_ads, X_out, X_ads_out, Z_out)
         if index is not None and index == torch.cuda.current_device():
             nz, ny, nx = solid.shape
-            _check(_lib.mp_step_noalloc(nx, ny, nz, solid.data_ptr(), None if u is None else u.data_ptr(), D_b, k_a,
-                                        k_d, direction, X.data_ptr(), X_ads.data_ptr(), X_out.data_ptr(),
-                                        X_ads_out.data_ptr(), Z_out.data_ptr(), _stream(stream)))
+            _check(_lib.mp_step_noalloc(nx, ny, nz, solid.data_ptr(), None if u is None else u.data_ptr(), float(D_b),
+                                        float(k_a), float(k_d), int(direction), X.data_ptr(), X_ads.data_ptr(),
+                                        X_out.data_ptr(), X_ads_out.data_ptr(), Z_out.data_ptr(), _stream(stream)))
             return
     if not (hasattr(solid, "data_ptr") and getattr(solid, "is_cuda", False) and len(solid.shape) == 3
             and str(solid.dtype) in ("torch.uint8", "torch.bool") and solid.is_contiguous()):
