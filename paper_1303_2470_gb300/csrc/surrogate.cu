@@ -1229,11 +1229,13 @@ enum CoarseOp { kPool, kPoolGrad, kUp, kUpGrad, kPoolGradRelu, kUpGradRelu };
 
 // src: the fine grid for kPool, kUpGrad(Relu), else the coarse one. kPoolGradRelu: dst[child] =
 // (g[child] + src[parent] / 8) where act[child] > 0, else 0 (both BF16 roundings of the separate
-// passes); kUpGradRelu: dst[parent] = sum of the children where act[parent] > 0, else 0
+// passes), and dst may be g: neither is restrict, and a thread reads its eight values of g, by
+// ordinary loads, before it writes any. kUpGradRelu: dst[parent] = sum of the children where
+// act[parent] > 0, else 0
 template <int kOp>
-__global__ void __launch_bounds__(256) k_coarse8(const bf16* __restrict__ src, const bf16* __restrict__ g,
-                                                 const bf16* __restrict__ act, bf16* __restrict__ dst, unsigned n,
-                                                 int D, int H, int W, int C8)
+__global__ void __launch_bounds__(256) k_coarse8(const bf16* __restrict__ src, const bf16* g,
+                                                 const bf16* __restrict__ act, bf16* dst, unsigned n, int D, int H,
+                                                 int W, int C8)
 {
     // D, H, W: coarse sizes; n: coarse voxels of the batch x C8
     const unsigned i = blockIdx.x * 256u + threadIdx.x;
@@ -1280,12 +1282,17 @@ __global__ void __launch_bounds__(256) k_coarse8(const bf16* __restrict__ src, c
             v = pack8(p);
             unpack8(v, p);  // rounded, as the separate pass stores it
         }
+        uint4 gv[8];
+        if constexpr (kOp == kPoolGradRelu) {
+#pragma unroll
+            for (int k = 0; k < 8; ++k) gv[k] = reinterpret_cast<const uint4*>(g)[child(k)];
+        }
 #pragma unroll
         for (int k = 0; k < 8; ++k) {
             const size_t o = child(k);
             if constexpr (kOp == kPoolGradRelu) {
                 float gf[8], af[8];
-                unpack8(__ldg(reinterpret_cast<const uint4*>(g) + o), gf);
+                unpack8(gv[k], gf);
                 unpack8(__ldg(reinterpret_cast<const uint4*>(act) + o), af);
 #pragma unroll
                 for (int e = 0; e < 8; ++e) gf[e] = af[e] > 0.0f ? gf[e] + p[e] : 0.0f;
