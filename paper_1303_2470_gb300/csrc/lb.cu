@@ -362,15 +362,20 @@ extern "C" int lb_steady(const mp_geometry* geom, const double force[3], double 
     // the row table where 16-bit offsets reach the neighbouring planes (at the fluid nodes of a
     // plane on average)
     const bool wide = kQ * (unsigned long long)NF >= (1ull << 32);
-    const bool use_rows = !wide && (double)G.n_fluid / G.nz * 1.2 + G.nx < 32000.0;
+    bool use_rows = !wide && (double)G.n_fluid / G.nz * 1.2 + G.nx < 32000.0;
     unsigned long long* res_d = nullptr;
     cudaError_t e = pool_malloc((void**)&g0, sizeof(float) * kQ * NF, s);
     if (e == cudaSuccess) e = pool_malloc((void**)&omask, sizeof(uint32_t) * NF, s);
     if (e == cudaSuccess) e = pool_malloc((void**)&fw, sizeof(uint2) * (size_t)(G.W > 0 ? G.W : 1), s);
-    if (e == cudaSuccess && use_rows) e = pool_malloc((void**)&rows, sizeof(uint4) * NF, s);
     if (e == cudaSuccess) e = pool_malloc((void**)&g1, sizeof(float) * kQ * NF, s);
     if (e == cudaSuccess) e = pool_malloc((void**)&uprev, sizeof(float) * 3 * NF, s);
     if (e == cudaSuccess) e = pool_malloc((void**)&res_d, sizeof(unsigned long long), s);
+    // last, and only if there is room for it: a tenth more memory, which the step can do without
+    if (e == cudaSuccess && use_rows && pool_malloc((void**)&rows, sizeof(uint4) * NF, s) != cudaSuccess) {
+        (void)cudaGetLastError();
+        rows = nullptr;
+        use_rows = false;
+    }
     // solid entries of the dense outputs stay zero; fluid entries are written at every check
     if (e == cudaSuccess) e = cudaMemsetAsync(u_out, 0, sizeof(float) * 3 * N, s);
     if (e == cudaSuccess && rho_out) e = cudaMemsetAsync(rho_out, 0, sizeof(float) * N, s);
