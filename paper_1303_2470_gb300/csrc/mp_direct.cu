@@ -871,7 +871,9 @@ template <int kB>
 __device__ __forceinline__ double ctx_series_total(const double* part, int nvb, int K, int j, double* s_tmp)
 {
     // up to 16 independent loads in flight a thread, added in a fixed order to four sums (FP64 adds
-    // are dear: sixteen sums with their tail cost a persistent step of 32^3 nodes 1.9 us of 5.1)
+    // are dear: sixteen sums with their tail cost a persistent step of 32^3 nodes 1.9 us of 5.1).
+    // Few blocks' sums, as small lattices have, go through the last loop: a loop of four
+    // with zeros for the missing terms cost 0.1-0.3 us a series
     double acc[4] = {0.0, 0.0, 0.0, 0.0};
     int b = threadIdx.x;
     for (; b + 15 * kB < nvb; b += 16 * kB) {
@@ -881,13 +883,14 @@ __device__ __forceinline__ double ctx_series_total(const double* part, int nvb, 
 #pragma unroll
         for (int e = 0; e < 16; ++e) acc[e & 3] += x[e];
     }
-    for (; b < nvb; b += 4 * kB) {
+    for (; b + 3 * kB < nvb; b += 4 * kB) {
         double x[4];
 #pragma unroll
-        for (int e = 0; e < 4; ++e) x[e] = b + e * kB < nvb ? __ldcg(part + (size_t)(b + e * kB) * K + j) : 0.0;
+        for (int e = 0; e < 4; ++e) x[e] = __ldcg(part + (size_t)(b + e * kB) * K + j);
 #pragma unroll
         for (int e = 0; e < 4; ++e) acc[e] += x[e];
     }
+    for (; b < nvb; b += kB) acc[0] += __ldcg(part + (size_t)b * K + j);
     double v = (acc[0] + acc[1]) + (acc[2] + acc[3]);
     v = warp_sum(v);
     if ((threadIdx.x & 31) == 0) s_tmp[threadIdx.x >> 5] = v;
