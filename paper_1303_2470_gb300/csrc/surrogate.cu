@@ -1125,10 +1125,11 @@ __global__ void __launch_bounds__(kWThreads) k_wgrad(const WgradArgs a)
     }
 }
 
-// dbias[c] += sum over voxels of dy[.][c]: a block sums kBiasRows voxels, a thread 8 channels
+// dbias[c] += sum over voxels of dy[.][c]: a block sums `block_rows` voxels, a thread 8 channels
 // (16 bytes) of every (256 / (C / 8))-th of them; blockIdx.y: blocks of 2048 channels
-constexpr int kBiasRows = 1024, kBiasCh = 2048;
-__global__ void __launch_bounds__(256) k_bias_grad(const bf16* __restrict__ dy, float* __restrict__ db, long long total, int C)
+constexpr int kBiasCh = 2048;
+__global__ void __launch_bounds__(256) k_bias_grad(const bf16* __restrict__ dy, float* __restrict__ db, long long total,
+                                                   int C, int block_rows)
 {
     __shared__ float part[256][8];
     const int c0 = blockIdx.y * kBiasCh, Cb = min(C - c0, kBiasCh);
@@ -1136,8 +1137,8 @@ __global__ void __launch_bounds__(256) k_bias_grad(const bf16* __restrict__ dy, 
     const int j = threadIdx.x % C8, r = threadIdx.x / C8;
     float s[8] = {0.f, 0.f, 0.f, 0.f, 0.f, 0.f, 0.f, 0.f};
     if (r < rows) {
-        const long long e0 = (long long)blockIdx.x * kBiasRows;
-        const int n = (int)(total - e0 < kBiasRows ? total - e0 : kBiasRows);
+        const long long e0 = (long long)blockIdx.x * block_rows;
+        const int n = (int)(total - e0 < block_rows ? total - e0 : block_rows);
         const uint4* p = reinterpret_cast<const uint4*>(dy + (size_t)e0 * C + c0) + j;
 #pragma unroll 4
         for (int e = r; e < n; e += rows) {
@@ -1767,7 +1768,11 @@ int sg_conv3d_wgrad_ex(const void* x, const void* dy, float* dw, float* dbias, i
     }
     MP_CUDA(cudaGetLastError());
     if (dbias) {
-        k_bias_grad<<<dim3(grid1(a.total, kBiasRows), (Cout + kBiasCh - 1) / kBiasCh), 256, 0, cs>>>((const bf16*)dy, dbias, a.total, Cout);
+        // two blocks an SM, of 64 to 1024 voxels: in blocks of 1024 the four of a 64 x 64 x 1 box with 256
+        // channels took 11 us longer
+        const int rows = (int)std::min<long long>(1024, std::max<long long>(64, (a.total + 2 * sms - 1) / (2 * sms)));
+        k_bias_grad<<<dim3(grid1(a.total, rows), (Cout + kBiasCh - 1) / kBiasCh), 256, 0, cs>>>((const bf16*)dy, dbias,
+                                                                                              a.total, Cout, rows);
         MP_CUDA(cudaGetLastError());
     }
     return MP_OK;
