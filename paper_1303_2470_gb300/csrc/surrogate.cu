@@ -1752,7 +1752,12 @@ int sg_conv3d_wgrad_ex(const void* x, const void* dy, float* dw, float* dbias, i
     MP_CUDA(cudaGetDevice(&dev));
     MP_CUDA(cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev));
     WgradTcArgs m{a.x, a.dy, a.dw, D, H, W, Cin, Cout, a.up, {}};
-    const bool tc = wgrad_plan(B, D, H, W, Cin, Cout, sms, &m.p);
+    // A unit of the tensor-core kernel adds up its partial sums for a whole column of 128 voxels; on the
+    // smallest boxes the general kernel, one block a tap and channel tile, is done earlier. Both, us without
+    // bias (general / tensor cores): 64 voxels, 64 -> 64 channels 6.4 / 10.8, 32 -> 32 4.7 / 6.8; 128
+    // voxels 6.8 / 10.7, 6.5 / 6.8; 256 voxels 10.6 / 10.7, 8.8 / 6.8; 384 voxels 12.8 / 10.8, 10.8 / 6.8
+    const bool few = a.total <= (channel_block(Cin) == 64 ? 256 : 128);
+    const bool tc = !few && wgrad_plan(B, D, H, W, Cin, Cout, sms, &m.p);
     if (nchunk * 27 > 2147483647LL || ci_tiles * co_tiles > 65535) {
         set_error("sg_conv3d_wgrad: too many voxels or channels");
         return MP_EINVAL;
