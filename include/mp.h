@@ -112,11 +112,19 @@ typedef struct {
                            state, restores the state and keeps the fastest (needs 24 free
                            entries in the series). See mp_variant.                          */
     int variant;        /* MP_SCHEME_DIRECT without autotune: 0 (one launch per step, link
-                           table, blocks of 256) or MP_VARIANT_* flags                       */
+                           table, blocks of 256) or MP_VARIANT_* flags. MP_SCHEME_FLUX: of the
+                           flags MP_VARIANT_RECOMPUTE alone counts, see there                 */
 } mp_options;
 
 /* ---- kernel variants of MP_SCHEME_DIRECT (mp_options.variant); all give the same fields ---- */
-#define MP_VARIANT_RECOMPUTE 1  /* link terms recomputed from the packed flow, no link table   */
+#define MP_VARIANT_RECOMPUTE 1  /* link terms recomputed from the packed flow, no link table. With
+                                   MP_SCHEME_FLUX: none of the tables that mp_step reads for a context
+                                   stepped on its own (slower steps, the same fields with FP32 and
+                                   binary16 storage, to rounding with FP64). They take 364 bytes per
+                                   fluid node and 8 per series with FP64, else 4 bytes and 4 (one
+                                   species) or 8 per direction and half a byte per series; by default
+                                   contexts keep them up to 64 MB, and beyond where they are at most
+                                   a quarter of the free device memory. Groups never read them.   */
 #define MP_VARIANT_PERSISTENT 2 /* one persistent launch per run of steps                       */
 #define MP_VARIANT_BLOCK128 4   /* blocks of 128 threads (default 256)                          */
 #define MP_VARIANT_BLOCK512 8   /* blocks of 512 threads                                        */

@@ -10,6 +10,21 @@ namespace mp {
 
 constexpr int kFluxGraph = 64;  // even: a replay ends on the buffer it started from
 
+// Tables are an option that costs memory: more than 64 MB only where they take at most a quarter of
+// what is free once the context's own arrays are in place, so that the capacity of a device (binary16
+// storage above all) is not spent on them. The context then recomputes, as with MP_VARIANT_RECOMPUTE.
+inline bool tables_fit(size_t bytes, size_t free_bytes) { return bytes <= (64u << 20) || bytes <= free_bytes / 4; }
+inline bool tables_fit(size_t bytes)
+{
+    if (tables_fit(bytes, 0)) return true;  // no look-up for small contexts
+    size_t free_b = 0, total_b = 0;
+    if (cudaMemGetInfo(&free_b, &total_b) != cudaSuccess) {
+        (void)cudaGetLastError();
+        return false;
+    }
+    return tables_fit(bytes, free_b);
+}
+
 // launch(pending, programmatic): the step from buffer c->cur; pending: the previous launch was a
 // step whose series is not appended yet. finish(parity): appends the series of the last step, which
 // read buffer `parity`.

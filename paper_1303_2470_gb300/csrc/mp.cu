@@ -1139,7 +1139,7 @@ int mp_init_batch(mp_ctx** out, const mp_geometry* g, const float* u, int n_spec
         rc = MP_ENEGPROB;
     }
     if (rc == MP_OK && c->scheme == MP_SCHEME_DIRECT) rc = direct_setup(c, opt.autotune, opt.variant);
-    if (rc == MP_OK && c->scheme == MP_SCHEME_FLUX)
+    if (rc == MP_OK && c->scheme == MP_SCHEME_FLUX && !(opt.variant & MP_VARIANT_RECOMPUTE))
         rc = c->precision == MP_FP64 ? flux64_setup(c) : flux32_setup(c);
     if (rc != MP_OK) {
         destroy(c);
@@ -1174,7 +1174,7 @@ int mp_step(mp_ctx* c, int64_t n)
     if (c->scheme == MP_SCHEME_DIRECT) return direct_step(c, n);
     if (c->flux32) return flux32_step(c, n);
     if (c->flux64) return flux64_step(c, n);
-    // without tables (no memory for them)
+    // without tables (no room for them, or MP_VARIANT_RECOMPUTE)
     return c->precision == MP_FP64   ? step_typed<double, double>(c, n)
            : c->precision == MP_FP16 ? step_typed<float, __half>(c, n)
                                      : step_typed<float, float>(c, n);

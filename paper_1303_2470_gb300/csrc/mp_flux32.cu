@@ -398,11 +398,15 @@ void flux32_free(mp_ctx* c)
     c->flux32 = nullptr;
 }
 
-// Tables, 8 bytes and more per fluid node; where they cannot be allocated the context keeps the
-// step of mp.cu (c->flux32 stays NULL).
+// Tables: 4 bytes per fluid node and 4 (one species) or 8 per direction, and half a byte per series;
+// where they do not fit (tables_fit) or cannot be allocated the context keeps the step of mp.cu
+// (c->flux32 stays NULL).
 int flux32_setup(mp_ctx* c)
 {
     const size_t NF = (size_t)c->geo.n_fluid, K = (size_t)(c->S * c->M);
+    const size_t nw = (NF + 31) / 32;  // warps of nodes
+    const size_t ust_bytes = sizeof(float) * (c->S == 1 ? 1 : 2) * (size_t)c->M * NF, part_bytes = sizeof(double) * 2 * K * nw;
+    if (!tables_fit(sizeof(int32_t) * NF + ust_bytes + part_bytes)) return MP_OK;
     Flux32* f = new (std::nothrow) Flux32();
     if (!f) return MP_OK;
     c->flux32 = f;
@@ -418,13 +422,13 @@ int flux32_setup(mp_ctx* c)
     a.M = c->M;
     a.K = (int)K;
     a.chunks = c->S == 1 ? 1 : c->SP / c->SC;
-    a.nw = (int)((NF + 31) / 32);
+    a.nw = (int)nw;
     a.napp = (int)std::min<size_t>(K, 64);
     a.dx = make_div((unsigned)c->geo.nx);
     a.dxy = make_div((unsigned)(c->geo.nx * c->geo.ny));
     cudaError_t e = cudaMalloc(&f->aidx, sizeof(int32_t) * NF);
-    if (e == cudaSuccess) e = cudaMalloc(&f->ust, sizeof(float) * (c->S == 1 ? 1 : 2) * (size_t)c->M * NF);
-    if (e == cudaSuccess) e = cudaMalloc(&f->part, sizeof(double) * 2 * K * (size_t)a.nw);
+    if (e == cudaSuccess) e = cudaMalloc(&f->ust, ust_bytes);
+    if (e == cudaSuccess) e = cudaMalloc(&f->part, part_bytes);
     if (e == cudaSuccess) e = cudaMalloc(&f->count, sizeof(long long) * 2);
     if (e != cudaSuccess) {
         (void)cudaGetLastError();

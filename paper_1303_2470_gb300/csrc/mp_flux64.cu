@@ -339,21 +339,14 @@ void flux64_free(mp_ctx* c)
 }
 
 // Builds the tables of an FP64 flux context whose fields are initialised. They take 364 bytes
-// per fluid node plus 8 per series; where that is more than a quarter of the free device
-// memory (looked up only beyond 64 MB) or cannot be allocated, the context keeps the step of
-// mp.cu, which recomputes the link terms (c->flux64 stays NULL).
+// per fluid node plus 8 per series; where that does not fit (tables_fit) or cannot be allocated, the
+// context keeps the step of mp.cu, which recomputes the link terms (c->flux64 stays NULL).
 int flux64_setup(mp_ctx* c)
 {
     const size_t NF = (size_t)c->geo.n_fluid, K = (size_t)(c->S * c->M);
     const size_t rows = (NF + 31) / 32 * 32;  // whole groups of 32 in the link tables
     const size_t bytes = rows * (18 * (sizeof(double2) + sizeof(int32_t)) + sizeof(int32_t) + sizeof(double) * K);
-    if (bytes > (64u << 20)) {
-        size_t free_b = 0, total_b = 0;
-        if (cudaMemGetInfo(&free_b, &total_b) != cudaSuccess || bytes > free_b / 4) {
-            (void)cudaGetLastError();
-            return MP_OK;
-        }
-    }
+    if (!tables_fit(bytes)) return MP_OK;
     Flux64* f = new (std::nothrow) Flux64();
     if (!f) return MP_OK;
     c->flux64 = f;
