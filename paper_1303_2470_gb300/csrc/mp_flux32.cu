@@ -14,6 +14,8 @@
 // Per step (the body of mp.cu -> this one): fcc 100^3 x 4 species 35.3 -> 16.7 us; 128^3 36.1 -> 26.1;
 // 256^3 256 -> 200; 48^3 10.3 -> 5.8; 64^3 x 16 species x 2 moments 132 -> 64.6; binary16 88^3 x 2 moments
 // 22.6 -> 14.7, 96^3 x 4 species 47.7 -> 26.1.
+#include <cooperative_groups.h>
+
 #include <algorithm>
 #include <cstring>
 #include <new>
@@ -62,10 +64,10 @@ struct Flux32 {
 namespace {
 
 constexpr uint32_t kAllLinks = (1u << 18) - 1u;
-constexpr int kAppendThreads = 256;
+constexpr int kFinishBlocks = 8, kFinishThreads = 128;  // a series of k_finish32_wide
 
 // appends the series of the step that read buffer `parity`: block b adds the series b, b + napp,
-// ... over the warps (FP64, fixed order)
+// ... over the warps (FP64, fixed order: four sums for each of kB threads; k_finish32_wide keeps to it)
 template <int kB>
 __device__ __forceinline__ void append32(const F32Args& a, int b, int parity)
 {
@@ -317,10 +319,69 @@ __global__ void __launch_bounds__(kB, kCP == 0 ? kSingleBlocks : kMultiBlocks)
     }
 }
 
-__global__ void __launch_bounds__(kAppendThreads) k_finish32(const __grid_constant__ F32Args a, int parity)
+// append32 as a launch of its own (the last step of a run)
+__global__ void __launch_bounds__(kB) k_finish32(const __grid_constant__ F32Args a, int parity)
 {
     pdl_enter();
-    append32<kAppendThreads>(a, blockIdx.x, parity);
+    append32<kB>(a, blockIdx.x, parity);
+}
+
+// The same where the series are sums of many warps (kWideSeries and more): nothing hides this launch,
+// and one SM adds two FP64 numbers a clock. The four sums of append32's kB threads are spread over the
+// blocks of a cluster, one sum a thread, and put together in the same order in the first block's
+// shared memory. Runs of one step, one block a series / a cluster: 64^3 (3.3 k warps) 12.6 / 13.3 us,
+// 128^3 (26 k) 42.0 / 36.3, 256^3 (210 k) 327 / 240.
+constexpr int kWideSeries = 6144;
+__global__ void __cluster_dims__(kFinishBlocks, 1, 1) __launch_bounds__(kFinishThreads)
+    k_finish32_wide(const __grid_constant__ F32Args a, int parity)
+{
+    static_assert(kFinishBlocks * kFinishThreads == 4 * kB, "one sum a thread");
+    namespace cg = cooperative_groups;
+    __shared__ double s_v[4 * kB];
+    __shared__ double s_w[kB / 32];
+    const cg::cluster_group cluster = cg::this_cluster();
+    const int rank = (int)cluster.block_rank(), b = (int)blockIdx.x / kFinishBlocks;
+    double* sums = cluster.map_shared_rank(s_v, 0);
+    pdl_enter();
+    const long long t1 = *(volatile long long*)(a.count + (parity ^ 1)) + 1;
+    const int q = rank * kFinishThreads + (int)threadIdx.x, first = q % kB, col = q / kB * kB;
+    for (int j = b; j < a.K; j += a.napp) {
+        const double* p = a.part + ((size_t)parity * a.K + j) * a.nw;
+        double v = 0.0;
+        int w = first;
+        for (; w + 28 * kB + 3 * kB < a.nw; w += 32 * kB) {
+            double x[8];
+#pragma unroll
+            for (int k = 0; k < 8; ++k) x[k] = __ldcg(p + w + col + 4 * k * kB);
+#pragma unroll
+            for (int k = 0; k < 8; ++k) v += x[k];
+        }
+        for (; w + 3 * kB < a.nw; w += 4 * kB) v += __ldcg(p + w + col);
+        if (col == 0)
+            for (; w < a.nw; w += kB) v += __ldcg(p + w);
+        sums[q] = v;
+        cluster.sync();
+        if (rank == 0) {
+#pragma unroll
+            for (int i = (int)threadIdx.x; i < kB; i += kFinishThreads) {
+                const double u = warp_sum((s_v[i] + s_v[i + kB]) + (s_v[i + 2 * kB] + s_v[i + 3 * kB]));
+                if ((i & 31) == 0) s_w[i >> 5] = u;
+            }
+            __syncthreads();
+            if (threadIdx.x == 0) {
+                double t = 0.0;
+                for (int k = 0; k < kB / 32; ++k) t += s_w[k];
+                const double z = t * a.zsc[j / a.M];
+                a.Z[(size_t)j * a.cap + t1] = z;
+                a.D[(size_t)j * a.cap + t1] = a.D[(size_t)j * a.cap + t1 - 1] + z;
+            }
+        }
+        cluster.sync();  // the first block's sums are free again, and stay until every block has written
+    }
+    if (q == 0 && b == 0) {
+        a.count[parity] = t1;
+        *a.tdev = t1;
+    }
 }
 
 // counts from the series position (after other launches have moved it): next: the buffer that the
@@ -381,7 +442,9 @@ int step32(mp_ctx* c, long long n)
                                     (TS*)c->P[1 - s], (const TS*)c->A[s], (TS*)c->A[1 - s], s, pending);
         },
         [&](int parity) {
-            return launch_pdl(k_finish32, dim3(a.napp), dim3(kAppendThreads), c->stream, a, parity);
+            return a.nw < kWideSeries
+                       ? launch_pdl(k_finish32, dim3(a.napp), dim3(kB), c->stream, a, parity)
+                       : launch_pdl(k_finish32_wide, dim3(kFinishBlocks * a.napp), dim3(kFinishThreads), c->stream, a, parity);
         });
 }
 
