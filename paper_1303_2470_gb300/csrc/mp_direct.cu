@@ -101,9 +101,10 @@ struct DArgs {
     float* A[2];
     float whf[MP_MAX_SPECIES], whe[MP_MAX_SPECIES], pa[MP_MAX_SPECIES], pd[MP_MAX_SPECIES];
     // partial sums of the K = S*M series, by step parity: [2][slots][K] (persistent and tiled
-    // launches), or one per warp of work items, [2][K][nw] (one launch per step)
+    // launches), or [2][K][nw] (one launch per step), one per warp of work items with several
+    // species and one per block with one
     double* part;
-    int nw, napp;  // one launch per step: warps of work items, blocks that append the series
+    int nw, napp;  // one launch per step: partial sums of a series, blocks that append the series
     // time index of the last appended step that read buffer 0 and 1. A step that reads buffer b
     // ends at time count[b] + 2; count[b] is written by the launch before it, never by its own.
     long long* count;
@@ -929,7 +930,7 @@ __device__ __forceinline__ void append_series(const DArgs& a, const double* part
 }
 
 // Appends Z, D of the series j0, j0 + napp, ... of context a for the step of parity `phase`, from
-// its warps' partial sums (FP64, fixed order); called by one whole block.
+// its nw partial sums a series (FP64, fixed order); called by one whole block.
 template <int kB>
 __device__ __forceinline__ void append_warps(const DArgs& a, int j0, int phase, double* s_tmp)
 {
@@ -951,10 +952,12 @@ __device__ __forceinline__ void append_warps(const DArgs& a, int j0, int phase, 
 // ---------------------------------------------------------------------------------------
 // One step of every context in the launch. The first blocks append the series of the previous
 // step (`pending`: the previous launch was a step whose partials are not yet added); the others
-// load everything static of their nodes, wait for the previous step, and store one partial sum
-// per warp and series: no block waits for another, and no warp for its block (a block barrier
-// before a reduction cost an eighth to a quarter of the stall cycles). The last step of a run is
-// appended by k_direct_finish.
+// load everything static of their nodes, wait for the previous step, and store their partial sums:
+// no block waits for another. With several species a partial sum is a warp's, so that no warp waits
+// for its block either (a block barrier before a reduction cost an eighth to a quarter of the stall
+// cycles); with one species, whose few series have few appending blocks, it is the block's
+// (a warp's: 128^3 20.3 -> 27.4 us, the appending blocks became the longest of the launch). The last
+// step of a run is appended by k_direct_finish.
 // ---------------------------------------------------------------------------------------
 template <int FP, bool kSingle, bool kTable, int kB, bool kPre>
 __device__ __forceinline__ void step_body(const DArgs& a, int vb, int phase)

@@ -101,23 +101,23 @@ __global__ void __launch_bounds__(kNaThreads, 8)
         for (int i = 1; i < kQ; ++i) {
             const int s = src_of(b, i);
             const bool open = (mask >> (i - 1)) & 1u;
-                float sx = 0.f, sy = 0.f, sz = 0.f;
-                if (kFlow) {
-                    sx = (open ? __ldg(u + s) : 0.0f);
-                    sy = (open ? __ldg(u + a.N + s) : 0.0f);
-                    sz = (open ? __ldg(u + 2 * a.N + s) : 0.0f);
-                }
-                const float xs = (open ? __ldg(X + s) : 0.0f);
-                const float as = rn_mul(-1.5f, rn_add(rn_add(rn_mul(sx, sx), rn_mul(sy, sy)), rn_mul(sz, sz)));
-                const float whl = is_face(i) ? whl_face : whl_edge;
-                const float pin = rn_fma(weight<float>(i), qlink(edot<float>(i, sx, sy, sz), as), whl);
-                const float pout = rn_fma(weight<float>(i), qlink(edot<float>(opposite(i), ux, uy, uz), ar), whl);
-                const float d = rn_add(delta, rn_sub(rn_mul(pin, xs), rn_mul(pout, xr)));
-                delta = open ? d : delta;
-                if (a.g >= 0) {
-                    const int c = ci(opposite(i), a.g);
-                    if (c != 0) us += open ? float(c) * pout : 0.0f;
-                }
+            float sx = 0.f, sy = 0.f, sz = 0.f;
+            if (kFlow) {
+                sx = (open ? __ldg(u + s) : 0.0f);
+                sy = (open ? __ldg(u + a.N + s) : 0.0f);
+                sz = (open ? __ldg(u + 2 * a.N + s) : 0.0f);
+            }
+            const float xs = (open ? __ldg(X + s) : 0.0f);
+            const float as = rn_mul(-1.5f, rn_add(rn_add(rn_mul(sx, sx), rn_mul(sy, sy)), rn_mul(sz, sz)));
+            const float whl = is_face(i) ? whl_face : whl_edge;
+            const float pin = rn_fma(weight<float>(i), qlink(edot<float>(i, sx, sy, sz), as), whl);
+            const float pout = rn_fma(weight<float>(i), qlink(edot<float>(opposite(i), ux, uy, uz), ar), whl);
+            const float d = rn_add(delta, rn_sub(rn_mul(pin, xs), rn_mul(pout, xr)));
+            delta = open ? d : delta;
+            if (a.g >= 0) {
+                const int c = ci(opposite(i), a.g);
+                if (c != 0) us += open ? float(c) * pout : 0.0f;
+            }
         }
         if (mask != (1u << (kQ - 1)) - 1u) {
             const float xa = Xa[n];

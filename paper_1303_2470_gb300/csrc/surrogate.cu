@@ -1667,7 +1667,8 @@ static int conv3d(const void* x, const void* w, const float* bias, void* y, floa
     }
     // the ring plus room to align it to a 1024-byte boundary
     const size_t smem = (size_t)kTStages * (kTABytes + (size_t)(bn / 8) * kTAtom) + kTAtom;
-    // instances with the input-channel count fixed at compile time for the network's layers
+    // boxes narrower than three voxels, other channel counts, weights off a 16-byte boundary: tap by
+    // tap, with the usual channel counts fixed at compile time
     void (*kern)(const ConvArgs) = K == 16   ? k_conv_tc<16>
                                    : K == 32 ? k_conv_tc<32>
                                    : K == 64 ? k_conv_tc<64>
