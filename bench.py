@@ -61,40 +61,34 @@ METRIC = "sorption-MP node-species updates/s (whole job incl. LB to steady)"
 UNIT = "node-species updates/s"
 
 # DRAM traffic per launch from ncu (dram__bytes_read.sum + dram__bytes_write.sum), valid only
-# while the kernel source hashes to `src_sha`; otherwise reported as null.
+# while the kernel source hashes to `src_sha`; otherwise reported as null. The direct scheme's
+# entries: kernel, link terms (table or recomputed). Captured on mp_direct.cu '3c86f04f9537c499',
+# which has changed since in a comment only.
+_PROBE_SCALE = 22_649_211 / 2_830_813  # fluid nodes of the 384^3 probe to those of its 192^3 case
 TRAFFIC = {
-    # ncu --set full, python bench.py --profile, k_step<float,2,1> launch 11 (caches flushed
-    # by ncu before the capture, so this is the cold-L2 traffic of one launch). Captured on
-    # mp.cu 'cd4af1701d41b82f'; the file changed since only in the flow-packing kernel (64-bit
-    # offsets), not in k_step.
-    "k_step<float>": {"bytes_per_launch": 48_607_488 + 1_392_640, "src_sha": "450a088ead29ab87"},
-    # ncu --metrics dram__bytes_read.sum,dram__bytes_write.sum, python bench.py --profile
-    # --scheme direct --variant 2: one persistent launch of 20 steps moved 1299.98 + 93.68 MB;
-    # per step (the unit of the roofline entry). Captured on mp_direct.cu 'be2e78e2a2bfa30f';
-    # the file changed since only in host code (the tiled variant's block size) and in the
-    # several-species kernels (register use, comments), not in this kernel.
-    "k_direct_persistent": {"bytes_per_launch": (1_299_980_800 + 93_677_056) // 20, "src_sha": "4588265e46e22840"},
-    # the same metrics, python bench.py --profile --scheme direct --variant 4 (one launch per
-    # step, link table, blocks of 128; the autotuner's choice when it times within noise of the
-    # persistent launch): three launches, 94.13 + 2.56 MB on average. ncu flushes the caches
-    # before each captured launch, so this is the cold-L2 traffic of a step (an upper bound;
-    # the persistent launch's warm steps move 69.7 MB).
-    "k_direct_step": {"bytes_per_launch": (93_998_080 + 94_247_168 + 94_153_984 + 4_150_528 + 1_185_536 + 2_335_744) // 3,
-                      "src_sha": "4588265e46e22840"},
-    # the same metrics, python bench.py --profile-probe --scheme direct --variant 7: one
-    # persistent launch of 20 steps of 192^3 x 4 species (2 830 813 fluid nodes) moved
-    # 6175.20 + 2775.19 MB; per step, scaled by the units to the 384^3 x 4 probe
-    # (22 649 211 fluid nodes). Captured on mp_direct.cu 'be2e78e2a2bfa30f'; since then the
-    # kernel keeps fewer registers live (fewer spills to local memory), same data accesses.
-    "k_direct_persistent@probe": {"bytes_per_launch": int((6_175_201_280 + 2_775_187_456) / 20 * 22_649_211 / 2_830_813),
-                                  "src_sha": "4588265e46e22840"},
-    # ncu --set full, python bench.py --profile-probe --scheme direct --variant 1 (one launch per
-    # step, recomputed link terms, blocks of 256): one step of 192^3 x 4 species moved
-    # 310.77 + 128.08 MB (cold L2); scaled by the units to the 384^3 x 4 probe. Captured on
-    # mp_direct.cu 'be2e78e2a2bfa30f'; the kernel has kept fewer registers live since, same
-    # data accesses.
-    "k_direct_step@probe": {"bytes_per_launch": int((310_765_824 + 128_075_776) * 22_649_211 / 2_830_813),
-                            "src_sha": "4588265e46e22840"},
+    # ncu --set full, python bench.py --profile --scheme flux, launch 9 (caches flushed by ncu before
+    # the capture, so this is the cold-L2 traffic of one launch)
+    "k_step32<float>": {"bytes_per_launch": 54_866_944 + 2_218_752, "src": "mp_flux32.cu", "src_sha": "56d2d2a19b7664e7"},
+    # ncu --cache-control none --metrics dram__bytes_read.sum,dram__bytes_write.sum, python bench.py
+    # --profile --scheme direct --variant 4: the mean of steps 13-18, 68.13 + 1.32 MB with what the
+    # step before left in L2 (95 MB with flushed caches)
+    "k_direct_step,table": {"bytes_per_launch": (67_763_456 + 68_155_904 + 68_147_968 + 68_216_832 + 68_210_176
+                                                 + 68_261_120 + 2_076_160 + 1_679_360 + 1_219_328 + 1_065_216
+                                                 + 1_020_416 + 855_552) // 6,
+                            "src": "mp_direct.cu", "src_sha": "c9bd7a5f73b3a7f6"},
+    # the same metrics, python bench.py --profile --scheme direct --variant 2: one persistent launch of
+    # 20 steps moved 1352.02 + 95.56 MB; per step (the unit of the roofline entry)
+    "k_direct_persistent,table": {"bytes_per_launch": (1_352_017_152 + 95_558_656) // 20, "src": "mp_direct.cu",
+                                  "src_sha": "c9bd7a5f73b3a7f6"},
+    # the same metrics, python bench.py --profile-probe --scheme direct --variant 4, 1 and 3 (20 steps
+    # in a launch) on 192^3 x 4 species (2 830 813 fluid nodes), scaled by the units to the 384^3 x 4
+    # probe (22 649 211 fluid nodes); the working set is beyond L2 at either size
+    "k_direct_step,table@probe": {"bytes_per_launch": int((470_632_619 + 110_017_793) * _PROBE_SCALE),
+                                  "src": "mp_direct.cu", "src_sha": "c9bd7a5f73b3a7f6"},
+    "k_direct_step,recompute@probe": {"bytes_per_launch": int((312_577_024 + 113_043_712) * _PROBE_SCALE),
+                                      "src": "mp_direct.cu", "src_sha": "c9bd7a5f73b3a7f6"},
+    "k_direct_persistent,recompute@probe": {"bytes_per_launch": int((6_175_266_560 + 2_708_710_912) / 20 * _PROBE_SCALE),
+                                            "src": "mp_direct.cu", "src_sha": "c9bd7a5f73b3a7f6"},
 }
 
 
@@ -107,6 +101,13 @@ JOB_FIXED_LAUNCHES = 24
 def _src_sha(name):
     p = os.path.join(ROOT, "paper_1303_2470_gb300", "csrc", name)
     return hashlib.sha256(open(p, "rb").read()).hexdigest()[:16]
+
+
+def _traffic(kernel, variant, suffix=""):
+    """Captured DRAM bytes per launch of an MP step kernel in the variant that ran, or None."""
+    key = kernel if variant == "flux" else f"{kernel},{variant.split(',')[1]}"
+    tr = TRAFFIC.get(key + suffix)
+    return tr["bytes_per_launch"] if tr and tr["src_sha"] == _src_sha(tr["src"]) else None
 
 
 def _peaks():
@@ -217,12 +218,10 @@ def run_hbm_probe(mp, peak, peak_kind, scheme_opts):
     nbytes = nf * (16 * S + 13) + ni * 16 * S
     ctx.close()
     if variant == "flux":
-        name, src = "k_step<float,multi>", "mp.cu"
+        name = "k_step32<float,multi>"
     else:
         name = "k_direct_persistent" if variant.startswith("persistent") else "k_direct_step"
-        src = "mp_direct.cu"
-    tr = TRAFFIC.get(name + "@probe")
-    traffic = tr["bytes_per_launch"] if tr and tr["src_sha"] == _src_sha(src) else None
+    traffic = _traffic(name, variant, "@probe")
     gbs = nbytes / step_s / 1e9
     return {"kernel": name, "variant": variant, "bound": "hbm", "achieved": gbs, "peak": peak, "unit": "GB/s",
             "frac": gbs / peak, "traffic": traffic, "algorithmic_bytes_per_step": nbytes,
@@ -235,15 +234,13 @@ def run_hbm_probe(mp, peak, peak_kind, scheme_opts):
 
 
 def mp_kernel_launches(variant, steps, tuned):
-    """Kernels of mp_step(steps) and of the scheme's set-up: one launch per step plus one that
-    appends the last step's series per run (graphs of 64 steps are runs), or one persistent
-    launch. The set-up adds the table kernel; the direct scheme's, when tuned, 20 + 2 steps of
-    each of the six one-step candidates (with their closing launches and the one that sets
-    their counts) and two launches of each of the six persistent ones."""
-    if variant == "flux":
-        return steps + -(-steps // 64) + 1
-    run = 1 if variant.startswith("persistent") else steps + -(-steps // 64)
-    return run + 1 + (6 * (22 + 3) + 6 * 2 if tuned else 0)
+    """Kernels of one mp_step(steps) on the default stream (no graphs) and of the scheme's set-up:
+    one launch per step plus one that appends the last step's series, or one persistent launch. The
+    set-up adds the table kernel and, for one-step launches, the one that sets their counts; the
+    direct scheme's, when tuned, 20 + 2 steps of each of the six one-step candidates (with their
+    closing launches and their counts) and two launches of each of the six persistent ones."""
+    run = 1 if variant.startswith("persistent") else steps + 2
+    return run + 1 + (6 * (22 + 3) + 6 * 2 if tuned and variant != "flux" else 0)
 
 
 def make_medium():
@@ -784,7 +781,7 @@ def main():
     eb = 2 if args.precision == "fp16" else 4                     # bytes per stored field value
     variant = info["variant"]
     if variant == "flux":
-        mp_name, mp_src = ("k_step<float,half>" if args.precision == "fp16" else "k_step<float>"), "mp.cu"
+        mp_name, mp_src = ("k_step32<half>" if args.precision == "fp16" else "k_step32<float>"), "mp_flux32.cu"
     else:
         # a persistent launch runs the whole run of steps: its per-step time is the unit
         mp_name = "k_direct_persistent" if variant.startswith("persistent") else "k_direct_step"
@@ -804,8 +801,7 @@ def main():
                       "algorithmic_bytes": lb_bytes, "gbs": lb_bytes / lb_launch_s / 1e9, "src": "lb.cu"},
     }
     dom = max(kern, key=lambda k: kern[k]["share"])
-    tr = TRAFFIC.get(dom)
-    traffic = tr["bytes_per_launch"] if tr and tr["src_sha"] == _src_sha(kern[dom]["src"]) else None
+    traffic = _traffic(dom, variant) if dom == mp_name else None
     roofline = {"kernel": dom, "bound": "hbm", "achieved": kern[dom]["gbs"], "peak": peak, "unit": "GB/s",
                 "frac": kern[dom]["gbs"] / peak, "traffic": traffic,
                 "peak_source": f"{peak_kind} (MEASURED_PEAKS.json hbm_gbs)" if peak_kind == "measured"

@@ -369,7 +369,8 @@ __host__ __device__ constexpr int wrap_slot(int i)
 // chunk; q_i is read (or recomputed) once per link and pass and serves the chunk's species (two
 // chunks a pass needed more registers than it saved table reads: 160^3 with 16 species 4-40% slower).
 // Sources are located in the fluid list by row (above).
-// Bound: the L1 gathers of 32-byte records (77% of its rate at 160^3) and latency. With the table the
+// Bound: the L1 gathers of 32-byte records (192^3 with 4 species, recomputed: 75 % of its rate; a group
+// of 96^3 and 128^3 with 16, table: 79 %; issue slots 54 % used) and latency. With the table the
 // loop has no branch, so that the loads of several links are in flight; a closed link reads the
 // node's own record and adds 0 x (160^3 with 4 species 165 -> 100 us a step, from 186 before both this
 // and the arguments in the constant bank). Recomputing, the flow of the source is needed first and

@@ -2,8 +2,9 @@
 // storage) stepped on their own: the same update with the same roundings (see k_step there), so
 // the fields are bitwise those of a grouped step.
 //
-// What bounds it: instruction issue and L1 latency (about 90 instructions per link, 42-53 % of
-// the issue slots used before). What differs from the grouped body:
+// What bounds it: the L1 gathers of the sources and their latency (128^3, one species: L1 at 75 % of
+// its rate, 53 % of the issue slots used, 677 instructions a node; the grouped body 725). What
+// differs from that body:
 //  * u*_g is tabulated (it depends on the flow only), which takes 30-60 instructions out of every
 //    node and its accumulators out of the registers;
 //  * no barrier: every warp stores its own partial sums (waiting for the block's slowest warp

@@ -35,13 +35,15 @@ struct NaArgs {
 // Same update as the library's step kernel, read from dense arrays: X(r) + sum of net link
 // fluxes, then the sorption exchange on interfacial nodes (paper Sec. "Algorithm",
 // Eqs. propagated_quantity, Pads, newP), and sum_r X'(r) u*_g(r) in FP64.
-// Everything is recomputed from the mask and the flow, about a thousand instructions a fluid
-// node, and issuing them is what bounds it: in a porous medium most lanes of a warp of
-// consecutive nodes are solid. So a block packs the fluid nodes of its 256 onto its 128 threads
-// (in one or two rounds), with 64 registers and no branch around a link, so that the loads of
-// several links are in flight; the sums are taken over the nodes in their own order all the
-// same. A call on 64^3 spheres (porosity 0.4) takes 14.3 us (one thread a node, a branch a link:
-// 20.8), on 127^3 51 us (93).
+// Everything is recomputed from the mask and the flow, about 1270 instructions a fluid node, and in
+// a porous medium most lanes of a warp of consecutive nodes are solid. So a block packs the fluid
+// nodes of its 256 onto its 128 threads (in one or two rounds), with 64 registers and no branch around
+// a link, so that the loads of several links are in flight; the sums are taken over the nodes in
+// their own order all the same. A call on 64^3 spheres (porosity 0.4) takes 14.3 us (one thread a
+// node, a branch a link: 20.8), on 127^3 51 us (93). What bounds it now: issuing takes 3.3 us of
+// 64^3 and half the time of 127^3; the 64^3 launch is 0.84 of a wave with 40 % of the issue slots
+// used, and waits on its chain (mask bytes, packing, two barriers, eighteen mask bytes, the
+// gathers) and then for the sum's launch.
 template <bool kFlow>
 __global__ void __launch_bounds__(kNaThreads, 8)
     k_step_noalloc(const __grid_constant__ NaArgs a, const uint8_t* __restrict__ solid, const float* __restrict__ u,
