@@ -66,7 +66,8 @@ int sg_check(void* stream);
  * dbias is not NULL, dbias[co] += sum_{b, v} dy[b][v][co] (FP32 accumulation; the caller
  * zeroes dw and dbias before the first call of a step). x BF16 [B][V][Cin], dy BF16
  * [B][V][Cout]. Summation order varies between runs (atomic adds). W >= 3 runs on the
- * 5th-generation tensor cores with bounded waits (sg_check), narrower boxes with mma.sync.
+ * 5th-generation tensor cores with bounded waits (sg_check), narrower boxes and those of up to 128
+ * voxels (256 where Cin is a multiple of 64) with mma.sync.
  * sg_conv3d_wgrad_ex: the same with x BF16 [B][D/2][H/2][W/2][Cin] read as its nearest-neighbour
  * upsampling when `up` is nonzero (D, H, W even).
  */

@@ -1,7 +1,7 @@
 // surrogate.cu -- kernels of the learned warm start for lb_steady (include/surrogate.h): 3x3x3
 // periodic convolutions, forward and both gradients, on the 5th-generation tensor cores
 // (tcgen05.mma with accumulators in tensor memory; the weight gradient of boxes narrower than three
-// voxels with mma.sync m16n8k16; BF16 operands, FP32 accumulation),
+// voxels or of very few with mma.sync m16n8k16; BF16 operands, FP32 accumulation),
 // pooling, upsampling, the masked loss and the Adam update. Nothing here belongs to the moment-propagation
 // method itself; the network's output only seeds lb_steady.
 #include <algorithm>
