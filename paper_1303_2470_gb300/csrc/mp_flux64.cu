@@ -254,6 +254,8 @@ __global__ void __launch_bounds__(256) k_finish64(const __grid_constant__ F64Arg
 
 // Tables of one context: sources, {in, out} link values, interface indices, u*_g. The values
 // are formed exactly as in the step of mp.cu.
+// kOne: one species, whose links need not be kept.
+template <bool kOne>
 __global__ void k_tables64(const F64Args a, const uint32_t* __restrict__ fmask, const uint32_t* __restrict__ iface,
                            const int32_t* __restrict__ ibase, const Flow4<double>* __restrict__ u4, int nx, int ny,
                            int nz, Div dx, Div dxy, int d0, int d1, int d2, int32_t* __restrict__ aidx,
@@ -267,13 +269,14 @@ __global__ void k_tables64(const F64Args a, const uint32_t* __restrict__ fmask, 
     const Flow4<double> ur = u4[n];
     const int dir[3] = {d0, d1, d2};
     aidx[k] = mask != (1u << 18) - 1u ? ibase[n >> 5] + __popc(iface[n >> 5] & ((1u << (n & 31)) - 1u)) : -1;
-    // the links once, then u*_g of every species from them (recomputing the links for each species took
-    // a third of mp_init with 16 species)
-    double qo[kQ];
+    // the links and the first species once, then u*_g of the others from the links (64^3 with 16
+    // species 202 us; with the links formed again for each species 428; one species 39)
+    [[maybe_unused]] double qo[kQ];
+    double us[3] = {0.0, 0.0, 0.0};
 #pragma unroll
     for (int i = 1; i < kQ; ++i) {
         const size_t at = at64(shared, k, i - 1);
-        qo[i] = 0.0;
+        if constexpr (!kOne) qo[i] = 0.0;
         if (!((mask >> (i - 1)) & 1u)) {
             src[at] = -1;
             tab[at] = make_double2(0.0, 0.0);
@@ -282,14 +285,19 @@ __global__ void k_tables64(const F64Args a, const uint32_t* __restrict__ fmask, 
         const int s = src_of(b, i);
         const Flow4<double> uf = u4[s];
         const double qin = qlink(edot<double>(i, uf.x, uf.y, uf.z), uf.w);
-        qo[i] = qlink(edot<double>(opposite(i), ur.x, ur.y, ur.z), ur.w);
+        const double qout = qlink(edot<double>(opposite(i), ur.x, ur.y, ur.z), ur.w);
+        if constexpr (!kOne) qo[i] = qout;
         const double whl = is_face(i) ? a.whf[0] : a.whe[0];
+        const double pout = rn_fma(weight<double>(i), qout, whl);
         src[at] = s;
-        tab[at] = a.S == 1 ? make_double2(rn_fma(weight<double>(i), qin, whl), rn_fma(weight<double>(i), qo[i], whl))
-                           : make_double2(qin, qo[i]);
+        tab[at] = kOne ? make_double2(rn_fma(weight<double>(i), qin, whl), pout) : make_double2(qin, qout);
+#pragma unroll
+        for (int m = 0; m < 3; ++m)
+            if (m < a.M) us[m] += (double)ci(opposite(i), dir[m]) * pout;
     }
-    for (int sp = 0; sp < a.S; ++sp) {
-        double us[3] = {0.0, 0.0, 0.0};
+    for (int m = 0; m < a.M; ++m) ust[(size_t)m * a.NF + k] = us[m];
+    for (int sp = 1; !kOne && sp < a.S; ++sp) {
+        us[0] = us[1] = us[2] = 0.0;
         const double whf = a.whf[sp], whe = a.whe[sp];
 #pragma unroll
         for (int i = 1; i < kQ; ++i) {
@@ -389,7 +397,8 @@ int flux64_setup(mp_ctx* c)
         a.pa[s] = c->ka[s];
         a.pd[s] = c->kd[s];
     }
-    k_tables64<<<(unsigned)((NF + 127) / 128), 128, 0, c->stream>>>(
+    auto tables = c->S == 1 ? k_tables64<true> : k_tables64<false>;
+    tables<<<(unsigned)((NF + 127) / 128), 128, 0, c->stream>>>(
         a, c->fmask, c->geo.iface, c->geo.ibase, (const Flow4<double>*)c->u4, c->geo.nx, c->geo.ny, c->geo.nz,
         make_div((unsigned)c->geo.nx), make_div((unsigned)(c->geo.nx * c->geo.ny)), c->dir[0], c->dir[1], c->dir[2],
         f->aidx, f->src, f->tab, f->ust, f->lanes > 1);
