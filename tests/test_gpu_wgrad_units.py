@@ -11,7 +11,8 @@ pytestmark = pytest.mark.gpu
 @pytest.mark.parametrize("B,D,H,W,K,N", [
     (4, 12, 12, 12, 96, 96), (4, 12, 12, 12, 128, 96), (1, 48, 48, 48, 32, 32), (1, 48, 48, 48, 32, 16),
     (2, 16, 16, 16, 96, 96), (4, 18, 7, 118, 32, 16), (4, 64, 4, 128, 32, 32), (3, 20, 34, 30, 64, 32),
-    (2, 24, 18, 40, 64, 64), (1, 40, 33, 64, 16, 16)])
+    (2, 24, 18, 40, 64, 64), (1, 40, 33, 64, 16, 16), (4, 32, 6, 64, 64, 32), (4, 24, 9, 80, 64, 32),
+    (4, 32, 6, 64, 128, 64)])
 def test_wgrad_exact_over_many_units(B, D, H, W, K, N):
     if not torch.cuda.is_available():
         pytest.skip("no CUDA device")
